@@ -258,11 +258,13 @@ int dvc_mcts_step(dvc_forest* f, int n_iterations, int mode, void* stream);
  * with warps_per_cta warps (every warp walks a tree, then all lanes share the
  * leaves' playouts; every 64 iterations all threads sample the next 64
  * determinizations of every tree, one thread each).  engine 2: per iteration two launches (backprop of the
- * previous iteration + select, then pooled rollouts) in a CUDA graph of 64
- * iterations; rollout CTAs pool trees_per_cta trees with warps_per_cta warps,
- * and the CTAs are split into `chains` (1..32) independent chains on
- * separate streams so that one chain's tree walks run beside another chain's
- * playouts.  The determinizations of the graph's 64 iterations are sampled
+ * previous iteration + select, then the playouts) in a CUDA graph of 64
+ * iterations; groups of trees_per_cta trees are split into `chains` (1..32)
+ * independent chains on separate streams so that one chain's tree walks run
+ * beside another chain's playouts.  Playouts run one game per lane in CTAs of
+ * four warps whatever the groups; under the ordering-aware policy and with
+ * lane compaction a group's playouts are pooled in one CTA of warps_per_cta
+ * warps.  The determinizations of the graph's 64 iterations are sampled
  * up front, one thread per tree and iteration.  engine 0 keeps the current
  * engine (the default is 2 for forests of more than four trees per SM, else 1).
  * trees_per_cta, warps_per_cta, chains 0 = the engine's defaults (fused:
@@ -342,8 +344,8 @@ int dvc_forest_counters(dvc_forest* f, uint64_t* d_out, void* stream);
 /* Lane compaction in the pipeline engine's two-player 24-tile playouts
  * (uniform policy, no may-stop leaves; other forests ignore it), off by
  * default (receivers = 0).  The paper studies the branch divergence of GPU
- * playouts (Sec. IV); this regroups running games instead: once a rollout
- * CTA's pool of playouts is empty, each of its warps from `receivers` on
+ * playouts (Sec. IV); this pools the playouts of a group of trees in one CTA
+ * and regroups running games: once a rollout CTA's pool of playouts is empty, each of its warps from `receivers` on
  * that has at most `donate_at` games running hands them (state and stream
  * position) to the CTA's first `receivers` warps, whose idle lanes finish
  * them.  Results are identical either way.  DVC_E_INVALID unless
@@ -359,9 +361,8 @@ int dvc_forest_compaction(dvc_forest* f, int receivers, int donate_at);
 int dvc_forest_work(dvc_forest* f, uint64_t* d_out, void* stream);
 /* Work counting (dvc_forest_counters, dvc_forest_work) on (the default) or
  * off.  The counts are instrumentation, not part of the search: off, the
- * playout kernels keep no counts (the two-player 24-tile playout kernel
- * then runs a counting-free variant, about 1.5 % faster) and both counters
- * keep their values; results are identical either way.  Takes effect at the
+ * playout kernels keep no counts (the pipeline engine's then run a
+ * counting-free variant) and both counters keep their values; results are identical either way.  Takes effect at the
  * next dvc_mcts_step.  DVC_E_INVALID for a null forest. */
 int dvc_forest_count_work(dvc_forest* f, int on);
 

@@ -506,147 +506,7 @@ __device__ __forceinline__ int random_guess_ordered(G& g, R& r, uint32_t cont_th
     return resolve(g, g.cur, 0u, 0xFFu, false, cont_thr, r);  // unreachable: total counts every kept guess
 }
 
-// One playout to the end (Sec. II-B); returns the winner.  Every guess turns
-// one tile face up, so a game has at most 26 guesses; the cap only stops a
-// malformed record (result kNone, credited to nobody).
-template <class R>
-__device__ __forceinline__ uint32_t playout(G g, R& r, uint32_t cont_thr, const uint32_t* magic = nullptr) {
-    for (int guard = 0; guard < 128; ++guard) {
-        const int res = random_guess(g, r, cont_thr, magic);
-        if (res == kGameOver) return g.winner;
-        if (res == kTurnOver) next_turn(g, r);
-    }
-    return kNone;
-}
-
-// The playout state with hands held relative to the mover: a0 is the hand of
-// seat cur, a1, a2, a3 those of seats cur + 1, cur + 2, cur + 3 (modulo np);
-// positions from np on hold 0.  The opponents are then visited in the
-// canonical order (from cur + 1) with no selection of hands by seat, and a
-// new turn rotates the four words once.  alive and winner stay by seat.
-struct GR {
-    uint32_t a0, a1, a2, a3;
-    uint32_t rev, jg0, jg1, jflag;
-    uint32_t cur, drawn, alive, winner, np, tmask;
-};
-
-__device__ __forceinline__ GR to_gr(const G& g) {
-    GR r;
-    uint32_t q1 = g.cur + 1u, q2 = g.cur + 2u, q3 = g.cur + 3u;
-    q1 = q1 >= g.np ? q1 - g.np : q1;
-    q2 = q2 >= g.np ? q2 - g.np : q2;
-    q3 = q3 >= g.np ? q3 - g.np : q3;
-    r.a0 = g.hand(g.cur);
-    r.a1 = g.hand(q1);
-    r.a2 = g.np > 2u ? g.hand(q2) : 0u;
-    r.a3 = g.np > 3u ? g.hand(q3) : 0u;
-    r.rev = g.rev;
-    r.jg0 = g.jg0;
-    r.jg1 = g.jg1;
-    r.jflag = g.jflag;
-    r.cur = g.cur;
-    r.drawn = g.drawn;
-    r.alive = g.alive;
-    r.winner = g.winner;
-    r.np = g.np;
-    r.tmask = g.tmask;
-    return r;
-}
-
-// One playout step in the relative form: random_guess, then next_turn if the
-// turn passes -- the same rules, the same words in the same order.
-template <class R>
-__device__ __forceinline__ int step_gen(GR& g, R& r, uint32_t cont_thr, const uint32_t* magic) {
-    r.ensure(4);
-    // the guess: opponent slots in canonical order times unknown identities
-    const uint32_t U = g.tmask & ~g.a0 & ~g.rev;
-    const uint32_t nid = __popc(U);
-    const uint32_t c1 = __popc(g.a1 & ~g.rev), c2 = __popc(g.a2 & ~g.rev), c3 = __popc(g.a3 & ~g.rev);
-    const uint32_t k = pick(r.next(), (c1 + c2 + c3) * nid);
-    uint32_t s = div_small(k, nid, magic);
-    const uint32_t i = k - s * nid;
-    uint32_t off = 1u, hq = g.a1;
-    if (s >= c1) {
-        s -= c1;
-        off = 2u;
-        hq = g.a2;
-        if (s >= c2) {
-            s -= c2;
-            off = 3u;
-            hq = g.a3;
-        }
-    }
-    const uint32_t target = hidden_in(g, hq, s);
-    const uint32_t tb = 1u << target;
-    if (__popc(U & (tb - 1u)) == i) {  // correct: the target is revealed
-        g.rev |= tb;
-        if (!(hq & ~g.rev)) {
-            uint32_t q = g.cur + off;
-            q = q >= g.np ? q - g.np : q;
-            g.alive &= ~(1u << q);
-        }
-        if (__popc(g.alive) == 1) {
-            g.winner = g.cur;
-            return kGameOver;
-        }
-        if (cont_thr != 0u && r.next() < cont_thr) return kGuessAgain;
-    } else {  // wrong: the mover reveals its drawn tile, else its leftmost face-down one
-        uint32_t t = g.drawn;
-        if (t == kNone) {  // the leftmost face-down tile: the lowest one unless a joker is face down
-            const uint32_t hid = g.a0 & ~g.rev;
-            t = (hid & kJokerMask) ? hidden_in(g, g.a0, 0u) : (uint32_t)__ffs(hid) - 1u;
-        }
-        g.rev |= 1u << t;
-        if (!(g.a0 & ~g.rev)) g.alive &= ~(1u << g.cur);
-        if (__popc(g.alive) == 1) {
-            g.winner = (uint32_t)__ffs(g.alive) - 1u;
-            return kGameOver;
-        }
-    }
-    // the next live seat moves: rotate the hands by d = its distance (1 .. np-1)
-    const uint32_t nc = next_alive(g.alive, g.cur, g.np);
-    const uint32_t d = nc > g.cur ? nc - g.cur : nc + g.np - g.cur;
-    if (g.np == 4u) {
-        if (d & 1u) {
-            const uint32_t t = g.a0;
-            g.a0 = g.a1;
-            g.a1 = g.a2;
-            g.a2 = g.a3;
-            g.a3 = t;
-        }
-        if (d & 2u) {
-            uint32_t t = g.a0;
-            g.a0 = g.a2;
-            g.a2 = t;
-            t = g.a1;
-            g.a1 = g.a3;
-            g.a3 = t;
-        }
-    } else if (g.np == 3u) {
-        const uint32_t b0 = d == 1u ? g.a1 : g.a2, b1 = d == 1u ? g.a2 : g.a0, b2 = d == 1u ? g.a0 : g.a1;
-        g.a0 = b0;
-        g.a1 = b1;
-        g.a2 = b2;
-    } else {
-        const uint32_t t = g.a0;
-        g.a0 = g.a1;
-        g.a1 = t;
-    }
-    g.cur = nc;
-    // ... and draws
-    const uint32_t pool = g.tmask & ~(g.a0 | g.a1 | g.a2 | g.a3);
-    if (!pool) {
-        g.drawn = kNone;
-        return kTurnOver;
-    }
-    const uint32_t t = nth_set(pool, pick(r.next(), __popc(pool)));
-    insert_gaps(g, g.a0, t, r);
-    g.a0 |= 1u << t;
-    g.drawn = t;
-    return kTurnOver;
-}
-
-// Words for the playout loop of the pooled kernel: a short queue that is
+// Words for playouts with a queue in registers: a short queue that is
 // topped up once, at the start of each game step, with enough words for the
 // whole step (a guess, a continue coin, a draw and a joker position at most),
 // so the step itself never branches to refill.

@@ -21,6 +21,7 @@ using namespace dvc_host;
 
 namespace {
 constexpr int kMaxChains = 32;  // independent chains of the pipeline graph
+constexpr long long kMaxGrid = 1ll << 30;  // CTAs per playout launch
 constexpr int kValueChains = 16;  // at most, in value mode (each chain pads its leaves to 128 rows)
 
 // Default launch shape of an engine for n trees on `sms` SMs with P playouts
@@ -214,15 +215,72 @@ __global__ void play_move_kernel(dvc_state* states, int n, const int32_t* action
     store_state(g, states[i]);
 }
 
-// Leaf-parallel playouts: thread -> (leaf, playout).  Win counts are summed
-// with integer atomics, so the result is independent of scheduling.
-template <bool ORD>
-__global__ void rollout_kernel(const dvc_state* leaves, int n_leaves, int P, uint64_t seed,
-                               const uint32_t* tree_ids, const uint32_t* leaf_ids, uint32_t cont_thr, int32_t* wins,
-                               unsigned long long* words, int32_t* flags) {
-    __shared__ uint32_t s_magic[32];
-    fill_magic(s_magic, threadIdx.x, blockDim.x);
+// Leaf-parallel playouts (dvc_play.cuh): game (leaf, j), 32 consecutive games
+// per warp, one per lane.  Win counts are summed with integer atomics, so the
+// result is independent of scheduling.
+// FAST2: the two-player state, for warps whose leaves are all of that variant;
+// the others are left to a launch of the general one with skip2 set, which
+// leaves out those warps (a context of the two-player variant may be given
+// leaves of any).
+constexpr int kRollWarps = 4;
+template <bool FAST2>
+__global__ void __launch_bounds__(32 * kRollWarps, 8)
+    rollout_kernel(const dvc_state* leaves, int n_leaves, int P, long long block0, uint64_t seed,
+                   const uint32_t* tree_ids, const uint32_t* leaf_ids, uint32_t cont_thr, int skip2, int32_t* wins,
+                   unsigned long long* words_out, int32_t* flags) {
+    __shared__ __align__(16) unsigned char s_sel[kSelBytes];
+    __shared__ __align__(16) unsigned char s_ring[kRingBytes * kRollWarps];
+    const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+    const long long total = (long long)n_leaves * P;
+    const long long p = ((block0 + blockIdx.x) * kRollWarps + warp) * 32 + lane;
+    uint32_t l = 0u, j = 0u;
+    bool busy = false, two = true;
+    G s;
+    if (p < total) {
+        l = total <= 0xFFFFFFFFll ? (uint32_t)p / (uint32_t)P : (uint32_t)(p / P);
+        j = (uint32_t)(p - (long long)l * P);
+        const dvc_state ls = leaves[l];
+        s = load_state(ls);
+        busy = ls.winner == kNone;
+        two = !busy || (s.np == 2u && s.tmask == kNumMask);
+        if (!busy && ls.winner < 4u && j == 0u && (FAST2 || !skip2)) atomicAdd(&wins[4 * l + ls.winner], P);
+    }
+    const bool all2 = __all_sync(0xFFFFFFFFu, two);
+    if ((FAST2 && !all2) || (!FAST2 && skip2 && all2)) busy = false;
+    if (!__syncthreads_or(busy)) return;
+    fill_select(s_sel, tid, 32 * kRollWarps);
     __syncthreads();
+    if (!__any_sync(0xFFFFFFFFu, busy)) return;
+    using Game = typename std::conditional<FAST2, Play2, PlayN>::type;
+    Game g;
+    PlayWords r;
+    g.idle();
+    r.ring = shared_addr(s_ring) + warp * kRingBytes + lane * 4u;
+    r.open(seed, 0u, 0u, 0u);
+    const uint32_t tab = shared_addr(s_sel);
+    bool pend = false;
+    if (busy) {
+        g.begin(s, tab);
+        pend = s.mstop != 0u;
+        r.open(seed, tree_ids[l], j, leaf_ids[l]);
+    }
+    uint32_t words = 0u, steps = 0u;
+    const uint32_t w = __any_sync(0xFFFFFFFFu, pend)
+                           ? play_games<Game, true, true>(g, r, busy, pend, seed, cont_thr, tab, words, steps)
+                           : play_games<Game, false, true>(g, r, busy, false, seed, cont_thr, tab, words, steps);
+    credit_wins(wins, l, w);
+    // no winner after 128 steps is a broken invariant
+    if (busy && w >= 4u) latch_error(flags, DVC_E_INTERNAL);
+    if (words_out) {
+        const unsigned long long sum = warp_sum_u64((unsigned long long)words);
+        if (lane == 0u && sum) atomicAdd(words_out, sum);
+    }
+}
+
+// The same under the ordering-aware policy: thread -> (leaf, playout).
+__global__ void rollout_ordered_kernel(const dvc_state* leaves, int n_leaves, int P, uint64_t seed,
+                                       const uint32_t* tree_ids, const uint32_t* leaf_ids, uint32_t cont_thr,
+                                       int32_t* wins, unsigned long long* words, int32_t* flags) {
     const long long total = (long long)n_leaves * P;
     unsigned long long my_words = 0ull;
     for (long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x; gid < total;
@@ -239,24 +297,14 @@ __global__ void rollout_kernel(const dvc_state* leaves, int n_leaves, int P, uin
             r.open(seed, tree_ids[l], (uint32_t)j, leaf_ids[l], kTagRoll);
             playout_begin(g, r, cont_thr);
             winner = kNone;
-            if constexpr (ORD) {
-                for (int guard = 0; guard < 128; ++guard) {
-                    r.ensure(4);
-                    const int res = random_guess_ordered(g, r, cont_thr);
-                    if (res == kGameOver) {
-                        winner = g.winner;
-                        break;
-                    }
-                    if (res == kTurnOver) next_turn(g, r);
+            for (int guard = 0; guard < 128; ++guard) {
+                r.ensure(4);
+                const int res = random_guess_ordered(g, r, cont_thr);
+                if (res == kGameOver) {
+                    winner = g.winner;
+                    break;
                 }
-            } else {
-                GR gr = to_gr(g);
-                for (int guard = 0; guard < 128; ++guard) {
-                    if (step_gen(gr, r, cont_thr, s_magic) == kGameOver) {
-                        winner = gr.winner;
-                        break;
-                    }
-                }
+                if (res == kTurnOver) next_turn(g, r);
             }
             // at most |T| guesses per game: no winner after 128 is a broken invariant
             if (winner == kNone) latch_error(flags, DVC_E_INTERNAL);
@@ -269,8 +317,6 @@ __global__ void rollout_kernel(const dvc_state* leaves, int n_leaves, int P, uin
         if ((threadIdx.x & 31u) == 0 && s) atomicAdd(words, s);
     }
 }
-
-
 
 // Split steps: one warp per tree for select and expand, results kept in
 // global memory between launches.
@@ -840,20 +886,29 @@ int dvc_rollout_batch(dvc_ctx* c, const dvc_state* d_leaves, int n_leaves, int p
     cudaError_t e = cudaMemsetAsync(d_wins, 0, sizeof(int32_t) * 4 * (size_t)n_leaves, st);
     if (e == cudaSuccess && d_words) e = cudaMemsetAsync(d_words, 0, sizeof(uint64_t), st);
     if (e != cudaSuccess) return cuda_fail(c, e, "dvc_rollout_batch memset");
-    int dev_sms = 0;
-    cudaDeviceGetAttribute(&dev_sms, cudaDevAttrMultiProcessorCount, c->device);
     const long long total = (long long)n_leaves * playouts_per_leaf;
-    const int block = 256;
-    long long blocks = (total + block - 1) / block;
-    blocks = std::min<long long>(blocks, (long long)dev_sms * 64);
-    if (c->cfg.policy)
-        rollout_kernel<true><<<(unsigned)blocks, block, 0, st>>>(d_leaves, n_leaves, playouts_per_leaf, seed,
-                                                                 d_tree_ids, d_leaf_ids, c->cfg.cont_thr, d_wins,
-                                                                 (unsigned long long*)d_words, c->d_flags);
-    else
-        rollout_kernel<false><<<(unsigned)blocks, block, 0, st>>>(d_leaves, n_leaves, playouts_per_leaf, seed,
-                                                                  d_tree_ids, d_leaf_ids, c->cfg.cont_thr, d_wins,
-                                                                  (unsigned long long*)d_words, c->d_flags);
+    if (c->cfg.policy) {
+        int dev_sms = 0;
+        cudaDeviceGetAttribute(&dev_sms, cudaDevAttrMultiProcessorCount, c->device);
+        const int block = 256;
+        const long long blocks = std::min<long long>((total + block - 1) / block, (long long)dev_sms * 64);
+        rollout_ordered_kernel<<<(unsigned)blocks, block, 0, st>>>(d_leaves, n_leaves, playouts_per_leaf, seed,
+                                                                   d_tree_ids, d_leaf_ids, c->cfg.cont_thr, d_wins,
+                                                                   (unsigned long long*)d_words, c->d_flags);
+        return check_launch(c, "rollout_ordered_kernel");
+    }
+    const long long blocks = (total + 32 * kRollWarps - 1) / (32 * kRollWarps);
+    const bool two = c->cfg.nplayers == 2 && c->cfg.ntiles == 24;
+    for (long long b0 = 0; b0 < blocks; b0 += kMaxGrid) {
+        const unsigned grid = (unsigned)std::min<long long>(blocks - b0, kMaxGrid);
+        if (two)
+            rollout_kernel<true><<<grid, 32 * kRollWarps, 0, st>>>(
+                d_leaves, n_leaves, playouts_per_leaf, b0, seed, d_tree_ids, d_leaf_ids, c->cfg.cont_thr, 0, d_wins,
+                (unsigned long long*)d_words, c->d_flags);
+        rollout_kernel<false><<<grid, 32 * kRollWarps, 0, st>>>(
+            d_leaves, n_leaves, playouts_per_leaf, b0, seed, d_tree_ids, d_leaf_ids, c->cfg.cont_thr, two ? 1 : 0,
+            d_wins, (unsigned long long*)d_words, c->d_flags);
+    }
     return check_launch(c, "rollout_kernel");
 }
 
@@ -1146,27 +1201,26 @@ int enqueue_pipe_iteration(dvc_forest* f, int b0, int b1, cudaStream_t st) {
     const bool pend = c->cfg.tree_continue || c->cfg.d_max == 0 || c->cfg.vanilla;
     const uint32_t smem = pipe_rollout_smem(L, threads);
     unsigned long long* words = f->no_count ? nullptr : f->d_words;
-    if (fast2 && !sp.policy && !pend && f->cmp_receivers > 0 && f->cmp_receivers < threads / 32)
+    if (sp.policy) {
+        if (fast2)
+            pipe_rollout_ordered_kernel<true><<<b1 - b0, threads, smem, st>>>(sp, n, L, b0, f->order, f->meta, f->pipe,
+                                                                             words);
+        else
+            pipe_rollout_ordered_kernel<false><<<b1 - b0, threads, smem, st>>>(sp, n, L, b0, f->order, f->meta,
+                                                                              f->pipe, words);
+    } else if (fast2 && !pend && f->cmp_receivers > 0 && f->cmp_receivers < threads / 32) {
         pipe_rollout_compact_kernel<<<b1 - b0, threads, pipe_compact_smem(L, threads, f->cmp_receivers), st>>>(
             sp, n, L, b0, f->order, f->meta, f->pipe, words, f->cmp_receivers, f->cmp_donate_at);
-    else if (fast2 && !sp.policy && !pend && f->no_count)
-        pipe_rollout_kernel<true, false, false, false><<<b1 - b0, threads, smem, st>>>(sp, n, L, b0, f->order,
-                                                                                      f->meta, f->pipe, nullptr);
-    else if (fast2 && !sp.policy && !pend)
-        pipe_rollout_kernel<true, false, false><<<b1 - b0, threads, smem, st>>>(sp, n, L, b0, f->order, f->meta,
-                                                                               f->pipe, words);
-    else if (fast2 && !sp.policy)
-        pipe_rollout_kernel<true, false, true><<<b1 - b0, threads, smem, st>>>(sp, n, L, b0, f->order, f->meta,
-                                                                              f->pipe, words);
-    else if (fast2)
-        pipe_rollout_kernel<true, true><<<b1 - b0, threads, smem, st>>>(sp, n, L, b0, f->order, f->meta, f->pipe,
-                                                                       words);
-    else if (!sp.policy)
-        pipe_rollout_kernel<false, false><<<b1 - b0, threads, smem, st>>>(sp, n, L, b0, f->order, f->meta, f->pipe,
-                                                                         words);
-    else
-        pipe_rollout_kernel<false, true><<<b1 - b0, threads, smem, st>>>(sp, n, L, b0, f->order, f->meta, f->pipe,
-                                                                        words);
+    } else {
+        auto k = fast2 ? (pend ? (words ? pipe_play_kernel<true, true, true> : pipe_play_kernel<true, true, false>)
+                               : (words ? pipe_play_kernel<true, false, true> : pipe_play_kernel<true, false, false>))
+                       : (pend ? (words ? pipe_play_kernel<false, true, true> : pipe_play_kernel<false, true, false>)
+                               : (words ? pipe_play_kernel<false, false, true> : pipe_play_kernel<false, false, false>));
+        const long long blocks = pipe_play_blocks(i1 - i0, sp.playouts);
+        for (long long b = 0; b < blocks; b += kMaxGrid)
+            k<<<(unsigned)std::min<long long>(blocks - b, kMaxGrid), 32 * kPlayWarps, 0, st>>>(
+                sp, i0, i1, b, f->order, f->meta, f->pipe, words);
+    }
     return check_launch(c, "pipeline kernels");
 }
 
@@ -1264,10 +1318,15 @@ int launch_pipeline(dvc_forest* f, int n_iterations, cudaStream_t st) {
         const int threads = pipe_rollout_threads(f);
         const int sm = (int)pipe_rollout_smem(f->trees_per_cta, threads);
         cudaError_t e = cudaSuccess;
-        // several rollout CTAs per SM need the largest shared-memory carveout
-        for (auto k : {pipe_rollout_kernel<true, false, false>, pipe_rollout_kernel<true, false, false, false>,
-                       pipe_rollout_kernel<true, false, true>, pipe_rollout_kernel<true, true, true>,
-                       pipe_rollout_kernel<false, false, true>, pipe_rollout_kernel<false, true, true>}) {
+        // several playout CTAs per SM need the largest shared-memory carveout
+        for (auto k : {pipe_play_kernel<true, true, true>, pipe_play_kernel<true, true, false>,
+                       pipe_play_kernel<true, false, true>, pipe_play_kernel<true, false, false>,
+                       pipe_play_kernel<false, true, true>, pipe_play_kernel<false, true, false>,
+                       pipe_play_kernel<false, false, true>, pipe_play_kernel<false, false, false>})
+            if (e == cudaSuccess)
+                e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                         (int)cudaSharedmemCarveoutMaxShared);
+        for (auto k : {pipe_rollout_ordered_kernel<true>, pipe_rollout_ordered_kernel<false>}) {
             if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
             if (e == cudaSuccess)
                 e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout,

@@ -3,14 +3,15 @@
 //   pipe_select   one warp per tree: backpropagate the previous iteration's
 //                 playout results, then determinize, descend, expand and
 //                 publish the next leaf;
-//   pipe_rollout  one CTA per group of trees: the P playouts of the group's leaves
-//                 form one pool that lanes draw from as they free up;
+//   pipe_play     the playouts of the leaves, one game per lane;
 //   pipe_backprop after the last iteration of a step: the pending backprop.
 // The tree walk needs many registers and the playout loop few, so giving each
 // its own kernel lets the playouts run at full occupancy.  Every tree still
 // runs its iterations strictly in order, so results equal the fused kernel's
 // and the oracle's bit for bit.
 #pragma once
+#include <type_traits>
+
 #include "dvc_pool.cuh"
 
 namespace dvc {
@@ -148,28 +149,86 @@ __global__ void __launch_bounds__(128)
     }
 }
 
-// Trees order[b*L .. b*L+L-1] belong to CTA b; this launch runs CTAs b0 + blockIdx.x.
-// The CTA's L x P playouts form one pool: a lane whose game ends takes the
-// next playout index (warp-aggregated: one shared-memory atomic per warp and
-// step), so lanes wait for the longest game only at the end of the pool.
-// Every lane queues its words in a shared-memory ring (RingQueue), refilled
-// warp-wide, so that the Philox rounds run for most lanes at once; for
-// two-player 24-tile games it also lets two 1024-thread CTAs fit on an SM.
-// ORD: the ordering-aware playout policy (sp.policy == 1), compiled apart.
+// The playouts of trees order[i0 .. i1-1]: game (tree, j) for j < sp.playouts,
+// 32 consecutive games per warp, one per lane (dvc_play.cuh); leaves that do
+// not run or ended inside the tree have none.  Warps share nothing but the
+// select table, so a CTA needs no barrier after it and ends with its longest
+// game; wins go straight to the tree's counts (select has zeroed them).
+// Four warps per CTA: the table is read once per 128 games.
 // PEND: leaves may begin where the mover may stop (the full game tree, or
 // d_max = 0); without it that check is compiled out of the playout loop,
 // since an in-tree action always clears the may-stop bit otherwise.
 // CNT: keep the work counters (random words, game steps) in words_out;
 // compiled out for forests that switched counting off.
-// Registers: 32 for the two-player path (two 1024-thread or three
-// 512-thread CTAs per SM, with room left in the register file for the
-// other chains' tree walks), up to 64 for the general path.
-template <bool FAST2, bool ORD = false, bool PEND = true, bool CNT = true>
+constexpr int kPlayWarps = 4;
+template <bool FAST2, bool PEND, bool CNT>
+__global__ void __launch_bounds__(32 * kPlayWarps, FAST2 ? 12 : 8)
+    pipe_play_kernel(SearchParams sp, int i0, int i1, long long block0, const int32_t* order, const TreeMeta* meta,
+                     PipeBufs P, unsigned long long* words_out) {
+    __shared__ __align__(16) unsigned char s_sel[kSelBytes];
+    __shared__ __align__(16) unsigned char s_ring[kRingBytes * kPlayWarps];
+    const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+    fill_select(s_sel, tid, 32 * kPlayWarps);
+    __syncthreads();
+    const uint32_t Pp = (uint32_t)sp.playouts;
+    const long long total = (long long)(i1 - i0) * Pp;
+    const long long first = ((block0 + blockIdx.x) * kPlayWarps + warp) * 32;
+    if (first >= total) return;
+    using Game = typename std::conditional<FAST2, Play2, PlayN>::type;
+    Game g;
+    PlayWords r;
+    g.idle();
+    r.ring = shared_addr(s_ring) + warp * kRingBytes + lane * 4u;
+    r.open(sp.seed, 0u, 0u, 0u);
+    const uint32_t tab = shared_addr(s_sel);
+    const long long p = first + lane;
+    int t = -1;
+    bool busy = false, pend = false;
+    if (p < total) {
+        const uint32_t e = total <= 0xFFFFFFFFll ? (uint32_t)p / Pp : (uint32_t)(p / Pp);
+        t = order[i0 + (int)e];
+        const dvc_state ls = P.leaf[t];
+        if (P.np[t] >= 0 && ls.winner == kNone) {
+            busy = true;
+            const G s = load_state(ls);
+            g.begin(s, tab);
+            pend = s.mstop != 0u;
+            r.open(sp.seed, meta[t].tree_id, (uint32_t)(p - (long long)e * Pp), (uint32_t)meta[t].done);
+        }
+    }
+    const bool mine = busy;
+    uint32_t words = 0u, steps = 0u;
+    const uint32_t w = play_games<Game, PEND, CNT>(g, r, busy, pend, sp.seed, sp.cont_thr, tab, words, steps);
+    credit_wins(P.wins, (uint32_t)t, w);
+    // no winner after 128 steps is a broken invariant
+    if (mine && w >= 4u) latch_error(P.flags, DVC_E_INTERNAL);
+    if (CNT && words_out) {  // words_out[0]: random words, words_out[1]: game steps (guesses)
+        const unsigned long long sum = warp_sum_u64((unsigned long long)words);
+        if (lane == 0 && sum) atomicAdd(words_out, sum);
+        if (lane == 0 && steps) atomicAdd(words_out + 1, (unsigned long long)steps);
+    }
+}
+
+// CTAs of pipe_play_kernel for n trees.
+inline long long pipe_play_blocks(int n, int playouts) {
+    return ((long long)n * playouts + 32 * kPlayWarps - 1) / (32 * kPlayWarps);
+}
+
+// Playouts under the ordering-aware policy (sp.policy == 1), whose step time
+// depends on the rows, so that lanes are refilled:
+// trees order[b*L .. b*L+L-1] belong to CTA b; this launch runs CTAs b0 + blockIdx.x.
+// The CTA's L x P playouts form one pool: a lane whose game ends takes the
+// next playout index (warp-aggregated: one shared-memory atomic per warp and
+// step), so lanes wait for the longest game only at the end of the pool.
+// Every lane queues its words in a shared-memory ring (RingQueue), refilled
+// warp-wide, so that the Philox rounds run for most lanes at once.
+// Registers: 32 for the two-player path (two 1024-thread or three 512-thread
+// CTAs per SM), up to 64 for the general path.
+template <bool FAST2>
 __global__ void __launch_bounds__(1024, FAST2 ? 2 : 1)
-    pipe_rollout_kernel(SearchParams sp, int n, int L, int b0, const int32_t* order, const TreeMeta* meta, PipeBufs P,
-                        unsigned long long* words_out) {
+    pipe_rollout_ordered_kernel(SearchParams sp, int n, int L, int b0, const int32_t* order, const TreeMeta* meta,
+                                PipeBufs P, unsigned long long* words_out) {
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ uint32_t s_magic[32];
     __shared__ unsigned long long s_lut12[FAST2 ? 4096 : 1];
     __shared__ int32_t s_n, s_next;
     uint32_t* s_ring = (uint32_t*)smem;                   // 16 words per thread
@@ -179,7 +238,6 @@ __global__ void __launch_bounds__(1024, FAST2 ? 2 : 1)
     uint32_t* s_it = s_tid + L;
     dvc_state* s_leaf = (dvc_state*)(((uintptr_t)(s_it + L) + 15) & ~(uintptr_t)15);
     const uint32_t tid = threadIdx.x, lane = tid & 31u;
-    fill_magic(s_magic, tid, blockDim.x);
     if constexpr (FAST2) fill_select12(s_lut12, tid, blockDim.x);
     if (tid == 0) {
         int32_t k = 0;
@@ -216,8 +274,7 @@ __global__ void __launch_bounds__(1024, FAST2 ? 2 : 1)
     RingQueue r;
     r.ring = s_ring + tid;
     r.stride = blockDim.x;
-    G g;    // general path, ordering-aware policy
-    GR gr;  // general path, uniform policy
+    G g;  // general path
     uint32_t h0 = 0, h1 = 0, rev = 0, cur = 0, drawn = kNone, winner = kNone;
     auto start = [&](uint32_t p) {
         k = Pp > 1u ? __umulhi(p, mP) : p;
@@ -234,7 +291,6 @@ __global__ void __launch_bounds__(1024, FAST2 ? 2 : 1)
         } else {
             g = load_state(ls);
             playout_begin(g, r, sp.cont_thr);
-            if constexpr (!ORD) gr = to_gr(g);
         }
         // a may-stop leaf's first continue coin is a game step of its own
         // (the fast path counts it as an iteration of its loop)
@@ -260,25 +316,20 @@ __global__ void __launch_bounds__(1024, FAST2 ? 2 : 1)
     for (;;) {
         const unsigned running = __ballot_sync(0xFFFFFFFFu, busy);
         if (!running) break;
-        if constexpr (CNT) wsteps += __popc(running);
+        wsteps += __popc(running);
         bool ended = false;
         if (busy) {
             int res;
             if constexpr (FAST2) {
-                if (PEND && winner == kPend)
+                if (winner == kPend)
                     res = step_2p24_pending(h0, h1, cur, drawn, winner, r, sp.cont_thr, s_lut12);
-                else if constexpr (ORD)
-                    res = step_2p24_ordered(h0, h1, rev, cur, drawn, winner, r, sp.cont_thr, s_lut12);
                 else
-                    res = step_2p24(h0, h1, rev, cur, drawn, winner, r, sp.cont_thr, s_magic, s_lut12);
-            } else if constexpr (ORD) {
+                    res = step_2p24_ordered(h0, h1, rev, cur, drawn, winner, r, sp.cont_thr, s_lut12);
+            } else {
                 r.ensure(4);
                 res = random_guess_ordered(g, r, sp.cont_thr);
                 if (res == kTurnOver) next_turn(g, r);
                 winner = g.winner;
-            } else {
-                res = step_gen(gr, r, sp.cont_thr, s_magic);
-                winner = gr.winner;
             }
             ++steps;
             if (res == kGameOver || steps >= 128u) {
@@ -287,7 +338,7 @@ __global__ void __launch_bounds__(1024, FAST2 ? 2 : 1)
                 // leaf's wins fall short of P (checked below)
                 const uint32_t w = res == kGameOver ? winner : kNone;
                 if (w < 4u) atomicAdd(&s_wins[4 * k + w], 1);
-                if constexpr (CNT) words += r.used();
+                words += r.used();
                 ended = true;
             }
         }
@@ -311,11 +362,11 @@ __global__ void __launch_bounds__(1024, FAST2 ? 2 : 1)
         if (s_wins[4 * e] + s_wins[4 * e + 1] + s_wins[4 * e + 2] + s_wins[4 * e + 3] != (int32_t)Pp)
             latch_error(P.flags, DVC_E_INTERNAL);
     }
-    if (CNT && words_out) {  // words_out[0]: random words, words_out[1]: game steps (guesses)
+    if (words_out) {  // words_out[0]: random words, words_out[1]: game steps (guesses)
         const unsigned long long sum = warp_sum_u64((unsigned long long)words);
         if (lane == 0 && sum) atomicAdd(words_out, sum);
         if (lane == 0 && wsteps) atomicAdd(words_out + 1, (unsigned long long)wsteps);
-        if constexpr (PEND && !FAST2) {
+        if constexpr (!FAST2) {
             // the general path draws a may-stop leaf's first continue coin when
             // a playout starts, outside the loop counted above: one step each
             if (tid == 0) {
@@ -327,20 +378,19 @@ __global__ void __launch_bounds__(1024, FAST2 ? 2 : 1)
     }
 }
 
-// Dynamic shared memory of pipe_rollout_kernel: the word rings and the
+// Dynamic shared memory of the pooled playout kernels: the word rings and the
 // listed leaves.
 __host__ __device__ inline uint32_t pipe_rollout_smem(int L, int threads) {
     return (uint32_t)(64 * threads + 4 * L + 16 * L + 4 * L + 4 * L + 16 + 32 * L);
 }
 
 // Lane compaction for the two-player 24-tile playouts (uniform policy, no
-// may-stop leaves), a variant of pipe_rollout_kernel measured against it
-// and off by default.  Warps 0 .. R-1 receive, the others donate: once the
+// may-stop leaves), off by default.  Warps 0 .. R-1 receive, the others donate: once the
 // CTA's pool of playouts is empty, a donor warp with at most `donate_at`
 // games still running posts them (state, leaf, stream position) to a mailbox
 // in shared memory and leaves the playout loop; receiver lanes that are idle
 // take posted games and finish them.  Every game goes on with the same words
-// of its own stream, so results equal the default kernel's.  Receivers stop
+// of its own stream, so results equal pipe_play_kernel's.  Receivers stop
 // once no donor is left and the mailbox is drained; every wait is bounded
 // (DVC_E_TIMEOUT latched if a limit is hit).
 constexpr int kMailFields = 11;

@@ -7,9 +7,8 @@
 //   1. tree phase -- warp w walks slots w, w+W, ...: take the iteration's
 //      determinization, descend by UCB1, expand one child, and publish the leaf;
 //   2. playout phase -- the P playouts of every published leaf form one pool;
-//      each lane takes the next playout of the pool as soon as its previous one
-//      ends (one guess, plus the draw that follows, per loop step), so lanes stay
-//      busy until the pool is empty;
+//      each warp takes the next 32 of it and plays them side by side
+//      (dvc_play.cuh), until the pool is empty;
 //   3. backprop -- each warp adds its trees' playout results along their paths.
 // Trees stay strictly sequential (iteration i+1 sees i's statistics), which is
 // what makes results bit-exact with the single-threaded oracle, while every
@@ -17,6 +16,7 @@
 // drop out of phase 1 and keep helping with phase 2, so uneven budgets balance
 // inside a CTA; across CTAs the host assigns trees by total work.
 #pragma once
+#include "dvc_play.cuh"
 #include "dvc_tree.cuh"
 
 namespace dvc {
@@ -48,7 +48,7 @@ __device__ __forceinline__ void latch_error(int32_t* flags, int32_t code) { atom
 
 // Shared-memory layout of one CTA with T slots and W warps.
 struct PoolLayout {
-    uint32_t pl, meta, root, leaf, path, mover, wins, misc, base, E, cnt, bytes;
+    uint32_t pl, meta, root, leaf, path, mover, wins, misc, base, E, cnt, ring, bytes;
     __host__ __device__ PoolLayout(int T, int W) {
         uint32_t o = 0;
         auto take = [&](uint32_t n) {
@@ -67,6 +67,7 @@ struct PoolLayout {
         base = take(4u * T);   // per slot: first iteration sampled ahead
         E = take(4u * 104u * W);
         cnt = take(4u * 8u);   // [parity][nleaf, next, ntrees, 0]
+        ring = take(kRingBytes * W);  // words of the playouts
         bytes = o;
     }
 };
@@ -81,8 +82,8 @@ __global__ void __launch_bounds__(MAXT, 1)
     mcts_pool_kernel(ForestDev F, SearchParams sp, int n_iter, const int32_t* order, int n_trees, int T,
                      dvc_state* det_ahead, uint4* tree0_ahead) {
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ uint32_t s_magic[32];
-    __shared__ unsigned long long s_lut12[FAST2 ? 4096 : 1];
+    __shared__ unsigned long long s_lut12[FAST2 && ORD ? 4096 : 1];
+    __shared__ __align__(16) unsigned char s_sel[ORD ? 16 : kSelBytes];
     const int W = (int)(blockDim.x >> 5);
     const PoolLayout L(T, W);
     DetPlan* s_pl = (DetPlan*)(smem + L.pl);
@@ -117,8 +118,8 @@ __global__ void __launch_bounds__(MAXT, 1)
         }
     }
     if (tid < 8) s_cnt[tid] = 0;
-    fill_magic(s_magic, tid, blockDim.x);
-    if constexpr (FAST2) fill_select12(s_lut12, tid, blockDim.x);
+    if constexpr (!ORD) fill_select(s_sel, tid, blockDim.x);
+    else if constexpr (FAST2) fill_select12(s_lut12, tid, blockDim.x);
     __syncthreads();
 
     uint32_t words = 0u, nsteps = 0u;  // per lane; summed in 64 bits per warp at the end
@@ -202,15 +203,48 @@ __global__ void __launch_bounds__(MAXT, 1)
             cnt[0] = n;
         }
         __syncthreads();
-        // ---- 2. playout phase: P playouts of each listed leaf, handed to lanes as they free up
-        {
+        // ---- 2. playout phase: P playouts of each listed leaf
+        if constexpr (!ORD) {
+            // 32 games at a time per warp, one per lane, until the pool is empty
+            using Game = typename std::conditional<FAST2, Play2, PlayN>::type;
+            const uint32_t P = (uint32_t)sp.playouts, total = (uint32_t)cnt[0] * P;
+            const uint32_t tab = shared_addr(s_sel);
+            for (;;) {
+                uint32_t first = 0;
+                if (lane == 0) first = (uint32_t)atomicAdd(&cnt[1], 32);
+                first = __shfl_sync(0xFFFFFFFFu, first, 0);
+                if (first >= total) break;
+                Game g;
+                PlayWords r;
+                g.idle();
+                r.ring = shared_addr(smem + L.ring) + warp * kRingBytes + lane * 4u;
+                r.open(sp.seed, 0u, 0u, 0u);
+                const uint32_t p = first + lane;
+                const bool busy = p < total;
+                bool pend = false;
+                int slot = 0;
+                if (busy) {
+                    const uint32_t k = p / P;
+                    slot = s_misc[4 * k + 3];
+                    const G st = load_state(s_leaf[slot]);
+                    g.begin(st, tab);
+                    pend = st.mstop != 0u;
+                    r.open(sp.seed, s_tm[slot].tree_id, p - k * P, (uint32_t)s_tm[slot].done);
+                }
+                const uint32_t w =
+                    play_games<Game, true, true>(g, r, busy, pend, sp.seed, sp.cont_thr, tab, words, nsteps);
+                credit_wins(s_wins, (uint32_t)slot, w);
+                // no winner after 128 steps is a broken invariant
+                if (busy && w >= 4u) latch_error(F.flags, DVC_E_INTERNAL);
+            }
+        } else {
+            // handed to lanes as they free up
             const int P = sp.playouts;
             const int total = cnt[0] * P;
             int slot = 0, steps = 0;
             WordQueue r;
             // state of the lane's current game
-            G g;    // general path, ordering-aware policy
-            GR gr;  // general path, uniform policy
+            G g;  // general path
             uint32_t h0 = 0, h1 = 0, rev = 0, cur = 0, drawn = kNone, winner = kNone;
             auto start = [&](int p) {
                 const int k = p / P;
@@ -227,7 +261,6 @@ __global__ void __launch_bounds__(MAXT, 1)
                 } else {
                     g = load_state(ls);
                     playout_begin(g, r, sp.cont_thr);
-                    if constexpr (!ORD) gr = to_gr(g);
                 }
                 // a may-stop leaf's first continue coin is a game step of its
                 // own (the fast path counts it as an iteration of its loop)
@@ -242,18 +275,13 @@ __global__ void __launch_bounds__(MAXT, 1)
                     if constexpr (FAST2) {
                         if (winner == kPend)
                             res = step_2p24_pending(h0, h1, cur, drawn, winner, r, sp.cont_thr, s_lut12);
-                        else if constexpr (ORD)
-                            res = step_2p24_ordered(h0, h1, rev, cur, drawn, winner, r, sp.cont_thr, s_lut12);
                         else
-                            res = step_2p24(h0, h1, rev, cur, drawn, winner, r, sp.cont_thr, s_magic, s_lut12);
-                    } else if constexpr (ORD) {
+                            res = step_2p24_ordered(h0, h1, rev, cur, drawn, winner, r, sp.cont_thr, s_lut12);
+                    } else {
                         r.ensure(4);
                         res = random_guess_ordered(g, r, sp.cont_thr);
                         if (res == kTurnOver) next_turn(g, r);
                         winner = g.winner;
-                    } else {
-                        res = step_gen(gr, r, sp.cont_thr, s_magic);
-                        winner = gr.winner;
                     }
                     ++steps;
                     if (res == kGameOver || steps >= 128) {
@@ -294,7 +322,8 @@ __global__ void __launch_bounds__(MAXT, 1)
     }
     if (F.words) {  // F.words[0]: random words, F.words[1]: game steps (guesses)
         const unsigned long long sum = warp_sum_u64((unsigned long long)words);
-        const unsigned long long st = warp_sum_u64((unsigned long long)nsteps);
+        // counted per lane, or (one game per lane) the same on every lane
+        const unsigned long long st = ORD ? warp_sum_u64((unsigned long long)nsteps) : (unsigned long long)nsteps;
         if (lane == 0 && sum) atomicAdd(F.words, sum);
         if (lane == 0 && st) atomicAdd(F.words + 1, st);
     }
