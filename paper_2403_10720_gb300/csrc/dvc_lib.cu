@@ -228,7 +228,8 @@ __global__ void __launch_bounds__(32 * kRollWarps, 8)
     rollout_kernel(const dvc_state* leaves, int n_leaves, int P, long long block0, uint64_t seed,
                    const uint32_t* tree_ids, const uint32_t* leaf_ids, uint32_t cont_thr, int skip2, int32_t* wins,
                    unsigned long long* words_out, int32_t* flags) {
-    __shared__ __align__(16) unsigned char s_sel[kSelBytes];
+    using Game = typename std::conditional<FAST2, Play2, PlayN>::type;
+    __shared__ __align__(16) unsigned char s_sel[SelectTable<Game::kChunk>::kBytes];
     __shared__ __align__(16) unsigned char s_ring[kRingBytes * kRollWarps];
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
     const long long total = (long long)n_leaves * P;
@@ -248,10 +249,9 @@ __global__ void __launch_bounds__(32 * kRollWarps, 8)
     const bool all2 = __all_sync(0xFFFFFFFFu, two);
     if ((FAST2 && !all2) || (!FAST2 && skip2 && all2)) busy = false;
     if (!__syncthreads_or(busy)) return;
-    fill_select(s_sel, tid, 32 * kRollWarps);
+    fill_select<Game::kChunk>(s_sel, tid, 32 * kRollWarps);
     __syncthreads();
     if (!__any_sync(0xFFFFFFFFu, busy)) return;
-    using Game = typename std::conditional<FAST2, Play2, PlayN>::type;
     Game g;
     PlayWords r;
     g.idle();
@@ -266,8 +266,8 @@ __global__ void __launch_bounds__(32 * kRollWarps, 8)
     }
     uint32_t words = 0u, steps = 0u;
     const uint32_t w = __any_sync(0xFFFFFFFFu, pend)
-                           ? play_games<Game, true, true>(g, r, busy, pend, seed, cont_thr, tab, words, steps)
-                           : play_games<Game, false, true>(g, r, busy, false, seed, cont_thr, tab, words, steps);
+                           ? play_games<Game, true, true, false>(g, r, busy, pend, seed, cont_thr, tab, words, steps)
+                           : play_games<Game, false, true, false>(g, r, busy, false, seed, cont_thr, tab, words, steps);
     credit_wins(wins, l, w);
     // no winner after 128 steps is a broken invariant
     if (busy && w >= 4u) latch_error(flags, DVC_E_INTERNAL);
@@ -339,14 +339,19 @@ __global__ void mcts_select_kernel(ForestDev F, SearchParams sp, int n, Descent*
     G det;
     det_sample(F.plans[t], F.tables + tm.table_off, root, dr, det);
     Descent dd;
-    descend(det, root.cur, F.nodes + tm.node_off, F.link + tm.node_off, F.ucb + tm.node_off, F.csl + tm.node_off, tm,
-            sp, (uint32_t)tm.done, paths + (size_t)t * kPathMax, movers + (size_t)t * kPathMax, s_E[wl], dd, nullptr,
-            set_table(F, tm));
+    TreeWords tw;
+    tw.open(sp.seed, tm.tree_id, (uint32_t)tm.done);
+    tw.b0 = tw.block(0u);
+    const Node* nodes = F.nodes + tm.node_off;
+    const Node r = nodes[0];
+    descend(det, root.cur, WalkNode{0, r.child, r.meta >> 12, F.csl[tm.node_off]}, nodes, F.link + tm.node_off,
+            F.ucb + tm.node_off, F.csl + tm.node_off, sp, tw, paths + (size_t)t * kPathMax,
+            movers + (size_t)t * kPathMax, s_E[wl], dd, set_table(F, tm));
     if (lane == 0) d = dd;
 }
 
 __global__ void mcts_expand_kernel(ForestDev F, int n, Descent* work, int32_t* paths, uint8_t* movers,
-                                   dvc_state* leaves, uint32_t* leaf_tree, uint32_t* leaf_iter, bool cont) {
+                                   dvc_state* leaves, uint32_t* leaf_tree, uint32_t* leaf_iter) {
     const int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (t >= n) return;
     const uint32_t lane = threadIdx.x & 31u;
@@ -367,8 +372,8 @@ __global__ void mcts_expand_kernel(ForestDev F, int n, Descent* work, int32_t* p
     int32_t used = tm.used;
     bool ok = true;
     if (d.found)
-        ok = expand_child(d, F.nodes + tm.node_off, F.link + tm.node_off, F.created + tm.node_off, tm, next_free,
-                          used, (uint32_t)tm.done, paths + (size_t)t * kPathMax, movers + (size_t)t * kPathMax, cont,
+        ok = expand_child(d, F.nodes + tm.node_off, F.link + tm.node_off, F.created + tm.node_off, tm, next_free, used,
+                          (uint32_t)tm.done, paths + (size_t)t * kPathMax, movers + (size_t)t * kPathMax,
                           set_table(F, tm));
     if (lane == 0) {
         tmr.next_free = next_free;
@@ -411,25 +416,16 @@ __global__ void root_stats_kernel(ForestDev F, int n, int32_t* out) {
     const uint32_t nchild = r.meta >> 12;
     int32_t best = -1, bv = 0, bw = 0;
     uint32_t brank = 0xFFFFFFFFu;
-    int32_t blk = r.child;
-    uint32_t seen = 0, k = 0;
-    while (seen < nchild) {
-        const uint32_t size = block_size(k, true, (uint32_t)tm.root_legal);
-        const uint32_t cnt = min(size, nchild - seen);
-        for (uint32_t e = 0; e < cnt; ++e) {
-            const Node c = nodes[blk + (int32_t)e];
-            const uint32_t code = c.meta & 0xFFFu;
-            const uint32_t rk = canon_rank(code, root.cur, root.np);
-            if (best < 0 || c.visits > bv || (c.visits == bv && rk < brank)) {
-                best = (int32_t)code;
-                bv = c.visits;
-                bw = c.wins;
-                brank = rk;
-            }
+    for (uint32_t i = 0; i < nchild; ++i) {
+        const Node c = nodes[r.child + (int32_t)i];
+        const uint32_t code = c.meta & 0xFFFu;
+        const uint32_t rk = canon_rank(code, root.cur, root.np);
+        if (best < 0 || c.visits > bv || (c.visits == bv && rk < brank)) {
+            best = (int32_t)code;
+            bv = c.visits;
+            bw = c.wins;
+            brank = rk;
         }
-        seen += cnt;
-        ++k;
-        if (seen < nchild) blk = F.link[tm.node_off + blk];
     }
     int32_t* o = out + 8 * t;
     o[0] = best;
@@ -463,20 +459,11 @@ __global__ void __launch_bounds__(256) root_stats_vanilla_kernel(ForestDev F, in
     for (uint32_t i = tid; i < nsets; i += blockDim.x) {
         const Node sn = nodes[r.child + (int32_t)i];
         const uint32_t nchild = sn.meta >> 12;
-        int32_t blk = sn.child;
-        uint32_t seen = 0, k = 0;
-        while (seen < nchild) {
-            const uint32_t size = block_size(k, false, 0u);
-            const uint32_t cnt = min(size, nchild - seen);
-            for (uint32_t e = 0; e < cnt; ++e) {
-                const Node c = nodes[blk + (int32_t)e];
-                const uint32_t code = c.meta & 0xFFFu;
-                atomicAdd(&s_v[code], c.visits);
-                atomicAdd(&s_w[code], c.wins);
-            }
-            seen += cnt;
-            ++k;
-            if (seen < nchild) blk = link[blk];
+        for (uint32_t e = 0; e < nchild; ++e) {
+            const Node c = nodes[child_slot(link, sn.child, e, false)];
+            const uint32_t code = c.meta & 0xFFFu;
+            atomicAdd(&s_v[code], c.visits);
+            atomicAdd(&s_w[code], c.wins);
         }
     }
     __syncthreads();
@@ -547,20 +534,11 @@ __global__ void __launch_bounds__(256) root_merge_kernel(ForestDev F, int K, int
         for (uint32_t pi = 0; pi < nparents; ++pi) {
             const Node pn = vanilla ? nodes[r.child + (int32_t)pi] : r;
             const uint32_t nchild = pn.meta >> 12;
-            int32_t blk = pn.child;
-            uint32_t seen = 0, kb = 0;
-            while (seen < nchild) {
-                const uint32_t size = block_size(kb, !vanilla, (uint32_t)tm.root_legal);
-                const uint32_t cnt = min(size, nchild - seen);
-                for (uint32_t e = tid; e < cnt; e += blockDim.x) {
-                    const Node c = nodes[blk + (int32_t)e];
-                    const uint32_t code = c.meta & 0xFFFu;
-                    atomicAdd(&s_v[code], c.visits);
-                    atomicAdd(&s_w[code], c.wins);
-                }
-                seen += cnt;
-                ++kb;
-                if (seen < nchild) blk = link[blk];
+            for (uint32_t e = tid; e < nchild; e += blockDim.x) {
+                const Node c = nodes[child_slot(link, pn.child, e, !vanilla)];
+                const uint32_t code = c.meta & 0xFFFu;
+                atomicAdd(&s_v[code], c.visits);
+                atomicAdd(&s_w[code], c.wins);
             }
         }
     }
@@ -625,18 +603,9 @@ __global__ void export_rows_kernel(ForestDev F, int t, const int32_t* iter_rank,
             out[4 * prow + 3] = nd.wins;
         }
         const uint32_t nchild = nd.meta >> 12;
-        int32_t blk = nd.child;
-        uint32_t seen = 0, k = 0;
-        while (seen < nchild) {
-            const uint32_t size = block_size(k, p == 0, (uint32_t)tm.root_legal);
-            const uint32_t cnt = min(size, nchild - seen);
-            for (uint32_t e = 0; e < cnt; ++e) {
-                const int32_t crow = iter_rank[created[blk + (int32_t)e]];
-                if (crow < rows) out[4 * crow + 1] = prow;
-            }
-            seen += cnt;
-            ++k;
-            if (seen < nchild) blk = link[blk];
+        for (uint32_t e = 0; e < nchild; ++e) {
+            const int32_t crow = iter_rank[created[child_slot(link, nd.child, e, p == 0)]];
+            if (crow < rows) out[4 * crow + 1] = prow;
         }
     }
 }
@@ -680,7 +649,6 @@ __device__ void init_tree(ForestDev& F, int t, DetPlan* plans, unsigned long lon
         r.child = -1;
         r.meta = 0u;
         nodes[0] = r;
-        F.link[tm.node_off] = -1;
         F.created[tm.node_off] = -1;
         pipe_np[t] = -1;  // no pipeline backprop pending
     }
@@ -1538,8 +1506,7 @@ int dvc_mcts_expand(dvc_forest* f, void* stream) {
     if (!f) return DVC_E_INVALID;
     if (int rc = set_device(f->ctx)) return rc;
     mcts_expand_kernel<<<(f->n * 32 + 127) / 128, 128, 0, (cudaStream_t)stream>>>(
-        dev_of(f), f->n, f->work, f->paths, f->movers, f->leaves, f->leaf_tree, f->leaf_iter,
-        f->ctx->cfg.tree_continue != 0);
+        dev_of(f), f->n, f->work, f->paths, f->movers, f->leaves, f->leaf_tree, f->leaf_iter);
     return check_launch(f->ctx, "mcts_expand_kernel");
 }
 

@@ -96,47 +96,64 @@ __global__ void __launch_bounds__(128)
     if (i >= i1) return;
     const int t = order ? order[i] : i;
     const uint32_t lane = threadIdx.x & 31u, wl = (threadIdx.x >> 5) & 3u;
-    pipe_apply_pending(F, sp, t, P);
+    // everything the walk starts from that the pending backprop does not
+    // change is loaded before it
     TreeMeta& tmr = F.meta[t];
     const TreeMeta tm = tmr;
-    if (tm.done >= P.step_end[t]) {
-        if (lane == 0) P.np[t] = -1;
-        return;
-    }
-    const uint32_t it = (uint32_t)tm.done;
+    const int32_t pending = P.np[t], step_end = P.step_end[t], base = P.det_base[t];
+    const int32_t done = tm.done + (pending >= 0 ? 1 : 0);
+    const uint32_t it = (uint32_t)done, ahead = it - (uint32_t)base;
+    const bool run = done < step_end;
     Node* nodes = F.nodes + tm.node_off;
     int32_t* link = F.link + tm.node_off;
-    const G root = load_state(F.roots[t]);
-    G det;
-    const uint32_t ahead = it - (uint32_t)P.det_base[t];
-    const uint4* tree0 = nullptr;
-    if (ahead < (uint32_t)kDetAhead) {
-        det = load_state(P.det[(size_t)t * kDetAhead + ahead]);
-        tree0 = P.tree0 + (size_t)t * kDetAhead + ahead;
-    } else {
-        Rng dr;
-        dr.open(sp.seed, tm.tree_id, 0u, it, kTagDet);
-        det_sample(F.plans[t], F.tables + tm.table_off, root, dr, det);
-    }
-    Descent d;
+    float2* ucb = F.ucb + tm.node_off;
+    float* csl = F.csl + tm.node_off;
     int32_t* path = P.path + (size_t)t * kPathMax;
     uint8_t* mover = P.mover + (size_t)t * kPathMax;
+    const Node root = nodes[0];
+    dvc_state ds = {};
+    uint4 tree0 = make_uint4(0u, 0u, 0u, 0u);
+    if (run && ahead < (uint32_t)kDetAhead) {
+        ds = P.det[(size_t)t * kDetAhead + ahead];
+        tree0 = P.tree0[(size_t)t * kDetAhead + ahead];
+    }
+    if (pending >= 0) {
+        backprop(nodes, ucb, csl, path, mover, pending, P.wins + 4 * t, sp.playouts, sp.c_uct);
+        __syncwarp();
+    }
+    if (!run || ahead >= (uint32_t)kDetAhead) {
+        if (lane == 0) {
+            tmr.done = done;
+            P.np[t] = -1;
+            if (run) {  // every iteration of a step is determinized ahead of it
+                P.step_end[t] = done;
+                latch_error(F.flags, DVC_E_INTERNAL);
+            }
+        }
+        return;
+    }
+    const G det = load_state(ds);
+    Descent d;
+    TreeWords tw;
+    tw.open(sp.seed, tm.tree_id, it);
+    tw.b0 = tree0;
     const SetTable st = VANILLA ? set_table(F, tm) : SetTable{nullptr, nullptr, 0u};
-    descend(det, root.cur, nodes, link, F.ucb + tm.node_off, F.csl + tm.node_off, tm, sp, it, path, mover, s_E[wl],
-            d, tree0, st);
+    // the determinization leaves the seat to move, who is the observer
+    descend(det, det.cur, WalkNode{0, root.child, root.meta >> 12, csl[0]}, nodes, link, ucb, csl, sp, tw, path, mover,
+            s_E[wl], d, st);
     bool ok = true;
     int32_t next_free = tm.next_free, used = tm.used;
     if (d.found)
-        ok = expand_child(d, nodes, link, F.created + tm.node_off, tm, next_free, used, it, path, mover,
-                          sp.tree_continue != 0, st);
+        ok = expand_child(d, nodes, link, F.created + tm.node_off, tm, next_free, used, it, path, mover, st);
     if (lane == 0) {
+        tmr.done = done;
         tmr.next_free = next_free;
         tmr.used = used;
         int32_t* w = P.wins + 4 * t;
-        w[0] = w[1] = w[2] = w[3] = 0;
+        *reinterpret_cast<int4*>(w) = make_int4(0, 0, 0, 0);
         if (!ok) {
             tmr.failed = 1;
-            P.step_end[t] = tm.done;
+            P.step_end[t] = done;
             P.np[t] = -1;
             latch_error(F.flags, DVC_E_OOM);
         } else {
@@ -165,16 +182,16 @@ template <bool FAST2, bool PEND, bool CNT>
 __global__ void __launch_bounds__(32 * kPlayWarps, FAST2 ? 12 : 8)
     pipe_play_kernel(SearchParams sp, int i0, int i1, long long block0, const int32_t* order, const TreeMeta* meta,
                      PipeBufs P, unsigned long long* words_out) {
-    __shared__ __align__(16) unsigned char s_sel[kSelBytes];
+    using Game = typename std::conditional<FAST2, Play2, PlayN>::type;
+    __shared__ __align__(16) unsigned char s_sel[SelectTable<Game::kChunk>::kBytes];
     __shared__ __align__(16) unsigned char s_ring[kRingBytes * kPlayWarps];
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
-    fill_select(s_sel, tid, 32 * kPlayWarps);
+    fill_select<Game::kChunk>(s_sel, tid, 32 * kPlayWarps);
     __syncthreads();
     const uint32_t Pp = (uint32_t)sp.playouts;
     const long long total = (long long)(i1 - i0) * Pp;
     const long long first = ((block0 + blockIdx.x) * kPlayWarps + warp) * 32;
     if (first >= total) return;
-    using Game = typename std::conditional<FAST2, Play2, PlayN>::type;
     Game g;
     PlayWords r;
     g.idle();
@@ -198,7 +215,7 @@ __global__ void __launch_bounds__(32 * kPlayWarps, FAST2 ? 12 : 8)
     }
     const bool mine = busy;
     uint32_t words = 0u, steps = 0u;
-    const uint32_t w = play_games<Game, PEND, CNT>(g, r, busy, pend, sp.seed, sp.cont_thr, tab, words, steps);
+    const uint32_t w = play_games<Game, PEND, CNT, false>(g, r, busy, pend, sp.seed, sp.cont_thr, tab, words, steps);
     credit_wins(P.wins, (uint32_t)t, w);
     // no winner after 128 steps is a broken invariant
     if (mine && w >= 4u) latch_error(P.flags, DVC_E_INTERNAL);

@@ -7,8 +7,8 @@
 //   1. tree phase -- warp w walks slots w, w+W, ...: take the iteration's
 //      determinization, descend by UCB1, expand one child, and publish the leaf;
 //   2. playout phase -- the P playouts of every published leaf form one pool;
-//      each warp takes the next 32 of it and plays them side by side
-//      (dvc_play.cuh), until the pool is empty;
+//      warp w plays games 32 w .. 32 w + 31 side by side (dvc_play.cuh), then
+//      those 32 W further on;
 //   3. backprop -- each warp adds its trees' playout results along their paths.
 // Trees stay strictly sequential (iteration i+1 sees i's statistics), which is
 // what makes results bit-exact with the single-threaded oracle, while every
@@ -83,7 +83,8 @@ __global__ void __launch_bounds__(MAXT, 1)
                      dvc_state* det_ahead, uint4* tree0_ahead) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ unsigned long long s_lut12[FAST2 && ORD ? 4096 : 1];
-    __shared__ __align__(16) unsigned char s_sel[ORD ? 16 : kSelBytes];
+    using Game = typename std::conditional<FAST2, Play2, PlayN>::type;
+    __shared__ __align__(16) unsigned char s_sel[ORD ? 16 : SelectTable<Game::kChunk>::kBytes];
     const int W = (int)(blockDim.x >> 5);
     const PoolLayout L(T, W);
     DetPlan* s_pl = (DetPlan*)(smem + L.pl);
@@ -118,7 +119,7 @@ __global__ void __launch_bounds__(MAXT, 1)
         }
     }
     if (tid < 8) s_cnt[tid] = 0;
-    if constexpr (!ORD) fill_select(s_sel, tid, blockDim.x);
+    if constexpr (!ORD) fill_select<Game::kChunk>(s_sel, tid, blockDim.x);
     else if constexpr (FAST2) fill_select12(s_lut12, tid, blockDim.x);
     __syncthreads();
 
@@ -157,20 +158,23 @@ __global__ void __launch_bounds__(MAXT, 1)
             Node* nodes = F.nodes + tm.node_off;
             int32_t* link = F.link + tm.node_off;
             int32_t* created = F.created + tm.node_off;
-            const G root = load_state(s_root[s]);
             const size_t a = (size_t)s_misc[4 * s + 2] * kDetAhead + (it - (uint32_t)s_base[s]);
             const G det = load_state(det_ahead[a]);
+            TreeWords tw;
+            tw.open(sp.seed, tm.tree_id, it);
+            tw.b0 = tree0_ahead[a];
+            const Node root = nodes[0];
             Descent d;
             int32_t* path = s_path + s * kPathMax;
             uint8_t* mover = s_mover + s * kPathMax;
             const SetTable st = set_table(F, tm);
-            descend(det, root.cur, nodes, link, F.ucb + tm.node_off, F.csl + tm.node_off, tm, sp, it, path, mover,
-                    s_E + warp * 104u, d, tree0_ahead + a, st);
+            // the determinization leaves the seat to move, who is the observer
+            descend(det, det.cur, WalkNode{0, root.child, root.meta >> 12, F.csl[tm.node_off]}, nodes, link,
+                    F.ucb + tm.node_off, F.csl + tm.node_off, sp, tw, path, mover, s_E + warp * 104u, d, st);
             bool ok = true;
             if (d.found) {
                 int32_t next_free = tm.next_free, used = tm.used;
-                ok = expand_child(d, nodes, link, created, tm, next_free, used, it, path, mover, sp.tree_continue != 0,
-                                  st);
+                ok = expand_child(d, nodes, link, created, tm, next_free, used, it, path, mover, st);
                 if (lane == 0) {
                     tm.next_free = next_free;
                     tm.used = used;
@@ -205,15 +209,10 @@ __global__ void __launch_bounds__(MAXT, 1)
         __syncthreads();
         // ---- 2. playout phase: P playouts of each listed leaf
         if constexpr (!ORD) {
-            // 32 games at a time per warp, one per lane, until the pool is empty
-            using Game = typename std::conditional<FAST2, Play2, PlayN>::type;
+            // 32 games at a time per warp, one per lane
             const uint32_t P = (uint32_t)sp.playouts, total = (uint32_t)cnt[0] * P;
             const uint32_t tab = shared_addr(s_sel);
-            for (;;) {
-                uint32_t first = 0;
-                if (lane == 0) first = (uint32_t)atomicAdd(&cnt[1], 32);
-                first = __shfl_sync(0xFFFFFFFFu, first, 0);
-                if (first >= total) break;
+            for (uint32_t first = warp * 32u; first < total; first += blockDim.x) {
                 Game g;
                 PlayWords r;
                 g.idle();
@@ -232,7 +231,7 @@ __global__ void __launch_bounds__(MAXT, 1)
                     r.open(sp.seed, s_tm[slot].tree_id, p - k * P, (uint32_t)s_tm[slot].done);
                 }
                 const uint32_t w =
-                    play_games<Game, true, true>(g, r, busy, pend, sp.seed, sp.cont_thr, tab, words, nsteps);
+                    play_games<Game, true, true, FAST2>(g, r, busy, pend, sp.seed, sp.cont_thr, tab, words, nsteps);
                 credit_wins(s_wins, (uint32_t)slot, w);
                 // no winner after 128 steps is a broken invariant
                 if (busy && w >= 4u) latch_error(F.flags, DVC_E_INTERNAL);

@@ -7,9 +7,21 @@
 // The children of a node live in blocks of consecutive slots -- the root's
 // first block is sized to its legal-guess count (fixed for the whole search),
 // other nodes' blocks grow 4, 8, 16, 32, 32, ... -- so a warp reads a block
-// with one coalesced load.  A block's successor is recorded in `link` at the
-// block's first slot.  With blocks no larger than four times the children
-// they hold, root block + 4 * budget slots always suffice.
+// with one coalesced load.  Block k >= 1 of a node is recorded in `link` at
+// the slot of the node's child k - 1: the first four links stand side by side
+// at the first block, so a warp knows the places of up to 92 children after
+// one load instead of following a chain of one link per block.  With blocks no
+// larger than four times the children they hold, root block + 4 * budget slots
+// always suffice.
+//
+// The walk is a chain of dependent steps of one warp, so what bounds it is
+// latency: loads one after another, the instructions between them, and their
+// fetch.  A level costs one load of the children (with their UCB1 terms, and
+// all that the next level needs of them: child block, child count, exploration
+// term) and, with more than four children, one of the links before it, both
+// issued ahead of the work that does not need them.  The determinized rows are
+// laid out one tile per lane, so slots, targets and draws are ballots and
+// warp-wide reductions instead of bit selects through tables.
 //
 // Vanilla MCTS-dvc (Sec. III-A): the root's children are plausible-number
 // sets, one per distinct assignment of the tiles the observer cannot see, and
@@ -21,7 +33,7 @@
 
 namespace dvc {
 
-struct Node {
+struct __align__(16) Node {
     int32_t visits;
     int32_t wins;
     int32_t child;  // slot of the first child block, -1 if none
@@ -116,49 +128,208 @@ struct SearchParams {
     int32_t tree_continue;  // 1: a correct in-tree guess keeps the turn (Fig. 2a)
 };
 
-__device__ __forceinline__ uint32_t block_size(uint32_t k, bool is_root, uint32_t root_legal) {
-    if (is_root && k == 0) return root_legal > 0u ? root_legal : 1u;
-    return k >= 3 ? 32u : (4u << k);
+// Child c of a node other than the root stands in block block_of(c) at
+// block_off(c); block k holds block_size(k) slots.
+__device__ __forceinline__ uint32_t block_of(uint32_t c) {
+    return c < 4u ? 0u : c < 12u ? 1u : c < 28u ? 2u : 3u + ((c - 28u) >> 5);
+}
+__device__ __forceinline__ uint32_t block_off(uint32_t c) {
+    return c < 4u ? c : c < 12u ? c - 4u : c < 28u ? c - 12u : (c - 28u) & 31u;
+}
+__device__ __forceinline__ uint32_t block_size(uint32_t k) { return k >= 3u ? 32u : 4u << k; }
+
+// Slot of child c: block k >= 1 is linked from child k - 1, so block_of(k - 1)
+// < k and the chain of blocks that leads to c is short (at most four for 4,095
+// children).  single: the root, whose children are one block.
+__device__ __forceinline__ int32_t child_slot(const int32_t* link, int32_t blk0, uint32_t c, bool single) {
+    if (single) return blk0 + (int32_t)c;
+    uint32_t at[4];
+    int n = 0;
+    uint32_t k = block_of(c);
+    while (k > 0u && n < 4) {
+        at[n++] = k - 1u;
+        k = block_of(k - 1u);
+    }
+    int32_t blk = blk0;
+    for (int i = n - 1; i >= 0; --i) blk = link[blk + (int32_t)block_off(at[i])];
+    return blk + (int32_t)block_off(c);
 }
 
-// What a descent produced: either a node to expand (found = 1, action act)
-// or a leaf to score (found = 0).
+// A node's blocks by lane: lane k holds block k's first slot, for as many of
+// the first 32 blocks as nchild children need (they hold 956 children).  All
+// lanes call.
+constexpr uint32_t kDirChildren = 28u + 29u * 32u;
+__device__ __forceinline__ int32_t block_dir(const int32_t* link, int32_t blk0, uint32_t nchild) {
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint32_t last = block_of(nchild - 1u);  // callers have nchild > 0
+    int32_t dir = blk0;
+    if (lane >= 1u && lane <= min(last, 4u)) dir = link[blk0 + (int32_t)lane - 1];
+    if (last > 4u) {  // blocks 5-12 are linked from block 1, 13-28 from block 2, the rest from block 3
+        const int32_t b1 = __shfl_sync(0xFFFFFFFFu, dir, 1), b2 = __shfl_sync(0xFFFFFFFFu, dir, 2);
+        const int32_t b3 = __shfl_sync(0xFFFFFFFFu, dir, 3);
+        const int32_t from = lane < 13u ? b1 - 5 : lane < 29u ? b2 - 13 : b3 - 29;
+        if (lane > 4u && lane <= last) dir = link[from + (int32_t)lane];
+    }
+    return dir;
+}
+
+// The words of an iteration's tree stream (tag 3), the same on every lane:
+// block 0 is given (b0, sampled ahead or block(0)); the blocks after it are
+// computed at the first need, one per lane.
+struct TreeWords {
+    uint32_t k0, k1, i, tw;
+    uint4 b0, more;  // block 0; this lane's block 1 + lane
+    uint32_t used;
+    bool ahead;
+
+    __device__ __forceinline__ uint4 block(uint32_t blk) const {
+        uint32_t a = blk, b = 0u, c = i, d = tw;
+        philox10(a, b, c, d, k0, k1);
+        return make_uint4(a, b, c, d);
+    }
+    __device__ __forceinline__ void open(uint64_t seed, uint32_t tree, uint32_t it) {
+        k0 = (uint32_t)seed;
+        k1 = tree;
+        i = it;
+        tw = kTagTree + 16u * (uint32_t)(seed >> 32);
+        used = 0u;
+        ahead = false;
+    }
+    // Make the next two words (the most a ply takes) available.
+    __device__ __forceinline__ void ensure() {
+        if (used > 2u && !ahead) {
+            more = block(1u + (threadIdx.x & 31u));
+            ahead = true;
+        }
+    }
+    __device__ __forceinline__ uint32_t next() {
+        const uint32_t n = used++, k = n & 3u;
+        const uint4 q = n < 4u ? b0 : more;
+        const uint32_t v = k == 0u ? q.x : k == 1u ? q.y : k == 2u ? q.z : q.w;
+        // at most two words per ply and at most kPathMax plies: 32 blocks suffice
+        return n < 4u ? v : __shfl_sync(0xFFFFFFFFu, v, (n - 4u) >> 2);
+    }
+};
+
+// The rows of a state laid out one tile per lane (lanes 0..25): the seat that
+// holds tile `lane` (4: nobody) and the tile's place in that seat's row.
+struct Rows {
+    uint32_t owner, pos;
+    __device__ __forceinline__ Rows(const G& g) {
+        const uint32_t lane = threadIdx.x & 31u, bit = lane < 26u ? 1u << lane : 0u;
+        uint32_t hp = 0u;
+        owner = 4u;
+        if (g.h0 & bit) { owner = 0u; hp = g.h0; }
+        if (g.h1 & bit) { owner = 1u; hp = g.h1; }
+        if (g.h2 & bit) { owner = 2u; hp = g.h2; }
+        if (g.h3 & bit) { owner = 3u; hp = g.h3; }
+        pos = __popc(hp & kNumMask & (bit - 1u));
+        if (g.tmask & kJokerMask) {
+            if (lane >= 24u) {
+                if (owner < 4u) pos = joker_pos(g, hp, lane - 24u);
+            } else {
+                const uint32_t k = pos;
+                if ((hp >> 24) & 1u) pos += g.jg0 <= k;
+                if ((hp >> 25) & 1u) pos += g.jg1 <= k;
+            }
+        }
+    }
+    // Face-down places of seat q's row.
+    __device__ __forceinline__ uint32_t hidden(const G& g, uint32_t q) const {
+        const bool in = owner == q && !((g.rev >> (threadIdx.x & 31u)) & 1u) && ((g.alive >> q) & 1u);
+        return __reduce_or_sync(0xFFFFFFFFu, in ? 1u << pos : 0u);
+    }
+};
+
+// tree_apply (dvc_device.cuh) by a whole warp: the same transition and words,
+// the state the same on every lane before and after.
+__device__ __forceinline__ void warp_apply(G& g, const Rows& v, uint32_t code, TreeWords& tw, bool cont) {
+    const uint32_t lane = threadIdx.x & 31u, cur = g.cur;
+    const bool was_stop = code == kStop;
+    if (!was_stop) {
+        const uint32_t q = code >> 10, sl = (code >> 5) & 31u, x = code & 31u;
+        const unsigned at = __ballot_sync(0xFFFFFFFFu, v.owner == q && v.pos == sl);
+        const uint32_t target = at ? (uint32_t)__ffs(at) - 1u : 0u;
+        const bool hit = x == target;
+        uint32_t tb = 1u << target;
+        if (!hit) {
+            uint32_t t = g.drawn;
+            if (t == kNone) {  // the leftmost face-down tile
+                const bool mine = v.owner == cur && !((g.rev >> lane) & 1u);
+                t = __reduce_min_sync(0xFFFFFFFFu, mine ? v.pos << 5 | lane : 0xFFFFu) & 31u;
+            }
+            tb = 1u << t;
+        }
+        g.rev |= tb;
+        const uint32_t seat = hit ? q : cur;
+        if (!(g.hand(seat) & ~g.rev)) g.alive &= ~(1u << seat);
+        g.mstop = 0u;
+        if (__popc(g.alive) == 1) {
+            g.winner = hit ? cur : (uint32_t)__ffs(g.alive) - 1u;
+            return;
+        }
+        if (cont && hit) {
+            g.mstop = 1u;
+            return;
+        }
+    }
+    g.mstop = 0u;
+    g.cur = next_alive(g.alive, cur, g.np);
+    const uint32_t pool = g.pool();
+    if (!pool) {
+        g.drawn = kNone;
+        return;
+    }
+    tw.ensure();
+    const uint32_t n = __umulhi(tw.next(), __popc(pool));
+    const bool here = ((pool >> lane) & 1u) && (uint32_t)__popc(pool & ((1u << lane) - 1u)) == n;
+    const uint32_t t = (uint32_t)__ffs(__ballot_sync(0xFFFFFFFFu, here)) - 1u;
+    insert_gaps(g, g.hand(g.cur), t, tw);
+    g.add(g.cur, 1u << t);
+    g.drawn = t;
+}
+
+// What a descent produced: a node to expand (found = 1, action act) or none
+// (found = 0), and the state to score: after the new action, or at the node.
 struct Descent {
-    G s;              // state at the node reached
-    Rng tr;           // tree stream after the in-tree draws so far
+    G s;
     int32_t node;     // slot reached
     int32_t found;    // 1: expand `act` below `node`
     uint32_t act;
+    uint32_t who;     // the seat that makes it
     int32_t nchild;   // children of `node`
-    int32_t last_blk, last_size, last_cnt, nblocks;
+    int32_t blk;      // first child block of `node`, -1 if none
     int32_t np;       // path length
     uint32_t set_cell;  // vanilla, act == kSet: the table cell for the new set
     uint4 set_key;      // vanilla, act == kSet: its key
 };
 
-// Warp-cooperative descent from the root for iteration `it`.  All 32 lanes
+// A node of the walk: slot, children, first child block, c * sqrt(ln visits).
+struct WalkNode {
+    int32_t slot, blk;
+    uint32_t nchild;
+    float csl;
+};
+
+// Warp-cooperative descent from the root for one iteration.  All 32 lanes
 // of the calling warp enter with the same arguments and leave with the same
 // Descent; lane 0 records the path in path[] / mover[] (shared or global).
-// E is a 4 x 26 word scratch (shared memory) for expanded-identity masks.
+// at: the root's node.  E is a 4 x 26 word scratch (shared memory) for
+// expanded-identity masks.  tw: the iteration's tree stream, opened.
 // ucb[slot] = (wins/n, 1/sqrt(n)) and csl[slot] = c * sqrt(ln n) are the
 // node's UCB1 terms, refreshed whenever its counts change (backprop), so a
 // selection scan costs one multiply-add per child.  They are the same IEEE
 // values a scan would compute from the counts.
-// tree0 (optional): the first block of the iteration's tree stream, computed
-// ahead of time (the same four words the stream would generate).
 // st: the plausible-set table of a vanilla tree.  The determinization's set
 // node is the first step below the root; a set not seen before is this
 // iteration's expansion (act = kSet) and its leaf is the determinized root.
-__device__ __forceinline__ void descend(const G& det, uint32_t obs, const Node* nodes, const int32_t* link,
-                                        const float2* ucb, const float* csl_of, const TreeMeta& tm,
-                                        const SearchParams& sp, uint32_t it, int32_t* path, uint8_t* mover,
-                                        uint32_t* E, Descent& d, const uint4* tree0 = nullptr,
+__device__ __forceinline__ void descend(const G& det, uint32_t obs, WalkNode at, const Node* nodes,
+                                        const int32_t* link, const float2* ucb, const float* csl_of,
+                                        const SearchParams& sp, TreeWords& tw, int32_t* path, uint8_t* mover,
+                                        uint32_t* E, Descent& d,
                                         const SetTable& st = SetTable{nullptr, nullptr, 0u}) {
     const uint32_t lane = threadIdx.x & 31u;
     d.s = det;
-    d.tr.open(sp.seed, tm.tree_id, 0u, it, kTagTree);
-    if (tree0) d.tr.preload(*tree0);
-    d.node = 0;
     d.found = 0;
     d.np = 1;
     if (lane == 0) {
@@ -172,17 +343,14 @@ __device__ __forceinline__ void descend(const G& det, uint32_t obs, const Node* 
         const int32_t slot = set_find(st, key, cell);
         if (slot < 0) {
             // a new set: appended to the root's single child block
-            const Node r = nodes[0];
-            const int32_t nsets = (int32_t)(r.meta >> 12);
             d.found = 1;
             d.act = kSet;
+            d.who = d.s.cur;
             d.set_cell = cell;
             d.set_key = key;
-            d.nchild = nsets;
-            d.nblocks = nsets ? 1 : 0;
-            d.last_blk = nsets ? r.child : -1;
-            d.last_size = tm.root_legal;
-            d.last_cnt = nsets;
+            d.node = 0;
+            d.nchild = (int32_t)at.nchild;
+            d.blk = at.blk;
             return;
         }
         if (lane == 0) {
@@ -190,169 +358,205 @@ __device__ __forceinline__ void descend(const G& det, uint32_t obs, const Node* 
             mover[1] = (uint8_t)obs;
         }
         d.np = 2;
-        d.node = slot;
+        const Node sn = nodes[slot];
+        at.slot = slot;
+        at.blk = sn.child;
+        at.nchild = sn.meta >> 12;
+        at.csl = csl_of[slot];
     }
     while (d.s.winner == kNone && depth < (uint32_t)sp.d_max) {
-        // loads that do not depend on one another are issued together: the
-        // node and its exploration term; below, each child with its UCB1
-        // terms, and the next block's start before this block is scanned
-        const Node nd = nodes[d.node];
-        const float csl_node = csl_of[d.node];  // any slot's entry exists; used only if it has children
-        const uint32_t nchild = nd.meta >> 12;
-        const uint32_t cur = d.s.cur;
+        const uint32_t cur = d.s.cur, np = d.s.np;
+        const bool single = at.slot == 0;
+        const bool wide = !single && at.nchild > 0u;
+        const int32_t dir = wide ? block_dir(link, at.blk, at.nchild) : at.blk;
+        // the legal actions of this determinization: STOP when allowed, and
+        // face-down places of the opponents x identities the mover cannot see
         const uint32_t U = d.s.tmask & ~d.s.hand(cur) & ~d.s.rev;
-        for (uint32_t e = lane; e < 104u; e += 32u) E[e] = 0u;
-        __syncwarp();
-        const float csl = nchild ? csl_node : 0.0f;
-        float best_sc = -1.0f;
-        uint32_t best_rank = 0xFFFFFFFFu;
-        int32_t best_slot = -1;
-        uint32_t best_code = 0;
-        int32_t blk = nd.child;
-        uint32_t seen = 0, k = 0;
-        bool stop_child = false;  // this lane saw the node's STOP child
-        d.last_blk = -1;
-        d.last_size = 0;
-        d.last_cnt = 0;
-        while (seen < nchild) {
-            const uint32_t size = block_size(k, d.node == 0, (uint32_t)tm.root_legal);
-            const uint32_t cnt = min(size, nchild - seen);
-            const int32_t next_blk = seen + cnt < nchild ? link[blk] : -1;
-            for (uint32_t e = lane; e < cnt; e += 32u) {
-                const Node ch = nodes[blk + (int32_t)e];
-                const float2 u = ucb[blk + (int32_t)e];  // set by the child's first backprop
-                const uint32_t code = ch.meta & 0xFFFu;
-                const uint32_t q = code >> 10, sl = (code >> 5) & 31u, x = code & 31u;
-                stop_child |= code == kStop;
-                if (code != kStop && sl < 26u) atomicOr(&E[q * 26u + sl], 1u << x);
-                if (action_legal(d.s, code)) {
-                    const float sc = __fadd_rn(u.x, __fmul_rn(csl, u.y));
-                    const uint32_t rk = canon_rank(code, cur, d.s.np);
-                    if (best_slot < 0 || sc > best_sc || (sc == best_sc && rk < best_rank)) {
+        uint32_t q1 = cur + 1u, q2 = cur + 2u, q3 = cur + 3u;
+        q1 = q1 >= np ? q1 - np : q1;
+        q2 = q2 >= np ? q2 - np : q2;
+        q3 = q3 >= np ? q3 - np : q3;
+        const Rows rows(d.s);
+        const uint32_t m1 = rows.hidden(d.s, q1);
+        uint32_t m2 = 0u, m3 = 0u;
+        if (np > 2u) m2 = rows.hidden(d.s, q2);
+        if (np > 3u) m3 = rows.hidden(d.s, q3);
+        const uint32_t legal =
+            (uint32_t)(__popc(m1) + __popc(m2) + __popc(m3)) * (uint32_t)__popc(U) + (d.s.mstop ? 1u : 0u);
+        if (legal == 0u) break;  // not in a running game
+        // slot of child c (a lane's own; every lane of the warp calls)
+        auto place = [&](uint32_t c) -> int32_t {
+            if (!wide) return at.blk + (int32_t)c;
+            const int32_t b = __shfl_sync(0xFFFFFFFFu, dir, block_of(c) & 31u);
+            if (c >= kDirChildren && c < at.nchild) return child_slot(link, at.blk, c, false);
+            return b + (int32_t)block_off(c);
+        };
+        uint32_t left = legal;  // legal actions without a child
+        uint32_t act = kStop;
+        float best_sc = 0.0f;
+        uint32_t best_rank = 0xFFFFFFFFu, best_meta = 0u;
+        int32_t best_slot = -1, best_blk = -1;
+        float best_csl = 0.0f;
+        if (at.nchild >= legal) {
+            // perhaps every legal action has its child: score the legal ones,
+            // two chunks of 32 children in flight
+            uint32_t seen = 0u;
+            for (uint32_t c0 = 0; c0 < at.nchild; c0 += 64u) {
+                Node ch[2];
+                float2 u[2];
+                float cs[2];
+                int32_t sl[2];
+#pragma unroll
+                for (uint32_t h = 0; h < 2u; ++h) {
+                    const uint32_t c = c0 + 32u * h + lane;
+                    sl[h] = -1;
+                    if (c0 + 32u * h < at.nchild) {
+                        const int32_t s = place(c);
+                        if (c < at.nchild) {
+                            sl[h] = s;
+                            ch[h] = nodes[s];
+                            u[h] = ucb[s];  // set by the child's first backprop
+                            cs[h] = csl_of[s];
+                        }
+                    }
+                }
+#pragma unroll
+                for (uint32_t h = 0; h < 2u; ++h) {
+                    if (sl[h] < 0) continue;
+                    const uint32_t code = ch[h].meta & 0xFFFu;
+                    const uint32_t q = code >> 10, x = code & 31u;
+                    const uint32_t off = q > cur ? q - cur - 1u : q + np - cur - 1u;
+                    const uint32_t m = off == 0u ? m1 : off == 1u ? m2 : m3;
+                    bool ok = ((m >> ((code >> 5) & 31u)) & 1u) && ((U >> x) & 1u) && q != cur;
+                    uint32_t rank = 1u + (off << 10 | (code & 1023u));  // canonical order, STOP first
+                    if (code == kStop) {
+                        ok = d.s.mstop != 0u;
+                        rank = 0u;
+                    }
+                    if (!ok) continue;
+                    ++seen;
+                    const float sc = __fadd_rn(u[h].x, __fmul_rn(at.csl, u[h].y));
+                    if (best_slot < 0 || sc > best_sc || (sc == best_sc && rank < best_rank)) {
                         best_sc = sc;
-                        best_rank = rk;
-                        best_slot = blk + (int32_t)e;
-                        best_code = code;
+                        best_rank = rank;
+                        best_slot = sl[h];
+                        best_meta = ch[h].meta;
+                        best_blk = ch[h].child;
+                        best_csl = cs[h];
                     }
                 }
             }
-            seen += cnt;
-            d.last_blk = blk;
-            d.last_size = (int32_t)size;
-            d.last_cnt = (int32_t)cnt;
-            ++k;
-            if (seen < nchild) blk = next_blk;
+            left = legal - __reduce_add_sync(0xFFFFFFFFu, seen);
         }
-        d.nblocks = (int32_t)k;
-        d.nchild = (int32_t)nchild;
-        __syncwarp();
-        // first legal action without a child, canonical order (STOP first)
-        uint32_t act = 0;
-        bool found = false;
-        if (d.s.mstop && !__any_sync(0xFFFFFFFFu, stop_child)) {
-            act = kStop;
-            found = true;
-        }
-        for (uint32_t off = 1; off < d.s.np && !found; ++off) {
-            uint32_t q = cur + off;
-            q = q >= d.s.np ? q - d.s.np : q;
-            if (!((d.s.alive >> q) & 1u)) continue;
-            const uint32_t nh = __popc(d.s.hand(q) & ~d.s.rev);
-            for (uint32_t h0 = 0; h0 < nh && !found; h0 += 32u) {
-                const uint32_t h = h0 + lane;
-                uint32_t avail = 0u, sp_ = 0u;
-                if (h < nh) {
-                    const uint32_t t = hidden_slot(d.s, q, h);
-                    sp_ = seq_pos(d.s, q, t);
-                    if (sp_ < 26u) avail = U & ~E[q * 26u + sp_];
+        if (left) {
+            // the first legal action without a child, in canonical order
+            bool stop_child = false;
+            if (at.nchild) {
+                for (uint32_t e = lane; e < 104u; e += 32u) E[e] = 0u;
+                __syncwarp();
+                for (uint32_t c0 = 0; c0 < at.nchild; c0 += 32u) {
+                    const uint32_t c = c0 + lane;
+                    const int32_t s = place(c);
+                    if (c >= at.nchild) continue;
+                    const uint32_t code = nodes[s].meta & 0xFFFu;
+                    const uint32_t sl = (code >> 5) & 31u;
+                    if (code == kStop) stop_child = true;
+                    else if (sl < 26u) atomicOr(&E[(code >> 10) * 26u + sl], 1u << (code & 31u));
                 }
-                const uint32_t bal = __ballot_sync(0xFFFFFFFFu, avail != 0u);
-                if (bal) {
-                    const uint32_t L = __ffs(bal) - 1u;
-                    const uint32_t spL = __shfl_sync(0xFFFFFFFFu, sp_, L);
-                    const uint32_t avL = __shfl_sync(0xFFFFFFFFu, avail, L);
-                    act = (q << 10) | (spL << 5) | ((uint32_t)__ffs(avL) - 1u);
-                    found = true;
+                __syncwarp();
+            }
+            if (!d.s.mstop || __any_sync(0xFFFFFFFFu, stop_child)) {
+                for (uint32_t off = 0; off < 3u; ++off) {
+                    const uint32_t m = off == 0u ? m1 : off == 1u ? m2 : m3;
+                    const uint32_t q = off == 0u ? q1 : off == 1u ? q2 : q3;
+                    uint32_t avail = (m >> lane) & 1u ? U : 0u;
+                    if (avail && at.nchild) avail &= ~E[q * 26u + lane];
+                    const unsigned bal = __ballot_sync(0xFFFFFFFFu, avail != 0u);
+                    if (bal) {
+                        const uint32_t sl = (uint32_t)__ffs(bal) - 1u;
+                        const uint32_t av = __shfl_sync(0xFFFFFFFFu, avail, sl);
+                        act = (q << 10) | (sl << 5) | ((uint32_t)__ffs(av) - 1u);
+                        break;
+                    }
                 }
             }
-        }
-        if (found) {
+            __syncwarp();  // E is read before a later walk of this warp clears it
             d.found = 1;
+            d.who = cur;
             d.act = act;
-            return;
-        }
-        // UCB1 argmax over lanes: higher score, then lower canonical rank
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const float osc = __shfl_xor_sync(0xFFFFFFFFu, best_sc, o);
-            const uint32_t ork = __shfl_xor_sync(0xFFFFFFFFu, best_rank, o);
-            const int32_t osl = __shfl_xor_sync(0xFFFFFFFFu, best_slot, o);
-            const uint32_t ocd = __shfl_xor_sync(0xFFFFFFFFu, best_code, o);
-            const bool take = osl >= 0 && (best_slot < 0 || osc > best_sc || (osc == best_sc && ork < best_rank));
-            if (take) {
-                best_sc = osc;
-                best_rank = ork;
-                best_slot = osl;
-                best_code = ocd;
+            d.node = at.slot;
+            d.nchild = (int32_t)at.nchild;
+            d.blk = at.blk;
+        } else {
+            // UCB1 argmax over lanes: highest score (scores are not negative,
+            // so their bits order like them), then lowest canonical rank
+            const uint32_t key = best_slot < 0 ? 0u : __float_as_uint(best_sc) + 1u;
+            const uint32_t top = __reduce_max_sync(0xFFFFFFFFu, key);
+            const uint32_t win =
+                __reduce_min_sync(0xFFFFFFFFu, key == top ? best_rank << 5 | lane : 0xFFFFFFFFu) & 31u;
+            const uint32_t meta = __shfl_sync(0xFFFFFFFFu, best_meta, win);
+            at.slot = __shfl_sync(0xFFFFFFFFu, best_slot, win);
+            at.blk = __shfl_sync(0xFFFFFFFFu, best_blk, win);
+            at.csl = __shfl_sync(0xFFFFFFFFu, best_csl, win);
+            at.nchild = meta >> 12;
+            act = meta & 0xFFFu;
+            if (lane == 0) {
+                path[d.np] = at.slot;
+                mover[d.np] = (uint8_t)cur;
             }
+            d.np++;
+            ++depth;
         }
-        const uint32_t who = d.s.cur;
-        tree_apply(d.s, best_code, d.tr, sp.tree_continue != 0);
-        if (lane == 0) {
-            path[d.np] = best_slot;
-            mover[d.np] = (uint8_t)who;
-        }
-        d.np++;
-        d.node = best_slot;
-        ++depth;
+        warp_apply(d.s, rows, act, tw, sp.tree_continue != 0);
+        if (d.found) break;
     }
 }
 
-// Create the child found by descend() and step the state through its action
-// (a new plausible set is entered in the tree's set table and leaves the state
-// as it is).  Lane-uniform; lane 0 writes memory.  next_free is the tree's
-// allocator (uniform register copy).  Returns false if the arena is exhausted.
+// Create the child found by descend() (a new plausible set is entered in the
+// tree's set table).  Lane-uniform; lane 0 writes memory.  next_free is the
+// tree's allocator (uniform register copy).  Returns false if the arena is
+// exhausted.
 __device__ __forceinline__ bool expand_child(Descent& d, Node* nodes, int32_t* link, int32_t* created,
                                              const TreeMeta& tm, int32_t& next_free, int32_t& used, uint32_t it,
-                                             int32_t* path, uint8_t* mover, bool cont,
+                                             int32_t* path, uint8_t* mover,
                                              const SetTable& st = SetTable{nullptr, nullptr, 0u}) {
     const uint32_t lane = threadIdx.x & 31u;
+    const uint32_t c = (uint32_t)d.nchild;
+    const bool single = d.node == 0;  // the root's one block holds every child it can have
     int32_t slot;
-    if (d.nchild == 0 || d.last_cnt >= d.last_size) {
+    if (c == 0u || (!single && block_off(c) == 0u)) {
         // a new child block: first block of this node, or the last one is full
-        const uint32_t k = d.nchild == 0 ? 0u : (uint32_t)d.nblocks;
-        const int32_t size = (int32_t)block_size(k, d.node == 0, (uint32_t)tm.root_legal);
+        const int32_t size = single ? (tm.root_legal > 0 ? tm.root_legal : 1) : (int32_t)block_size(block_of(c));
         if (next_free + size > tm.cap) return false;
         slot = next_free;
         next_free += size;
         for (int32_t e = (int32_t)lane; e < size; e += 32) created[slot + e] = -1;  // slots not yet nodes
         if (lane == 0) {
-            if (d.nchild == 0) nodes[d.node].child = slot;
-            else link[d.last_blk] = slot;
-            link[slot] = -1;
+            if (c == 0u) nodes[d.node].child = slot;
+            else link[child_slot(link, d.blk, block_of(c) - 1u, false)] = slot;
         }
+        __syncwarp();
     } else {
-        slot = d.last_blk + d.last_cnt;
+        if (single && (int32_t)c >= tm.root_legal) return false;  // unreachable: the block holds every child
+        slot = child_slot(link, d.blk, c, single);
     }
     if (lane == 0) {
-        Node c;
-        c.visits = 0;
-        c.wins = 0;
-        c.child = -1;
-        c.meta = d.act;
-        nodes[slot] = c;
+        Node n;
+        n.visits = 0;
+        n.wins = 0;
+        n.child = -1;
+        n.meta = d.act;
+        nodes[slot] = n;
         created[slot] = (int32_t)it;
         nodes[d.node].meta += 1u << 12;
         path[d.np] = slot;
-        mover[d.np] = (uint8_t)d.s.cur;
+        mover[d.np] = (uint8_t)d.who;
         if (d.act == kSet) {
             st.key[d.set_cell] = d.set_key;
             st.slot[d.set_cell] = slot;
         }
     }
-    if (d.act != kSet) tree_apply(d.s, d.act, d.tr, cont);
     d.np++;
-    d.node = slot;
     ++used;
     return true;
 }
@@ -372,10 +576,10 @@ __device__ __forceinline__ void backprop(Node* nodes, float2* ucb, float* csl, c
     for (int32_t e = (int32_t)lane; e < np; e += 32) {
         const int32_t slot = path[e];
         Node* n = &nodes[slot];
-        const int32_t v = n->visits + playouts;
-        const int32_t w = n->wins + wins[mover[e]];
-        n->visits = v;
-        n->wins = w;
+        const int2 vw = *reinterpret_cast<const int2*>(n);
+        const int32_t v = vw.x + playouts;
+        const int32_t w = vw.y + wins[mover[e]];
+        *reinterpret_cast<int2*>(n) = make_int2(v, w);
         const float dv = __int2float_rn(v);
         ucb[slot] = make_float2(__fdiv_rn(__int2float_rn(w), dv), __fdiv_rn(1.0f, __fsqrt_rn(dv)));
         csl[slot] = __fmul_rn(c_uct, __fsqrt_rn(ln_series(dv)));
