@@ -94,7 +94,12 @@ struct dvc_forest {
 
 namespace {
 
-constexpr int kDetChunk = 256;
+// dvc_determinize: CTAs, and table slots in the workspace (128 MB); tables of
+// up to kDetSharedCells cells stand in shared memory instead (48 KB, four CTAs
+// per SM).
+constexpr int kDetSlots = 512;
+constexpr uint32_t kDetSharedCells = 6144;
+constexpr int kDetThreads = 256;
 
 __device__ __forceinline__ void latch(int32_t* flags, int32_t code) { atomicCAS(&flags[0], 0, code); }
 
@@ -171,28 +176,40 @@ __global__ void init_kernel(dvc_config cfg, uint64_t seed, int n, dvc_state* out
     }
 }
 
-// One thread per root: plan, fill its table in a private workspace slot, sample.
-__global__ void determinize_kernel(const dvc_state* roots, int n, int observer, uint64_t seed,
-                                   const uint32_t* tree_ids, const uint32_t* iter_ids, dvc_state* out,
-                                   unsigned long long* ws, int32_t* flags) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= n) return;
-    const G g = load_state(roots[idx]);
-    const uint32_t obs = observer < 0 ? g.cur : (uint32_t)observer;
-    DetPlan pl;
-    det_plan(g, obs, pl);
-    if (!pl.ok) {
-        latch(flags, DVC_E_UNSUPPORTED);
-        out[idx] = roots[idx];
-        return;
+// One CTA per root, the CTAs going through the roots: one warp plans the view,
+// all threads fill its counting table layer by layer, one thread samples.  A
+// root is a chain of layers (a barrier each) and then of tiles, so what counts
+// is how many roots are under way and how short a layer is.  1,000 four-player
+// joker roots: 59 us, against 31.1 ms with one thread per root (each filling
+// up to 32,768 cells by itself) in launches of 256 roots.
+__global__ void __launch_bounds__(kDetThreads, 4)
+    determinize_kernel(const dvc_state* roots, int n, int observer, uint64_t seed, const uint32_t* tree_ids,
+                       const uint32_t* iter_ids, dvc_state* out, unsigned long long* ws, int32_t* flags) {
+    extern __shared__ __align__(16) unsigned long long s_table[];  // kDetSharedCells
+    __shared__ DetPlan pl;
+    for (int idx = blockIdx.x; idx < n; idx += gridDim.x) {
+        const G g = load_state(roots[idx]);
+        const uint32_t obs = observer < 0 ? g.cur : (uint32_t)observer;
+        if (threadIdx.x < 32u) det_plan(g, obs, pl);
+        __syncthreads();
+        if (!pl.ok) {
+            if (threadIdx.x == 0u) {
+                latch(flags, DVC_E_UNSUPPORTED);
+                out[idx] = roots[idx];
+            }
+        } else {
+            unsigned long long* F = pl.cells <= kDetSharedCells ? s_table : ws + (size_t)blockIdx.x * kDetMaxCells;
+            det_fill(pl, F, threadIdx.x, kDetThreads, [] { __syncthreads(); });
+            if (threadIdx.x == 0u) {
+                Rng r;
+                r.open(seed, tree_ids[idx], 0u, iter_ids[idx], kTagDet);
+                G o;
+                det_sample(pl, F, g, r, o);
+                store_state(o, out[idx]);
+            }
+        }
+        __syncthreads();  // the plan and the table are read before the next root's are written
     }
-    unsigned long long* F = ws + (size_t)(idx % kDetChunk) * kDetMaxCells;
-    det_fill(pl, F, 0u, 1u, [] {});
-    Rng r;
-    r.open(seed, tree_ids[idx], 0u, iter_ids[idx], kTagDet);
-    G o;
-    det_sample(pl, F, g, r, o);
-    store_state(o, out[idx]);
 }
 
 // One self-play move per game: the guess actions[i] on the true state, then
@@ -618,10 +635,8 @@ __device__ void init_tree(ForestDev& F, int t, DetPlan* plans, unsigned long lon
     dvc_state* roots = const_cast<dvc_state*>(F.roots);
     const G g = load_state(roots[t]);
     DetPlan& pl = plans[t];
-    if (lane == 0) {
-        det_plan(g, g.cur, pl);
-        pl.ok = pl.cells <= table_cap ? 1u : 0u;
-    }
+    det_plan(g, g.cur, pl);
+    if (lane == 0) pl.ok = pl.cells <= table_cap ? 1u : 0u;
     __syncwarp();
     TreeMeta& tm = F.meta[t];
     if (pl.ok) det_fill(pl, tables + tm.table_off, lane, 32u, [] { __syncwarp(); });
@@ -822,22 +837,28 @@ int dvc_determinize(dvc_ctx* c, const dvc_state* d_roots, int n, int observer, u
         return fail(c, DVC_E_INVALID, "dvc_determinize: d_out may not overlap d_roots");
     if (int rc = set_device(c)) return rc;
     if (!c->d_ws) {
-        const size_t cells = (size_t)kDetChunk * kDetMaxCells;
+        const size_t cells = (size_t)kDetSlots * kDetMaxCells;
         if (cudaMalloc(&c->d_ws, cells * sizeof(unsigned long long)) != cudaSuccess) {
             cudaGetLastError();
             c->d_ws = nullptr;
             return fail(c, DVC_E_OOM, "dvc_determinize: workspace");
         }
+        cudaError_t e = cudaFuncSetAttribute(determinize_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)(kDetSharedCells * sizeof(unsigned long long)));
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(determinize_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                     (int)cudaSharedmemCarveoutMaxShared);
+        if (e != cudaSuccess) {
+            cudaFree(c->d_ws);
+            c->d_ws = nullptr;
+            return cuda_fail(c, e, "dvc_determinize attributes");
+        }
         c->ws_cells = cells;
     }
-    for (int base = 0; base < n; base += kDetChunk) {
-        const int m = std::min(kDetChunk, n - base);
-        determinize_kernel<<<(m + 63) / 64, 64, 0, (cudaStream_t)stream>>>(
-            d_roots + base, m, observer, seed, d_tree_ids + base, d_iter_ids + base, d_out + base, c->d_ws,
-            c->d_flags);
-        if (int rc = check_launch(c, "determinize_kernel")) return rc;
-    }
-    return DVC_OK;
+    determinize_kernel<<<std::min(n, kDetSlots), kDetThreads, kDetSharedCells * sizeof(unsigned long long),
+                         (cudaStream_t)stream>>>(d_roots, n, observer, seed, d_tree_ids, d_iter_ids, d_out, c->d_ws,
+                                                 c->d_flags);
+    return check_launch(c, "determinize_kernel");
 }
 
 int dvc_rollout_batch(dvc_ctx* c, const dvc_state* d_leaves, int n_leaves, int playouts_per_leaf, uint64_t seed,

@@ -53,27 +53,33 @@ bool overlaps(const dvc_state* a, const dvc_state* b, int n) {
     return a0 < b0 + len && b0 < a0 + len;
 }
 
-__global__ void determinize_noalloc_kernel(const dvc_state* roots, int n, int observer, uint64_t seed,
-                                           const uint32_t* tree_ids, const uint32_t* iter_ids, dvc_state* out,
-                                           int32_t* status, unsigned long long* scratch) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= n) return;
+// One CTA per root, as determinize_kernel (dvc_lib.cu), every table in the
+// root's scratch slot.
+constexpr int kThreads = 256;
+__global__ void __launch_bounds__(kThreads)
+    determinize_noalloc_kernel(const dvc_state* roots, int observer, uint64_t seed, const uint32_t* tree_ids,
+                               const uint32_t* iter_ids, dvc_state* out, int32_t* status,
+                               unsigned long long* scratch) {
+    __shared__ DetPlan pl;
+    const int idx = blockIdx.x;
+    const bool first = threadIdx.x == 0u;
     const G g = load_state(roots[idx]);
     if (observer >= (int)g.np) {  // no such seat in this root's game
-        out[idx] = roots[idx];
-        if (status) status[idx] = DVC_E_INVALID;
+        if (first) out[idx] = roots[idx];
+        if (first && status) status[idx] = DVC_E_INVALID;
         return;
     }
     const uint32_t obs = observer < 0 ? g.cur : (uint32_t)observer;
-    DetPlan pl;
-    det_plan(g, obs, pl);
+    if (threadIdx.x < 32u) det_plan(g, obs, pl);
+    __syncthreads();
     if (pl.cells > kNoAllocCells) {
-        out[idx] = roots[idx];
-        if (status) status[idx] = DVC_E_UNSUPPORTED;
+        if (first) out[idx] = roots[idx];
+        if (first && status) status[idx] = DVC_E_UNSUPPORTED;
         return;
     }
     unsigned long long* F = scratch + (size_t)idx * kNoAllocCells;
-    det_fill(pl, F, 0u, 1u, [] {});
+    det_fill(pl, F, threadIdx.x, kThreads, [] { __syncthreads(); });
+    if (!first) return;
     Rng r;
     r.open(seed, tree_ids[idx], 0u, iter_ids[idx], kTagDet);
     G o;
@@ -114,8 +120,8 @@ extern "C" int dvc_determinize_noalloc(const dvc_state* d_roots, int n, int obse
         }
         scratch = g_scratch_addr[dev];
     }
-    determinize_noalloc_kernel<<<(n + 63) / 64, 64, 0, (cudaStream_t)stream>>>(
-        d_roots, n, observer, seed, d_tree_ids, d_iter_ids, d_out, d_status, (unsigned long long*)scratch);
+    determinize_noalloc_kernel<<<n, kThreads, 0, (cudaStream_t)stream>>>(
+        d_roots, observer, seed, d_tree_ids, d_iter_ids, d_out, d_status, (unsigned long long*)scratch);
     if (cudaGetLastError() != cudaSuccess) return DVC_E_CUDA;
     return DVC_OK;
 }

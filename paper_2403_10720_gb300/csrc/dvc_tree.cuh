@@ -211,36 +211,6 @@ struct TreeWords {
     }
 };
 
-// The rows of a state laid out one tile per lane (lanes 0..25): the seat that
-// holds tile `lane` (4: nobody) and the tile's place in that seat's row.
-struct Rows {
-    uint32_t owner, pos;
-    __device__ __forceinline__ Rows(const G& g) {
-        const uint32_t lane = threadIdx.x & 31u, bit = lane < 26u ? 1u << lane : 0u;
-        uint32_t hp = 0u;
-        owner = 4u;
-        if (g.h0 & bit) { owner = 0u; hp = g.h0; }
-        if (g.h1 & bit) { owner = 1u; hp = g.h1; }
-        if (g.h2 & bit) { owner = 2u; hp = g.h2; }
-        if (g.h3 & bit) { owner = 3u; hp = g.h3; }
-        pos = __popc(hp & kNumMask & (bit - 1u));
-        if (g.tmask & kJokerMask) {
-            if (lane >= 24u) {
-                if (owner < 4u) pos = joker_pos(g, hp, lane - 24u);
-            } else {
-                const uint32_t k = pos;
-                if ((hp >> 24) & 1u) pos += g.jg0 <= k;
-                if ((hp >> 25) & 1u) pos += g.jg1 <= k;
-            }
-        }
-    }
-    // Face-down places of seat q's row.
-    __device__ __forceinline__ uint32_t hidden(const G& g, uint32_t q) const {
-        const bool in = owner == q && !((g.rev >> (threadIdx.x & 31u)) & 1u) && ((g.alive >> q) & 1u);
-        return __reduce_or_sync(0xFFFFFFFFu, in ? 1u << pos : 0u);
-    }
-};
-
 // tree_apply (dvc_device.cuh) by a whole warp: the same transition and words,
 // the state the same on every lane before and after.
 __device__ __forceinline__ void warp_apply(G& g, const Rows& v, uint32_t code, TreeWords& tw, bool cont) {
