@@ -41,6 +41,20 @@ __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t saddr) {
     return d;
 }
 
+// The same for an MN-major tile (K rows of 64 elements along M or N, 128 bytes
+// each, 128-byte swizzle): the stride-dimension offset is that between groups
+// of eight K rows (1024 bytes), the leading-dimension offset that between
+// 64-element columns of the tile (`chunk` bytes).
+__device__ __forceinline__ uint64_t smem_desc_mn128(uint32_t saddr, uint32_t chunk) {
+    uint64_t d = 0;
+    d |= (uint64_t)((saddr >> 4) & 0x3FFFu);
+    d |= (uint64_t)((chunk >> 4) & 0x3FFFu) << 16;
+    d |= (uint64_t)(1024u >> 4) << 32;
+    d |= (uint64_t)1u << 46;
+    d |= (uint64_t)2u << 61;
+    return d;
+}
+
 // The same for a K-major tile without swizzle: core matrices of 8 rows x 16
 // bytes; lbo = bytes between the two 8-element halves of a 16-wide K slice,
 // sbo = bytes between 8-row groups; swizzle mode 0.
@@ -54,9 +68,11 @@ __device__ __forceinline__ uint64_t smem_desc_noswz(uint32_t saddr, uint32_t lbo
 }
 
 // Instruction descriptor for kind::f16: D FP32 (bits 4-5 = 1), A and B BF16
-// (bits 7-9 = 1, 10-12 = 1), both K-major, N >> 3 in bits 17-22, M >> 4 in 24-28.
-__host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N) {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+// (bits 7-9 = 1, 10-12 = 1), A and B K-major (bits 15, 16: 1 = MN-major), N >> 3
+// in bits 17-22, M >> 4 in 24-28.
+__host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N, bool a_mn = false, bool b_mn = false) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | (a_mn ? 1u << 15 : 0u) | (b_mn ? 1u << 16 : 0u) |
+           ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
@@ -171,6 +187,30 @@ __device__ __forceinline__ float gelu(float x) {
     return 0.5f * x * (1.0f + tanh_hw(0.79788456080286536f * (x + 0.044715f * x * x * x)));
 }
 
+// Derivative of the tanh-form GELU: with u = k (z + a z^3), t = tanh(u):
+// 0.5 (1 + t) + 0.5 z (1 - t^2) k (1 + 3 a z^2).
+__device__ __forceinline__ float gelu_grad(float z) {
+    const float k = 0.79788456080286536f, a = 0.044715f;
+    const float t = tanh_hw(k * (z + a * z * z * z));
+    return 0.5f * (1.0f + t) + 0.5f * z * (1.0f - t * t) * k * (1.0f + 3.0f * a * z * z);
+}
+
+// Column sums over a warp's 32 rows of 16 columns (one row per lane): halves of
+// the columns are exchanged and added, 16 shuffles in all; lane 2 c ends with
+// column c in v[0] (and lane 2 c + 1 with the same).
+__device__ __forceinline__ void warp_colsum16(float* v, int lane) {
+#pragma unroll
+    for (int h = 8, o = 16; h >= 1; h >>= 1, o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < h; ++i) {
+            const float give = up ? v[i] : v[i + h], keep = up ? v[i + h] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xFFFFFFFFu, give, o);
+        }
+    }
+    v[0] += __shfl_xor_sync(0xFFFFFFFFu, v[0], 1);
+}
+
 struct GemmArgs {
     const __nv_bfloat16* A;  // M x K
     const __nv_bfloat16* B;  // N x K
@@ -198,6 +238,10 @@ struct GemmArgs {
     // rows x 8 columns are 512 contiguous bytes (one coalesced store).
     int a_blocked;  // A in the K-blocked layout
     int c_blocked;  // C written in the K-blocked layout
+    // Backward epilogue (BACK): C = acc * gelu'(Z) in BF16, and the FP32 products'
+    // column sums over each 32 rows in colsum[(row / 32)][N].
+    const float* Z;  // M x N, pre-activations
+    float* colsum;
 };
 
 // Element (r, c) of a K-blocked matrix with W columns.
@@ -235,7 +279,10 @@ constexpr int kGemmThreads = 32 * (4 + kGemmEpiWarps);  // warp 0 TMA, warp 1 MM
 // BN in {16, 32, 64, 128, 256}.  tA: A as a (K, M) tensor, box (64, 128);
 // tB: B as (K, N), box (64, BN); both 128-byte swizzled.  Grid: at most one
 // CTA per SM; CTA c takes tiles c, c + gridDim.x, ...
-template <int BN>
+// BMN: B is K x N row-major instead (a layer's own weights where the backward
+// pass needs their transpose), tB (N, K), box (64, 64), read MN-major.
+// BACK: the backward epilogue (M a multiple of 32, N of 16).
+template <int BN, bool BMN = false, bool BACK = false>
 __global__ void __launch_bounds__(kGemmThreads, 1)
     gemm_bf16_tc_kernel(const __grid_constant__ CUtensorMap tA, const __grid_constant__ CUtensorMap tB, GemmArgs a) {
     using Cfg = GemmCfg<BN>;
@@ -296,7 +343,13 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
                         bulk_load(sa, a.A + kblocked_index(m0, kc * kGemmBK, a.K), Cfg::kA, &s_full[s]);
                     else
                         tma_load_2d(sa, &tA, kc * kGemmBK, m0, &s_full[s]);
-                    tma_load_2d(sa + Cfg::kA, &tB, kc * kGemmBK, n0, &s_full[s]);
+                    if constexpr (BMN) {
+#pragma unroll
+                        for (int j = 0; j < BN / 64; ++j)
+                            tma_load_2d(sa + Cfg::kA + (uint32_t)j * 8192u, &tB, n0 + 64 * j, kc * kGemmBK, &s_full[s]);
+                    } else {
+                        tma_load_2d(sa + Cfg::kA, &tB, kc * kGemmBK, n0, &s_full[s]);
+                    }
                 }
             }
             s_issued = it;
@@ -305,7 +358,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         if (lane == 0) {
             // MMA issuer: tile j accumulates into buffer j & 1 once the
             // epilogue has drained that buffer's previous tile
-            const uint32_t idesc = idesc_bf16_f32(kGemmBM, BN);
+            const uint32_t idesc = idesc_bf16_f32(kGemmBM, BN, false, BMN);
             int it = 0, j = 0;
             bool stop = false;
             for (int t = blockIdx.x; t < tiles && !stop; t += gridDim.x, ++j) {
@@ -329,7 +382,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
                     for (int kk = 0; kk < kGemmBK / 16; ++kk) {
                         const uint64_t ad = a.a_blocked ? smem_desc_noswz(sa + (uint32_t)kk * 4096u, 2048u, 128u)
                                                         : smem_desc_sw128(sa + (uint32_t)kk * 32u);
-                        const uint64_t bd = smem_desc_sw128(sa + Cfg::kA + (uint32_t)kk * 32u);
+                        const uint64_t bd = BMN ? smem_desc_mn128(sa + Cfg::kA + (uint32_t)kk * 2048u, 8192u)
+                                                : smem_desc_sw128(sa + Cfg::kA + (uint32_t)kk * 32u);
                         tc_mma(acc, ad, bd, idesc, (kc > 0 || kk > 0) ? 1u : 0u);
                     }
                     tc_commit(&s_empty[s]);
@@ -363,6 +417,29 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
 #pragma unroll 1
             for (int c0 = cbeg; c0 < cbeg + cw && c0 < BN; c0 += 16) {  // cw is a multiple of 16
                 float v[16];
+                if constexpr (BACK) {
+                    const int nb = n0 + c0;
+                    float z[16];
+                    if (live) {
+                        const float4* zp = reinterpret_cast<const float4*>(a.Z + (size_t)row * a.N + nb);
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) reinterpret_cast<float4*>(z)[i] = zp[i];
+                    }
+                    tc_ld16(acc + (uint32_t)c0, v);
+                    uint32_t w[8];
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) v[i] = live ? __fmul_rn(v[i], gelu_grad(z[i])) : 0.0f;
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        __nv_bfloat162 p = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
+                        w[i] = *reinterpret_cast<uint32_t*>(&p);
+                    }
+                    if (live) st_global_v8(a.C + (size_t)row * a.N + nb, w);
+                    warp_colsum16(v, lane);
+                    if (!(lane & 1) && m0 + quarter * 32 < a.M)
+                        a.colsum[(size_t)(m0 / 32 + quarter) * a.N + nb + (lane >> 1)] = v[0];
+                    continue;
+                }
                 tc_ld16(acc + (uint32_t)c0, v);
                 if (live) {
                     const int nb = n0 + c0;
@@ -446,6 +523,140 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     if (warp == 0) {
         tc_fence_after();
         tc_dealloc(tmem, Cfg::kCols);
+    }
+}
+
+// Weight gradients of all layers in one launch: per layer dW = dZ^T H over the
+// batch (K = rows), both operands read MN-major straight from the row-major
+// activations.  A layer's 512 x 512 outputs are only 16 tiles of 128 x 128, so
+// the rows are split: CTA (problem, tile, split) leaves the FP32 sums of its rows
+// in part[split], and the optimiser adds the splits in order.  Two CTAs per SM
+// (three 32 KB stages each).  What bounds it is operand traffic from L2.
+// The last problem is the output layer, transposed: D[512][64] = H3^T dZ4, its
+// first four columns written as the 4 x 512 gradient.
+struct DwProblem {
+    int first;        // its first CTA within a split
+    int tiles_n;      // column tiles
+    int cols;         // columns of the gradient (row stride)
+    int boxes_b;      // 64-column boxes of B per tile (2, or 1 for 64 columns)
+    int transposed;   // write D[m][n] to [n][m] for n < 4
+    size_t offset;    // of the gradient in the parameter array
+};
+struct DwArgs {
+    CUtensorMap a[4], b[4];
+    DwProblem p[4];
+    int ctas, splits, nk;  // CTAs per split; 64-row slices of the batch
+    float* part;
+    size_t stride;  // floats between splits
+    int32_t* flags;
+    uint64_t wait_ns;
+};
+constexpr int kDwStages = 3;
+constexpr uint32_t kDwStage = 32768u;
+constexpr uint32_t kDwSmem = kDwStages * kDwStage + 1024u;
+constexpr int kDwThreads = 256;
+
+__global__ void __launch_bounds__(kDwThreads, 2) gemm_dw_kernel(const __grid_constant__ DwArgs a) {
+    extern __shared__ __align__(1024) unsigned char gsm[];
+    __shared__ uint64_t s_full[kDwStages], s_empty[kDwStages], s_acc;
+    __shared__ uint32_t s_tmem;
+    __shared__ int s_fail, s_issued, s_consumed;
+    volatile int* fail = &s_fail;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int split = (int)blockIdx.x / a.ctas, cta = (int)blockIdx.x % a.ctas;
+    int q = 0;
+    while (q < 3 && cta >= a.p[q + 1].first) ++q;
+    const DwProblem pr = a.p[q];
+    const int tile = cta - pr.first, m0 = tile / pr.tiles_n * 128, n0 = tile % pr.tiles_n * 128;
+    const int k0 = (int)((long long)a.nk * split / a.splits), k1 = (int)((long long)a.nk * (split + 1) / a.splits);
+    const int nk = k1 - k0;  // at least 1: splits <= nk
+    const uint32_t base = (smem_u32(gsm) + 1023u) & ~1023u;
+    if (tid == 0) {
+        for (int s = 0; s < kDwStages; ++s) {
+            mbar_init(&s_full[s], 1);
+            mbar_init(&s_empty[s], 1);
+        }
+        mbar_init(&s_acc, 1);
+        s_fail = s_issued = s_consumed = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) tc_alloc(&s_tmem, 128u);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = s_tmem;
+    const uint32_t bytes = 16384u + 8192u * (uint32_t)pr.boxes_b;
+    if (warp == 0 && lane == 0) {
+        int it = 0;
+        for (; it < nk; ++it) {
+            const int s = it % kDwStages, r = it / kDwStages;
+            if ((it >= kDwStages && !mbar_wait(&s_empty[s], (uint32_t)(r - 1) & 1u, a.wait_ns)) || *fail) {
+                *fail = 1;
+                break;
+            }
+            const uint32_t sa = base + (uint32_t)s * kDwStage;
+            mbar_expect_tx(&s_full[s], bytes);
+            for (int j = 0; j < 2; ++j)
+                tma_load_2d(sa + (uint32_t)j * 8192u, &a.a[q], m0 + 64 * j, (k0 + it) * 64, &s_full[s]);
+            for (int j = 0; j < pr.boxes_b; ++j)
+                tma_load_2d(sa + 16384u + (uint32_t)j * 8192u, &a.b[q], n0 + 64 * j, (k0 + it) * 64, &s_full[s]);
+        }
+        s_issued = it;
+    }
+    if (warp == 1 && lane == 0) {
+        const uint32_t idesc = idesc_bf16_f32(128, 64 * pr.boxes_b, true, true);
+        int it = 0;
+        for (; it < nk; ++it) {
+            const int s = it % kDwStages;
+            if (!mbar_wait(&s_full[s], (uint32_t)(it / kDwStages) & 1u, a.wait_ns) || *fail) {
+                *fail = 1;
+                break;
+            }
+            tc_fence_after();
+            const uint32_t sa = base + (uint32_t)s * kDwStage;
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk)
+                tc_mma(tmem, smem_desc_mn128(sa + (uint32_t)kk * 2048u, 8192u),
+                       smem_desc_mn128(sa + 16384u + (uint32_t)kk * 2048u, 8192u), idesc, (it > 0 || kk > 0) ? 1u : 0u);
+            tc_commit(&s_empty[s]);
+        }
+        s_consumed = it;
+        tc_commit(&s_acc);  // arrives when every MMA issued above has completed
+    }
+    __syncthreads();
+    const bool ok = __syncthreads_and(mbar_wait(&s_acc, 0, a.wait_ns) && !*fail) != 0;
+    if (ok) {
+        tc_fence_after();
+        const int quarter = warp & 3, half = warp >> 2;
+        const uint32_t acc = tmem + ((uint32_t)(quarter * 32) << 16);
+        const int row = m0 + quarter * 32 + lane;
+        float* out = a.part + (size_t)split * a.stride + pr.offset;
+        if (pr.transposed) {
+            float v[16];
+            tc_ld16(acc, v);
+            if (half == 0)
+                for (int o = 0; o < 4; ++o) out[(size_t)o * 512 + row] = v[o];
+        } else {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                float v[16];
+                const int col = half * 64 + c * 16;
+                tc_ld16(acc + (uint32_t)col, v);
+                float* o = out + (size_t)row * pr.cols + n0 + col;
+                st_global_v8(o, reinterpret_cast<const uint32_t*>(v));
+                st_global_v8(o + 8, reinterpret_cast<const uint32_t*>(v + 8));
+            }
+        }
+    } else if (tid == 0) {  // the copies still in flight land before the block ends
+        for (int it = s_consumed; it < s_issued; ++it)
+            mbar_wait(&s_full[it % kDwStages], (uint32_t)(it / kDwStages) & 1u, a.wait_ns);
+        if (a.flags) atomicCAS(a.flags, 0, -4);  // DVC_E_TIMEOUT
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0) {
+        tc_fence_after();
+        tc_dealloc(tmem, 128u);
     }
 }
 

@@ -33,17 +33,23 @@ constexpr int kLogitFloats = kHeadParts * 4 > VO ? kHeadParts * 4 : VO;
 constexpr size_t OFF_W1 = 0, OFF_B1 = OFF_W1 + (size_t)VH * VF, OFF_W2 = OFF_B1 + VH, OFF_B2 = OFF_W2 + (size_t)VH * VH,
                  OFF_W3 = OFF_B2 + VH, OFF_B3 = OFF_W3 + (size_t)VH * VH, OFF_W4 = OFF_B3 + VH,
                  OFF_B4 = OFF_W4 + 4 * VH, NPARAM = OFF_B4 + 4;
+// row splits of the weight gradients (280 CTAs at two per SM: one wave), and
+// floats from one split to the next (32-byte aligned)
+constexpr int kDwSplits = 5;
+constexpr size_t kDwStride = (NPARAM + 7) / 8 * 8;
 
 }  // namespace
 
 struct dvc_value_net {
     float *master, *m, *v, *grad;
-    __nv_bfloat16 *W1, *W2, *W3, *W4;  // W4: 16 x 512, rows 4.. zero
-    __nv_bfloat16 *W2T, *W3T, *W4T;    // W4T: 512 x 64, columns 4.. zero
+    __nv_bfloat16 *W1, *W2, *W3, *W4;  // W4: 64 x 512, rows 4.. zero
     float* b4p;                        // 16
     int cap;                           // workspace rows (multiple of 128)
-    __nv_bfloat16 *X, *H1, *H2, *H3, *XT, *H1T, *H2T, *H3T, *dZ, *dZT, *dZ4, *dZ4T;
-    float *Z1, *Z2, *Z3, *L, *dH, *dZ4f, *tmp, *part, *loss;
+    __nv_bfloat16 *X, *H1, *H2, *H3, *dZ[3], *dZ4;  // dZ of layers 1..3; of the output layer, 64 columns
+    float *Z1, *Z2, *Z3, *L;
+    float* colsum;                     // bias gradients of layers 1..3 by 32 rows: 3 x (rows / 32) x 512
+    float* rowpart;                    // per CTA of the loss kernel: loss, four output-bias gradients, padding (8)
+    float* dwpart;                     // weight gradients by row split: kDwSplits x kDwStride
     long long step;
 };
 
@@ -220,151 +226,170 @@ __global__ void softmax_head_kernel(const float* parts, const float* b4, const d
 }
 
 // Cross-entropy against soft labels (absolute seats) and dL/dlogits / n.
-// Rows >= n get zero gradient.  dZ4 (npad x 64, BF16, K-padded), dZ4T (16 x
-// npad, BF16), dZ4f (npad x 16, FP32); per-row loss into rowloss.
-__global__ void loss_grad_kernel(const float* L, const dvc_state* states, const float* labels, int n, int npad,
-                                 __nv_bfloat16* dZ4, __nv_bfloat16* dZ4T, float* dZ4f, float* rowloss) {
-    const int row = blockIdx.x * blockDim.x + threadIdx.x;
-    if (row >= npad) return;
-    float d[VO];
-    for (int r = 0; r < VO; ++r) d[r] = 0.0f;
+// Rows >= n get zero gradient.  dZ4 (npad x 64, BF16, K-padded); per CTA the
+// sums of the losses and of the FP32 logit gradients in rowpart[cta][0..4].
+constexpr int kLossThreads = 128;
+__global__ void __launch_bounds__(kLossThreads)
+    loss_grad_kernel(const float* L, const dvc_state* states, const float* labels, int n, int npad,
+                     __nv_bfloat16* dZ4, float* rowpart) {
+    __shared__ float s_sum[kLossThreads / 32][5];
+    const int row = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float d[4] = {0.0f, 0.0f, 0.0f, 0.0f};
     float loss = 0.0f;
     if (row < n) {
         const dvc_state& s = states[row];
         const int P = (s.nplayers >= 2 && s.nplayers <= 4) ? s.nplayers : 2;
         const int cur = s.cur < P ? s.cur : 0;
-        const float* z = L + (size_t)row * VO;
+        const float4 zv = *reinterpret_cast<const float4*>(L + (size_t)row * VO);
+        const float z[4] = {zv.x, zv.y, zv.z, zv.w};
         float mx = z[0];
-        for (int r = 1; r < P; ++r) mx = fmaxf(mx, z[r]);
+#pragma unroll
+        for (int r = 1; r < 4; ++r)
+            if (r < P) mx = fmaxf(mx, z[r]);
         float sum = 0.0f;
-        for (int r = 0; r < P; ++r) sum += expf(z[r] - mx);
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+            if (r < P) sum += expf(z[r] - mx);
         const float lse = mx + logf(sum);
-        for (int r = 0; r < P; ++r) {
-            const float y = labels[(size_t)row * 4 + (cur + r) % P];
-            const float p = expf(z[r] - lse);
-            if (y > 0.0f) loss -= y * (z[r] - lse);
-            d[r] = (p - y) / (float)n;
-        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+            if (r < P) {
+                const float y = labels[(size_t)row * 4 + (cur + r) % P];
+                const float p = expf(z[r] - lse);
+                if (y > 0.0f) loss -= y * (z[r] - lse);
+                d[r] = (p - y) / (float)n;
+            }
     }
-    rowloss[row] = loss;
-    for (int r = 0; r < 64; ++r) dZ4[(size_t)row * 64 + r] = __float2bfloat16_rn(r < VO ? d[r] : 0.0f);
-    for (int r = 0; r < VO; ++r) {
-        dZ4T[(size_t)r * npad + row] = __float2bfloat16_rn(d[r]);
-        dZ4f[(size_t)row * VO + r] = d[r];
+    if (row < npad) {
+        uint4* out = reinterpret_cast<uint4*>(dZ4 + (size_t)row * 64);
+        const __nv_bfloat162 lo = __floats2bfloat162_rn(d[0], d[1]), hi = __floats2bfloat162_rn(d[2], d[3]);
+        out[0] = make_uint4(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi), 0u, 0u);
+#pragma unroll
+        for (int j = 1; j < 8; ++j) out[j] = make_uint4(0u, 0u, 0u, 0u);
     }
-}
-
-// out[c][r] = in[r][c] for an R x C BF16 matrix (R, C multiples of 32).
-__global__ void transpose_bf16_kernel(const __nv_bfloat16* in, __nv_bfloat16* out, int R, int C) {
-    __shared__ __nv_bfloat16 tile[32][33];
-    const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
-    for (int i = threadIdx.y; i < 32; i += blockDim.y) tile[i][threadIdx.x] = in[(size_t)(r0 + i) * C + c0 + threadIdx.x];
+    float v[5] = {loss, d[0], d[1], d[2], d[3]};
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xFFFFFFFFu, v[k], o);
+        if (lane == 0) s_sum[warp][k] = v[k];
+    }
     __syncthreads();
-    for (int i = threadIdx.y; i < 32; i += blockDim.y)
-        out[(size_t)(c0 + i) * R + r0 + threadIdx.x] = tile[threadIdx.x][i];
-}
-
-// Derivative of the tanh-form GELU (dvc_gemm.cuh): with u = k (z + a z^3),
-// t = tanh(u): 0.5 (1 + t) + 0.5 z (1 - t^2) k (1 + 3 a z^2).
-__device__ __forceinline__ float gelu_grad(float z) {
-    const float k = 0.79788456080286536f, a = 0.044715f;
-    const float t = tanh_hw(k * (z + a * z * z * z));
-    return 0.5f * (1.0f + t) + 0.5f * z * (1.0f - t * t) * k * (1.0f + 3.0f * a * z * z);
-}
-
-// dZ = dH * GELU'(Z): FP32 in place in dH, BF16 copy in dZ.
-__global__ void gelu_back_kernel(float* dH, const float* Z, __nv_bfloat16* dZ, size_t count) {
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (size_t)gridDim.x * blockDim.x) {
-        const float v = dH[i] * gelu_grad(Z[i]);
-        dH[i] = v;
-        dZ[i] = __float2bfloat16_rn(v);
+    if (threadIdx.x < 5) {
+        float acc = 0.0f;
+        for (int w = 0; w < kLossThreads / 32; ++w) acc += s_sum[w][threadIdx.x];
+        rowpart[(size_t)blockIdx.x * 8 + threadIdx.x] = acc;
     }
 }
 
-// Column sums of an R x C FP32 matrix in a fixed order: partial sums over
-// row blocks of 256, then one thread per column adds the blocks in order.
-__global__ void colsum_partial_kernel(const float* A, int R, int C, float* part) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    const int rb = blockIdx.y;
-    if (c >= C) return;
-    float acc = 0.0f;
-    const int r1 = min(R, (rb + 1) * 256);
-    for (int r = rb * 256; r < r1; ++r) acc += A[(size_t)r * C + c];
-    part[(size_t)rb * C + c] = acc;
+// AdamW on one FP32 master parameter (weight decay on weight matrices only).
+struct AdamCoef {
+    float lr, b1, b2, eps, wd, c1, c2;
+};
+__device__ __forceinline__ float adamw_one(float w, float& m, float& v, float gi, bool is_bias, const AdamCoef& a) {
+    const float mi = a.b1 * m + (1.0f - a.b1) * gi;
+    const float vi = a.b2 * v + (1.0f - a.b2) * gi * gi;
+    m = mi;
+    v = vi;
+    float upd = (mi / a.c1) / (sqrtf(vi / a.c2) + a.eps);
+    if (!is_bias) upd += a.wd * w;
+    return w - a.lr * upd;
 }
 
-__global__ void colsum_final_kernel(const float* part, int nb, int C, float* out, int cols_out) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= cols_out) return;
-    float acc = 0.0f;
-    for (int b = 0; b < nb; ++b) acc += part[(size_t)b * C + c];
-    out[c] = acc;
+__device__ __forceinline__ bool is_bias_index(size_t i) {
+    return (i >= OFF_B1 && i < OFF_W2) || (i >= OFF_B2 && i < OFF_W3) || (i >= OFF_B3 && i < OFF_W4) || i >= OFF_B4;
 }
 
-__global__ void mean_kernel(const float* x, int n, float* out) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    float acc = 0.0f;
-    for (int i = 0; i < n; ++i) acc += x[i];
-    *out = acc / (float)n;
+// The BF16 working copy of master weights i .. i + 3 (no biases).
+__device__ __forceinline__ void store_bf16_weights(const dvc_value_net& v, size_t i, float4 w) {
+    __nv_bfloat16* dst = i < OFF_B1 ? v.W1 + i : i < OFF_B2 ? v.W2 + (i - OFF_W2) : i < OFF_B3 ? v.W3 + (i - OFF_W3)
+                                                                                            : v.W4 + (i - OFF_W4);
+    const __nv_bfloat162 lo = __floats2bfloat162_rn(w.x, w.y), hi = __floats2bfloat162_rn(w.z, w.w);
+    *reinterpret_cast<uint2*>(dst) =
+        make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
 }
 
-__global__ void copy_rows_kernel(const float* src, float* dst, size_t count) {
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (size_t)gridDim.x * blockDim.x)
-        dst[i] = src[i];
-}
-
-// AdamW on the FP32 master copy; weight decay on weight matrices only.
-__global__ void adamw_kernel(float* w, float* m, float* v, const float* g, size_t count, float lr, float b1, float b2,
-                             float eps, float wd, float c1, float c2) {
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (size_t)gridDim.x * blockDim.x) {
-        const bool is_bias = (i >= OFF_B1 && i < OFF_W2) || (i >= OFF_B2 && i < OFF_W3) ||
-                             (i >= OFF_B3 && i < OFF_W4) || i >= OFF_B4;
-        const float gi = g[i];
-        const float mi = b1 * m[i] + (1.0f - b1) * gi;
-        const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
-        m[i] = mi;
-        v[i] = vi;
-        float upd = (mi / c1) / (sqrtf(vi / c2) + eps);
-        if (!is_bias) upd += wd * w[i];
-        w[i] -= lr * upd;
-    }
-}
-
-// BF16 working copies (and transposes) of the master weights.
-__global__ void refresh_kernel(const float* w, __nv_bfloat16* W1, __nv_bfloat16* W2, __nv_bfloat16* W3,
-                               __nv_bfloat16* W4, __nv_bfloat16* W2T, __nv_bfloat16* W3T, __nv_bfloat16* W4T,
-                               float* b4p) {
-    const size_t total = (size_t)VH * VF + 2 * (size_t)VH * VH + (size_t)VO * VH;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        if (i < (size_t)VH * VF) {
-            W1[i] = __float2bfloat16_rn(w[OFF_W1 + i]);
-            continue;
+// End of a training step in one launch: sum the partial gradients (weights over
+// the row splits, biases over the 32-row column sums, output biases and loss
+// over the loss kernel's CTAs, all in a fixed order), AdamW, BF16 copies.
+// CTAs 0 .. kAdamMain-1 take four weights per thread; then 16 CTAs per hidden
+// layer take 32 biases each, and the last one the output biases and the loss.
+// What bounds it is memory: gradient partials, master, moments and their updates.
+constexpr int kAdamThreads = 256;
+constexpr int kAdamMain = (int)((NPARAM / 4 + kAdamThreads - 1) / kAdamThreads);
+constexpr int kAdamGrid = kAdamMain + 3 * (VH / 32) + 1;
+__global__ void __launch_bounds__(kAdamThreads)
+    adamw_kernel(dvc_value_net v, int splits, int row_blocks, int loss_ctas, int n, AdamCoef a, float* loss_out) {
+    const int tid = threadIdx.x;
+    if ((int)blockIdx.x < kAdamMain) {
+        const size_t i = ((size_t)blockIdx.x * kAdamThreads + tid) * 4;
+        if (i >= NPARAM || is_bias_index(i)) return;  // tensors begin at multiples of four
+        float4 g = *reinterpret_cast<const float4*>(v.dwpart + i);
+        for (int s = 1; s < splits; ++s) {
+            const float4 x = *reinterpret_cast<const float4*>(v.dwpart + (size_t)s * kDwStride + i);
+            g.x += x.x;
+            g.y += x.y;
+            g.z += x.z;
+            g.w += x.w;
         }
-        size_t j = i - (size_t)VH * VF;
-        if (j < (size_t)VH * VH) {
-            const __nv_bfloat16 b = __float2bfloat16_rn(w[OFF_W2 + j]);
-            W2[j] = b;
-            W2T[(j % VH) * VH + j / VH] = b;
-            continue;
-        }
-        j -= (size_t)VH * VH;
-        if (j < (size_t)VH * VH) {
-            const __nv_bfloat16 b = __float2bfloat16_rn(w[OFF_W3 + j]);
-            W3[j] = b;
-            W3T[(j % VH) * VH + j / VH] = b;
-            continue;
-        }
-        j -= (size_t)VH * VH;  // W4 padded: 16 x 512
-        const size_t r = j / VH, c = j % VH;
-        const __nv_bfloat16 b = __float2bfloat16_rn(r < 4 ? w[OFF_W4 + r * VH + c] : 0.0f);
-        W4[j] = b;
+        float4 w = *reinterpret_cast<const float4*>(v.master + i), m = *reinterpret_cast<const float4*>(v.m + i);
+        float4 u = *reinterpret_cast<const float4*>(v.v + i);
+        w.x = adamw_one(w.x, m.x, u.x, g.x, false, a);
+        w.y = adamw_one(w.y, m.y, u.y, g.y, false, a);
+        w.z = adamw_one(w.z, m.z, u.z, g.z, false, a);
+        w.w = adamw_one(w.w, m.w, u.w, g.w, false, a);
+        *reinterpret_cast<float4*>(v.grad + i) = g;
+        *reinterpret_cast<float4*>(v.master + i) = w;
+        *reinterpret_cast<float4*>(v.m + i) = m;
+        *reinterpret_cast<float4*>(v.v + i) = u;
+        store_bf16_weights(v, i, w);
+        return;
     }
-    // W4T: 512 x 64 (K-padded), b4 padded
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < (size_t)VH * 64; i += (size_t)gridDim.x * blockDim.x) {
-        const size_t k = i / 64, r = i % 64;
-        W4T[i] = __float2bfloat16_rn(r < 4 ? w[OFF_W4 + r * VH + k] : 0.0f);
+    __shared__ float s_part[kAdamThreads];
+    const int e = (int)blockIdx.x - kAdamMain;
+    size_t i = 0;
+    float acc = 0.0f;
+    bool mine = false;
+    if (e < 3 * (VH / 32)) {
+        const int layer = e / (VH / 32), col = e % (VH / 32) * 32 + (tid & 31);
+        const float* p = v.colsum + (size_t)layer * row_blocks * VH + col;
+        for (int r = tid >> 5; r < row_blocks; r += kAdamThreads / 32) acc += p[(size_t)r * VH];
+        s_part[tid] = acc;
+        __syncthreads();
+        acc = 0.0f;
+        for (int w = 0; w < kAdamThreads / 32; ++w) acc += s_part[w * 32 + (tid & 31)];
+        i = (layer == 0 ? OFF_B1 : layer == 1 ? OFF_B2 : OFF_B3) + (size_t)col;
+        mine = tid < 32;
+    } else {
+        const int k = tid & 7;  // 0: loss, 1..4: output biases
+        if (k < 5)
+            for (int r = tid >> 3; r < loss_ctas; r += kAdamThreads / 8) acc += v.rowpart[(size_t)r * 8 + k];
+        s_part[tid] = acc;
+        __syncthreads();
+        acc = 0.0f;
+        for (int w = 0; w < kAdamThreads / 8; ++w) acc += s_part[w * 8 + k];
+        if (tid == 0 && loss_out) *loss_out = acc / (float)n;
+        i = OFF_B4 + (size_t)(k - 1);
+        mine = tid >= 1 && tid < 5;
     }
-    if (blockIdx.x == 0 && threadIdx.x < VO) b4p[threadIdx.x] = threadIdx.x < 4 ? w[OFF_B4 + threadIdx.x] : 0.0f;
+    if (!mine) return;
+    float m = v.m[i], u = v.v[i];
+    const float w = adamw_one(v.master[i], m, u, acc, true, a);
+    v.grad[i] = acc;
+    v.master[i] = w;
+    v.m[i] = m;
+    v.v[i] = u;
+    if (i >= OFF_B4) v.b4p[i - OFF_B4] = w;
+}
+
+// BF16 working copies of the master weights, zero padding included.
+__global__ void refresh_kernel(dvc_value_net v) {
+    const size_t nthr = (size_t)gridDim.x * blockDim.x, t0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    for (size_t q = t0; q < NPARAM / 4; q += nthr)
+        if (!is_bias_index(4 * q))
+            store_bf16_weights(v, 4 * q, *reinterpret_cast<const float4*>(v.master + 4 * q));
+    for (size_t j = 4 * VH + t0; j < 64 * (size_t)VH; j += nthr) v.W4[j] = __float2bfloat16_rn(0.0f);
+    if (t0 < VO) v.b4p[t0] = t0 < 4 ? v.master[OFF_B4 + t0] : 0.0f;
 }
 
 // Glorot-uniform weights from Philox (key = seed, counter = index), zero biases.
@@ -390,9 +415,9 @@ __global__ void init_params_kernel(float* w, uint64_t seed) {
 
 // ------------------------------------------------------------------ host helpers
 
-template <int BN>
+template <int BN, bool BMN = false, bool BACK = false>
 cudaError_t gemm_attributes() {
-    return cudaFuncSetAttribute(gemm_bf16_tc_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    return cudaFuncSetAttribute(gemm_bf16_tc_kernel<BN, BMN, BACK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)GemmCfg<BN>::kSmem);
 }
 
@@ -415,6 +440,7 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
 
 // A row-major rows x K BF16 matrix as the 2-D tensor (K, rows) read in boxes
 // of 64 x box_rows with the 128-byte swizzle; rows past the end read as zero.
+// (For an operand read MN-major, "K" is its M or N and the rows are K.)
 bool encode_kmajor(CUtensorMap* m, const __nv_bfloat16* p, int rows, int K, int box_rows) {
     const PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
     if (!enc) return false;
@@ -427,22 +453,23 @@ bool encode_kmajor(CUtensorMap* m, const __nv_bfloat16* p, int rows, int K, int 
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int BN>
+template <int BN, bool BMN = false, bool BACK = false>
 cudaError_t launch_gemm(const GemmArgs& a, cudaStream_t st) {
     // inside a stream capture the attributes were set beforehand (dvc_value_prepare)
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     cudaError_t e = cudaStreamIsCapturing(st, &cs);
-    if (e == cudaSuccess && cs == cudaStreamCaptureStatusNone) e = gemm_attributes<BN>();
+    if (e == cudaSuccess && cs == cudaStreamCaptureStatusNone) e = gemm_attributes<BN, BMN, BACK>();
     if (e != cudaSuccess) return e;
     CUtensorMap tA, tB;
-    if (!encode_kmajor(&tA, a.A, a.M, a.K, kGemmBM) || !encode_kmajor(&tB, a.B, a.N, a.K, BN))
+    if (!encode_kmajor(&tA, a.A, a.M, a.K, kGemmBM) ||
+        !(BMN ? encode_kmajor(&tB, a.B, a.K, a.N, 64) : encode_kmajor(&tB, a.B, a.N, a.K, BN)))
         return cudaErrorInvalidValue;
     const long long tiles = (long long)((a.M + kGemmBM - 1) / kGemmBM) * (a.N / BN);
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const unsigned grid = (unsigned)std::min<long long>(tiles, std::max(sms, 1));
-    gemm_bf16_tc_kernel<BN><<<grid, kGemmThreads, GemmCfg<BN>::kSmem, st>>>(tA, tB, a);
+    gemm_bf16_tc_kernel<BN, BMN, BACK><<<grid, kGemmThreads, GemmCfg<BN>::kSmem, st>>>(tA, tB, a);
     return cudaGetLastError();
 }
 
@@ -472,6 +499,52 @@ cudaError_t gemm_head(const __nv_bfloat16* A, const __nv_bfloat16* B, const floa
     return launch_gemm<256>(a, st);  // N = 512: two 256-column tiles x four column groups = kHeadParts
 }
 
+// dZ = (dZn Wn) * gelu'(Z): the gradient at the layer below, Wn (512 outputs of
+// the layer above, K rows) x 512 read MN-major, with the bias gradient's sums.
+cudaError_t gemm_back(const __nv_bfloat16* dZn, int K, const __nv_bfloat16* Wn, const float* Z, __nv_bfloat16* dZ,
+                      float* colsum, int M, int32_t* flags, cudaStream_t st) {
+    GemmArgs a{};
+    a.A = dZn;
+    a.B = Wn;
+    a.C = dZ;
+    a.M = M;
+    a.N = VH;
+    a.K = K;
+    a.act = kActNone;
+    a.flags = flags;
+    a.wait_ns = kGemmWaitNs;
+    a.Z = Z;
+    a.colsum = colsum;
+    return launch_gemm<256, true, true>(a, st);
+}
+
+// Weight gradients of all four layers into v->dwpart, in `splits` row splits.
+cudaError_t gemm_dw(dvc_value_net* v, int npad, int32_t* flags, int& splits, cudaStream_t st) {
+    DwArgs a{};
+    const __nv_bfloat16* A[4] = {v->dZ[0], v->dZ[1], v->dZ[2], v->H3};
+    const __nv_bfloat16* B[4] = {v->X, v->H1, v->H2, v->dZ4};
+    const int wa[4] = {VH, VH, VH, VH}, wb[4] = {VF, VH, VH, 64};
+    const size_t off[4] = {OFF_W1, OFF_W2, OFF_W3, OFF_W4};
+    int first = 0;
+    for (int q = 0; q < 4; ++q) {
+        if (!encode_kmajor(&a.a[q], A[q], npad, wa[q], 64) || !encode_kmajor(&a.b[q], B[q], npad, wb[q], 64))
+            return cudaErrorInvalidValue;
+        const int tn = std::max(1, wb[q] / 128);
+        a.p[q] = DwProblem{first, tn, wb[q], wb[q] >= 128 ? 2 : 1, q == 3 ? 1 : 0, off[q]};
+        first += wa[q] / 128 * tn;
+    }
+    a.ctas = first;
+    a.nk = npad / 64;
+    splits = std::min(kDwSplits, a.nk);
+    a.splits = splits;
+    a.part = v->dwpart;
+    a.stride = kDwStride;
+    a.flags = flags;
+    a.wait_ns = kGemmWaitNs;
+    gemm_dw_kernel<<<a.ctas * splits, kDwThreads, kDwSmem, st>>>(a);
+    return cudaGetLastError();
+}
+
 int net_alloc(dvc_ctx* c) {
     if (c->vnet) return DVC_OK;
     dvc_value_net* v = new dvc_value_net();
@@ -481,10 +554,7 @@ int net_alloc(dvc_ctx* c) {
               cudaMalloc(&v->W1, (size_t)VH * VF * 2) == cudaSuccess &&
               cudaMalloc(&v->W2, (size_t)VH * VH * 2) == cudaSuccess &&
               cudaMalloc(&v->W3, (size_t)VH * VH * 2) == cudaSuccess &&
-              cudaMalloc(&v->W4, (size_t)VO * VH * 2) == cudaSuccess &&
-              cudaMalloc(&v->W2T, (size_t)VH * VH * 2) == cudaSuccess &&
-              cudaMalloc(&v->W3T, (size_t)VH * VH * 2) == cudaSuccess &&
-              cudaMalloc(&v->W4T, (size_t)VH * 64 * 2) == cudaSuccess && cudaMalloc(&v->b4p, VO * 4) == cudaSuccess;
+              cudaMalloc(&v->W4, (size_t)64 * VH * 2) == cudaSuccess && cudaMalloc(&v->b4p, VO * 4) == cudaSuccess;
     if (!ok || cudaMemset(v->m, 0, NPARAM * 4) != cudaSuccess || cudaMemset(v->v, 0, NPARAM * 4) != cudaSuccess ||
         cudaMemset(v->grad, 0, NPARAM * 4) != cudaSuccess) {
         cudaGetLastError();
@@ -496,12 +566,12 @@ int net_alloc(dvc_ctx* c) {
 }
 
 void free_work(dvc_value_net* v) {
-    void* ptrs[] = {v->X,  v->H1,  v->H2, v->H3,   v->XT,   v->H1T, v->H2T, v->H3T, v->dZ,  v->dZT, v->dZ4,
-                    v->dZ4T, v->Z1, v->Z2, v->Z3, v->L, v->dH, v->dZ4f, v->tmp, v->part, v->loss};
+    void* ptrs[] = {v->X, v->H1, v->H2, v->H3, v->dZ[0], v->dZ[1], v->dZ[2], v->dZ4,
+                    v->Z1, v->Z2, v->Z3, v->L, v->colsum, v->rowpart, v->dwpart};
     for (void* p : ptrs)
         if (p) cudaFree(p);
-    v->X = v->H1 = v->H2 = v->H3 = v->XT = v->H1T = v->H2T = v->H3T = v->dZ = v->dZT = v->dZ4 = v->dZ4T = nullptr;
-    v->Z1 = v->Z2 = v->Z3 = v->L = v->dH = v->dZ4f = v->tmp = v->part = v->loss = nullptr;
+    v->X = v->H1 = v->H2 = v->H3 = v->dZ[0] = v->dZ[1] = v->dZ[2] = v->dZ4 = nullptr;
+    v->Z1 = v->Z2 = v->Z3 = v->L = v->colsum = v->rowpart = v->dwpart = nullptr;
     v->cap = 0;
 }
 
@@ -512,25 +582,29 @@ int ensure_work(dvc_ctx* c, int npad) {
     const size_t r = (size_t)npad;
     auto al = [&](void** p, size_t bytes) { return cudaMalloc(p, bytes) == cudaSuccess; };
     const bool ok = al((void**)&v->X, r * VF * 2) && al((void**)&v->H1, r * VH * 2) && al((void**)&v->H2, r * VH * 2) &&
-                    al((void**)&v->H3, r * VH * 2) && al((void**)&v->XT, r * VF * 2) && al((void**)&v->H1T, r * VH * 2) &&
-                    al((void**)&v->H2T, r * VH * 2) && al((void**)&v->H3T, r * VH * 2) &&
-                    al((void**)&v->dZ, r * VH * 2) && al((void**)&v->dZT, r * VH * 2) && al((void**)&v->dZ4, r * 64 * 2) &&
-                    al((void**)&v->dZ4T, r * VO * 2) && al((void**)&v->Z1, r * VH * 4) && al((void**)&v->Z2, r * VH * 4) &&
-                    al((void**)&v->Z3, r * VH * 4) && al((void**)&v->L, r * kLogitFloats * 4) && al((void**)&v->dH, r * VH * 4) &&
-                    al((void**)&v->dZ4f, r * VO * 4) && al((void**)&v->tmp, (size_t)VO * VH * 4) &&
-                    al((void**)&v->part, ((r + 255) / 256) * (size_t)VF * 4) && al((void**)&v->loss, (r + 1) * 4);
+                    al((void**)&v->H3, r * VH * 2) && al((void**)&v->dZ[0], r * VH * 2) &&
+                    al((void**)&v->dZ[1], r * VH * 2) && al((void**)&v->dZ[2], r * VH * 2) &&
+                    al((void**)&v->dZ4, r * 64 * 2) && al((void**)&v->Z1, r * VH * 4) && al((void**)&v->Z2, r * VH * 4) &&
+                    al((void**)&v->Z3, r * VH * 4) && al((void**)&v->L, r * kLogitFloats * 4) &&
+                    al((void**)&v->colsum, 3 * (r / 32) * VH * 4) && al((void**)&v->rowpart, r / kLossThreads * 8 * 4) &&
+                    al((void**)&v->dwpart, (size_t)kDwSplits * kDwStride * 4);
     if (!ok) {
         cudaGetLastError();
         free_work(v);
         return fail(c, DVC_E_OOM, "value network: workspace of " + std::to_string(npad) + " rows");
     }
+    // a training step's own kernels: their attributes are set here, so that a step may be captured after any call
+    cudaError_t e = gemm_attributes<256, true, true>();
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(gemm_dw_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDwSmem);
+    if (e != cudaSuccess) return cuda_fail(c, e, "value network attributes");
     v->cap = npad;
     return DVC_OK;
 }
 
 int refresh(dvc_ctx* c, cudaStream_t st) {
     dvc_value_net* v = c->vnet;
-    refresh_kernel<<<256, 256, 0, st>>>(v->master, v->W1, v->W2, v->W3, v->W4, v->W2T, v->W3T, v->W4T, v->b4p);
+    refresh_kernel<<<256, 256, 0, st>>>(*v);
     return check_launch(c, "refresh_kernel");
 }
 
@@ -572,19 +646,6 @@ int forward(dvc_ctx* c, const dvc_state* states, int n, int npad, bool train, cu
     dvc_value_net* v = c->vnet;
     return forward_into(c, states, n, npad, v->X, v->H1, v->H2, v->H3, v->L, train ? v->Z1 : nullptr,
                         train ? v->Z2 : nullptr, train ? v->Z3 : nullptr, !train, st);
-}
-
-int transpose(dvc_ctx* c, const __nv_bfloat16* in, __nv_bfloat16* out, int R, int C, cudaStream_t st) {
-    transpose_bf16_kernel<<<dim3(C / 32, R / 32), dim3(32, 8), 0, st>>>(in, out, R, C);
-    return check_launch(c, "transpose_bf16_kernel");
-}
-
-int colsum(dvc_ctx* c, const float* A, int R, int C, float* out, int cols_out, cudaStream_t st) {
-    dvc_value_net* v = c->vnet;
-    const int nb = (R + 255) / 256;
-    colsum_partial_kernel<<<dim3((C + 127) / 128, nb), 128, 0, st>>>(A, R, C, v->part);
-    colsum_final_kernel<<<(cols_out + 127) / 128, 128, 0, st>>>(v->part, nb, C, out, cols_out);
-    return check_launch(c, "colsum");
 }
 
 int check_states_args(dvc_ctx* c, const void* d_states, int n) {
@@ -670,50 +731,24 @@ int dvc_value_train_step(dvc_ctx* c, const dvc_state* d_states, const float* d_l
     dvc_value_net* v = c->vnet;
     int32_t* fl = c->d_flags;
     if (int rc = forward(c, d_states, n, npad, true, st)) return rc;
-    loss_grad_kernel<<<(npad + 127) / 128, 128, 0, st>>>(v->L, d_states, d_labels, n, npad, v->dZ4, v->dZ4T, v->dZ4f,
-                                                          v->loss);
+    loss_grad_kernel<<<npad / kLossThreads, kLossThreads, 0, st>>>(v->L, d_states, d_labels, n, npad, v->dZ4,
+                                                                  v->rowpart);
     if (int rc = check_launch(c, "loss_grad_kernel")) return rc;
-    if (d_loss) mean_kernel<<<1, 32, 0, st>>>(v->loss, n, d_loss);
-    int rc = transpose(c, v->X, v->XT, npad, VF, st);
-    if (!rc) rc = transpose(c, v->H1, v->H1T, npad, VH, st);
-    if (!rc) rc = transpose(c, v->H2, v->H2T, npad, VH, st);
-    if (!rc) rc = transpose(c, v->H3, v->H3T, npad, VH, st);
-    if (rc) return rc;
-    float* g = v->grad;
-    cudaError_t e;
-    // layer 4
-    e = gemm(v->dZ4T, v->H3T, nullptr, nullptr, v->tmp, VO, VH, npad, kActNone, fl, st);
-    if (e != cudaSuccess) return cuda_fail(c, e, "value backward 4");
-    copy_rows_kernel<<<16, 256, 0, st>>>(v->tmp, g + OFF_W4, (size_t)4 * VH);
-    if ((rc = colsum(c, v->dZ4f, npad, VO, g + OFF_B4, 4, st))) return rc;
-    e = gemm(v->dZ4, v->W4T, nullptr, nullptr, v->dH, npad, VH, 64, kActNone, fl, st);
-    if (e != cudaSuccess) return cuda_fail(c, e, "value backward dH3");
-    // layers 3, 2, 1
-    const float* Zs[3] = {v->Z3, v->Z2, v->Z1};
-    const __nv_bfloat16* Hin_T[3] = {v->H2T, v->H1T, v->XT};
-    const __nv_bfloat16* WT[3] = {v->W3T, v->W2T, nullptr};
-    const size_t offW[3] = {OFF_W3, OFF_W2, OFF_W1}, offB[3] = {OFF_B3, OFF_B2, OFF_B1};
-    const int kin[3] = {VH, VH, VF};
-    for (int l = 0; l < 3; ++l) {
-        const size_t cnt = (size_t)npad * VH;
-        gelu_back_kernel<<<1024, 256, 0, st>>>(v->dH, Zs[l], v->dZ, cnt);
-        if ((rc = check_launch(c, "gelu_back_kernel"))) return rc;
-        if ((rc = colsum(c, v->dH, npad, VH, g + offB[l], VH, st))) return rc;
-        if ((rc = transpose(c, v->dZ, v->dZT, npad, VH, st))) return rc;
-        e = gemm(v->dZT, Hin_T[l], nullptr, nullptr, g + offW[l], VH, kin[l], npad, kActNone, fl, st);
-        if (e != cudaSuccess) return cuda_fail(c, e, "value backward dW");
-        if (WT[l]) {
-            e = gemm(v->dZ, WT[l], nullptr, nullptr, v->dH, npad, VH, VH, kActNone, fl, st);
-            if (e != cudaSuccess) return cuda_fail(c, e, "value backward dH");
-        }
-    }
-    // AdamW
+    // the gradient at each hidden layer, from the top
+    const size_t blocks = (size_t)npad / 32 * VH;
+    cudaError_t e = gemm_back(v->dZ4, 64, v->W4, v->Z3, v->dZ[2], v->colsum + 2 * blocks, npad, fl, st);
+    if (e == cudaSuccess)
+        e = gemm_back(v->dZ[2], VH, v->W3, v->Z2, v->dZ[1], v->colsum + blocks, npad, fl, st);
+    if (e == cudaSuccess) e = gemm_back(v->dZ[1], VH, v->W2, v->Z1, v->dZ[0], v->colsum, npad, fl, st);
+    int splits = 1;
+    if (e == cudaSuccess) e = gemm_dw(v, npad, fl, splits, st);
+    if (e != cudaSuccess) return cuda_fail(c, e, "value backward");
     v->step += 1;
-    const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f, wd = 1e-4f;
-    const float c1 = 1.0f - powf(b1, (float)v->step), c2 = 1.0f - powf(b2, (float)v->step);
-    adamw_kernel<<<1024, 256, 0, st>>>(v->master, v->m, v->v, g, NPARAM, lr, b1, b2, eps, wd, c1, c2);
-    if ((rc = check_launch(c, "adamw_kernel"))) return rc;
-    return refresh(c, st);
+    AdamCoef a{lr, 0.9f, 0.999f, 1e-8f, 1e-4f, 0.0f, 0.0f};
+    a.c1 = 1.0f - powf(a.b1, (float)v->step);
+    a.c2 = 1.0f - powf(a.b2, (float)v->step);
+    adamw_kernel<<<kAdamGrid, kAdamThreads, 0, st>>>(*v, splits, npad / 32, npad / kLossThreads, n, a, d_loss);
+    return check_launch(c, "adamw_kernel");
 }
 
 int dvc_value_grads(dvc_ctx* c, float* d_out, void* stream) {
@@ -874,7 +909,7 @@ void dvc_value_free(dvc_ctx* c) {
     if (!c || !c->vnet) return;
     dvc_value_net* v = c->vnet;
     free_work(v);
-    void* ptrs[] = {v->master, v->m, v->v, v->grad, v->W1, v->W2, v->W3, v->W4, v->W2T, v->W3T, v->W4T, v->b4p};
+    void* ptrs[] = {v->master, v->m, v->v, v->grad, v->W1, v->W2, v->W3, v->W4, v->b4p};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     delete v;
