@@ -98,12 +98,16 @@ __device__ __forceinline__ uint64_t global_ns() {
 }
 
 // Bounded wait: false once limit_ns of global time have passed (checked every
-// 64 polls) or after kWaitLimit polls, whichever comes first.
+// 64 polls) or after kWaitLimit polls, whichever comes first.  The first polls,
+// where a working pipeline's waits end, do not read the global timer.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t phase, uint64_t limit_ns) {
-    const uint64_t t0 = global_ns();
+    uint64_t t0 = 0;
     for (uint32_t i = 0; i < kWaitLimit; ++i) {
         if (mbar_try_wait(bar, phase)) return true;
-        if ((i & 63u) == 63u && global_ns() - t0 > limit_ns) return false;
+        if ((i & 63u) != 63u) continue;
+        const uint64_t t = global_ns();
+        if (i == 63u) t0 = t;
+        else if (t - t0 > limit_ns) return false;
     }
     return false;
 }
@@ -121,17 +125,26 @@ __device__ __forceinline__ void tc_dealloc(uint32_t taddr, uint32_t ncols) {
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
+// MMAs, commits and copies are issued by one elected lane of a warp that runs
+// its loop together: the operands then stay in uniform registers, which a
+// branch on the lane number would force through the vector registers for every
+// instruction.  All 32 lanes call.
 __device__ __forceinline__ void tc_mma(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
+        "{\n\t.reg .pred p, e;\n\t"
+        "elect.sync _|e, 0xFFFFFFFF;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(dtmem),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc));
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(dtmem),
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc)
+        : "memory");
 }
 
 __device__ __forceinline__ void tc_commit(uint64_t* bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-                 : "memory");
+    asm volatile(
+        "{\n\t.reg .pred e;\n\t"
+        "elect.sync _|e, 0xFFFFFFFF;\n\t"
+        "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(smem_u32(bar))
+        : "memory");
 }
 
 // 32 lanes x 16 columns of 32-bit accumulators (lane = row of the tile).
@@ -153,24 +166,34 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
 }
 
 __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
+    asm volatile(
+        "{\n\t.reg .pred e;\n\t"
+        "elect.sync _|e, 0xFFFFFFFF;\n\t"
+        "@e mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n\t}" ::"r"(smem_u32(bar)),
+        "r"(bytes)
+        : "memory");
 }
 
 // Contiguous copy of `bytes` (a multiple of 16, both addresses 16-byte
 // aligned) from global to shared memory, completing `bytes` of the barrier's
 // transaction count.
 __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint64_t* bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-                 "l"(src), "r"(bytes), "r"(smem_u32(bar))
-                 : "memory");
+    asm volatile(
+        "{\n\t.reg .pred e;\n\t"
+        "elect.sync _|e, 0xFFFFFFFF;\n\t"
+        "@e cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n\t}" ::"r"(dst),
+        "l"(src), "r"(bytes), "r"(smem_u32(bar))
+        : "memory");
 }
 
 // 2-D TMA load of box (x = K offset, y = row offset) into shared memory,
 // completing `bytes` of the barrier's transaction count.
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
     asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
-            dst),
+        "{\n\t.reg .pred e;\n\t"
+        "elect.sync _|e, 0xFFFFFFFF;\n\t"
+        "@e cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+        "\n\t}" ::"r"(dst),
         "l"((uint64_t)map), "r"(x), "r"(y), "r"(smem_u32(bar))
         : "memory");
 }
@@ -323,76 +346,75 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     tc_fence_after();
     const uint32_t tmem = s_tmem;
     if (warp == 0) {
-        if (lane == 0) {
-            // producer: K slices of every tile of this CTA, up to S in flight
-            int it = 0;
-            bool stop = false;
-            for (int t = blockIdx.x; t < tiles && !stop; t += gridDim.x) {
-                const int m0 = (t / ntn) * kGemmBM, n0 = (t % ntn) * BN;
-                for (int kc = 0; kc < nk; ++kc, ++it) {
-                    const int s = it % S, r = it / S;
-                    if (a.starve || (it >= S && !mbar_wait(&s_empty[s], (uint32_t)(r - 1) & 1u, a.wait_ns)) ||
-                        *fail) {
-                        *fail = 1;
-                        stop = true;
-                        break;
-                    }
-                    const uint32_t sa = base + (uint32_t)s * Cfg::kStage;
-                    mbar_expect_tx(&s_full[s], Cfg::kStage);
-                    if (a.a_blocked)  // the four 4 KB blocks of K slice kc of row tile m0 / 128
-                        bulk_load(sa, a.A + kblocked_index(m0, kc * kGemmBK, a.K), Cfg::kA, &s_full[s]);
-                    else
-                        tma_load_2d(sa, &tA, kc * kGemmBK, m0, &s_full[s]);
-                    if constexpr (BMN) {
+        // producer: K slices of every tile of this CTA, up to S in flight
+        int it = 0;
+        bool stop = false;
+        for (int t = blockIdx.x; t < tiles && !stop; t += gridDim.x) {
+            const int m0 = (t / ntn) * kGemmBM, n0 = (t % ntn) * BN;
+            for (int kc = 0; kc < nk; ++kc, ++it) {
+                const int s = it % S, r = it / S;
+                if (__any_sync(0xFFFFFFFFu,
+                               a.starve ||
+                                   (it >= S && !mbar_wait(&s_empty[s], (uint32_t)(r - 1) & 1u, a.wait_ns)) ||
+                                   *fail)) {
+                    *fail = 1;
+                    stop = true;
+                    break;
+                }
+                const uint32_t sa = base + (uint32_t)s * Cfg::kStage;
+                mbar_expect_tx(&s_full[s], Cfg::kStage);
+                if (a.a_blocked)  // the four 4 KB blocks of K slice kc of row tile m0 / 128
+                    bulk_load(sa, a.A + kblocked_index(m0, kc * kGemmBK, a.K), Cfg::kA, &s_full[s]);
+                else
+                    tma_load_2d(sa, &tA, kc * kGemmBK, m0, &s_full[s]);
+                if constexpr (BMN) {
 #pragma unroll
-                        for (int j = 0; j < BN / 64; ++j)
-                            tma_load_2d(sa + Cfg::kA + (uint32_t)j * 8192u, &tB, n0 + 64 * j, kc * kGemmBK, &s_full[s]);
-                    } else {
-                        tma_load_2d(sa + Cfg::kA, &tB, kc * kGemmBK, n0, &s_full[s]);
-                    }
+                    for (int j = 0; j < BN / 64; ++j)
+                        tma_load_2d(sa + Cfg::kA + (uint32_t)j * 8192u, &tB, n0 + 64 * j, kc * kGemmBK, &s_full[s]);
+                } else {
+                    tma_load_2d(sa + Cfg::kA, &tB, kc * kGemmBK, n0, &s_full[s]);
                 }
             }
-            s_issued = it;
         }
+        if (lane == 0) s_issued = it;
     } else if (warp == 1) {
-        if (lane == 0) {
-            // MMA issuer: tile j accumulates into buffer j & 1 once the
-            // epilogue has drained that buffer's previous tile
-            const uint32_t idesc = idesc_bf16_f32(kGemmBM, BN, false, BMN);
-            int it = 0, j = 0;
-            bool stop = false;
-            for (int t = blockIdx.x; t < tiles && !stop; t += gridDim.x, ++j) {
-                const int b = j & 1, u = j >> 1;
-                if (u > 0 && !mbar_wait(&s_acce[b], (uint32_t)(u - 1) & 1u, a.wait_ns)) {
+        // MMA issuer: tile j accumulates into buffer j & 1 once the
+        // epilogue has drained that buffer's previous tile
+        const uint32_t idesc = idesc_bf16_f32(kGemmBM, BN, false, BMN);
+        int it = 0, j = 0;
+        bool stop = false;
+        for (int t = blockIdx.x; t < tiles && !stop; t += gridDim.x, ++j) {
+            const int b = j & 1, u = j >> 1;
+            if (__any_sync(0xFFFFFFFFu,
+                           u > 0 && !mbar_wait(&s_acce[b], (uint32_t)(u - 1) & 1u, a.wait_ns))) {
+                *fail = 1;
+                break;
+            }
+            tc_fence_after();
+            const uint32_t acc = tmem + (uint32_t)b * Cfg::kAccCols;
+            for (int kc = 0; kc < nk; ++kc, ++it) {
+                const int s = it % S, r = it / S;
+                if (__any_sync(0xFFFFFFFFu, !mbar_wait(&s_full[s], (uint32_t)r & 1u, a.wait_ns) || *fail)) {
                     *fail = 1;
+                    stop = true;
                     break;
                 }
                 tc_fence_after();
-                const uint32_t acc = tmem + (uint32_t)b * Cfg::kAccCols;
-                for (int kc = 0; kc < nk; ++kc, ++it) {
-                    const int s = it % S, r = it / S;
-                    if (!mbar_wait(&s_full[s], (uint32_t)r & 1u, a.wait_ns) || *fail) {
-                        *fail = 1;
-                        stop = true;
-                        break;
-                    }
-                    tc_fence_after();
-                    const uint32_t sa = base + (uint32_t)s * Cfg::kStage;
+                const uint32_t sa = base + (uint32_t)s * Cfg::kStage;
 #pragma unroll
-                    for (int kk = 0; kk < kGemmBK / 16; ++kk) {
-                        const uint64_t ad = a.a_blocked ? smem_desc_noswz(sa + (uint32_t)kk * 4096u, 2048u, 128u)
-                                                        : smem_desc_sw128(sa + (uint32_t)kk * 32u);
-                        const uint64_t bd = BMN ? smem_desc_mn128(sa + Cfg::kA + (uint32_t)kk * 2048u, 8192u)
-                                                : smem_desc_sw128(sa + Cfg::kA + (uint32_t)kk * 32u);
-                        tc_mma(acc, ad, bd, idesc, (kc > 0 || kk > 0) ? 1u : 0u);
-                    }
-                    tc_commit(&s_empty[s]);
+                for (int kk = 0; kk < kGemmBK / 16; ++kk) {
+                    const uint64_t ad = a.a_blocked ? smem_desc_noswz(sa + (uint32_t)kk * 4096u, 2048u, 128u)
+                                                    : smem_desc_sw128(sa + (uint32_t)kk * 32u);
+                    const uint64_t bd = BMN ? smem_desc_mn128(sa + Cfg::kA + (uint32_t)kk * 2048u, 8192u)
+                                            : smem_desc_sw128(sa + Cfg::kA + (uint32_t)kk * 32u);
+                    tc_mma(acc, ad, bd, idesc, (kc > 0 || kk > 0) ? 1u : 0u);
                 }
-                if (!stop) tc_commit(&s_accf[b]);
+                tc_commit(&s_empty[s]);
             }
-            s_consumed = it;
-            tc_commit(&s_done);  // arrives when every MMA issued above has completed
+            if (!stop) tc_commit(&s_accf[b]);
         }
+        if (lane == 0) s_consumed = it;
+        tc_commit(&s_done);  // arrives when every MMA issued above has completed
     } else if (warp >= 4) {
         // epilogue: warp w reads tensor-memory lanes 32 (w mod 4) .. +31 (one
         // output row per thread) and one of up to four column groups
@@ -528,48 +550,46 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
 
 // Weight gradients of all layers in one launch: per layer dW = dZ^T H over the
 // batch (K = rows), both operands read MN-major straight from the row-major
-// activations.  A layer's 512 x 512 outputs are only 16 tiles of 128 x 128, so
-// the rows are split: CTA (problem, tile, split) leaves the FP32 sums of its rows
-// in part[split], and the optimiser adds the splits in order.  Two CTAs per SM
-// (three 32 KB stages each).  What bounds it is operand traffic from L2.
+// activations, tiles of 128 x 64 (108 of them: one wave).  Each tile sums all
+// rows in one accumulator: splitting them over CTAs and adding the parts was
+// measured at 20 us against 40 us, but rounds otherwise than one sum, and
+// AdamW's first steps (g / |g|) turn that into visible differences where a
+// gradient is near zero.  What bounds it is the chain of 4 MMAs per 64 rows (512 in
+// all for 8,192 rows, about 130 cycles each) and, close to it, operand traffic
+// from L2 (24 KB per 64 rows and tile).
 // The last problem is the output layer, transposed: D[512][64] = H3^T dZ4, its
 // first four columns written as the 4 x 512 gradient.
 struct DwProblem {
-    int first;        // its first CTA within a split
-    int tiles_n;      // column tiles
-    int cols;         // columns of the gradient (row stride)
-    int boxes_b;      // 64-column boxes of B per tile (2, or 1 for 64 columns)
-    int transposed;   // write D[m][n] to [n][m] for n < 4
-    size_t offset;    // of the gradient in the parameter array
+    int first;       // its first CTA
+    int tiles_n;     // column tiles
+    int cols;        // columns of the gradient (row stride)
+    int transposed;  // write D[m][n] to [n][m] for n < 4
+    size_t offset;   // of the gradient in the parameter array
 };
 struct DwArgs {
     CUtensorMap a[4], b[4];
     DwProblem p[4];
-    int ctas, splits, nk;  // CTAs per split; 64-row slices of the batch
-    float* part;
-    size_t stride;  // floats between splits
+    int nk;  // 64-row slices of the batch
+    float* grad;
     int32_t* flags;
     uint64_t wait_ns;
 };
-constexpr int kDwStages = 3;
-constexpr uint32_t kDwStage = 32768u;
+constexpr int kDwStages = 8;
+constexpr uint32_t kDwStage = 24576u;
 constexpr uint32_t kDwSmem = kDwStages * kDwStage + 1024u;
 constexpr int kDwThreads = 256;
 
-__global__ void __launch_bounds__(kDwThreads, 2) gemm_dw_kernel(const __grid_constant__ DwArgs a) {
+__global__ void __launch_bounds__(kDwThreads, 1) gemm_dw_kernel(const __grid_constant__ DwArgs a) {
     extern __shared__ __align__(1024) unsigned char gsm[];
     __shared__ uint64_t s_full[kDwStages], s_empty[kDwStages], s_acc;
     __shared__ uint32_t s_tmem;
     __shared__ int s_fail, s_issued, s_consumed;
     volatile int* fail = &s_fail;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int split = (int)blockIdx.x / a.ctas, cta = (int)blockIdx.x % a.ctas;
     int q = 0;
-    while (q < 3 && cta >= a.p[q + 1].first) ++q;
+    while (q < 3 && (int)blockIdx.x >= a.p[q + 1].first) ++q;
     const DwProblem pr = a.p[q];
-    const int tile = cta - pr.first, m0 = tile / pr.tiles_n * 128, n0 = tile % pr.tiles_n * 128;
-    const int k0 = (int)((long long)a.nk * split / a.splits), k1 = (int)((long long)a.nk * (split + 1) / a.splits);
-    const int nk = k1 - k0;  // at least 1: splits <= nk
+    const int tile = (int)blockIdx.x - pr.first, m0 = tile / pr.tiles_n * 128, n0 = tile % pr.tiles_n * 64;
     const uint32_t base = (smem_u32(gsm) + 1023u) & ~1023u;
     if (tid == 0) {
         for (int s = 0; s < kDwStages; ++s) {
@@ -580,35 +600,35 @@ __global__ void __launch_bounds__(kDwThreads, 2) gemm_dw_kernel(const __grid_con
         s_fail = s_issued = s_consumed = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 0) tc_alloc(&s_tmem, 128u);
+    if (warp == 0) tc_alloc(&s_tmem, 64u);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = s_tmem;
-    const uint32_t bytes = 16384u + 8192u * (uint32_t)pr.boxes_b;
-    if (warp == 0 && lane == 0) {
+    if (warp == 0) {
         int it = 0;
-        for (; it < nk; ++it) {
+        for (; it < a.nk; ++it) {
             const int s = it % kDwStages, r = it / kDwStages;
-            if ((it >= kDwStages && !mbar_wait(&s_empty[s], (uint32_t)(r - 1) & 1u, a.wait_ns)) || *fail) {
+            if (__any_sync(0xFFFFFFFFu,
+                           (it >= kDwStages && !mbar_wait(&s_empty[s], (uint32_t)(r - 1) & 1u, a.wait_ns)) || *fail)) {
                 *fail = 1;
                 break;
             }
             const uint32_t sa = base + (uint32_t)s * kDwStage;
-            mbar_expect_tx(&s_full[s], bytes);
-            for (int j = 0; j < 2; ++j)
-                tma_load_2d(sa + (uint32_t)j * 8192u, &a.a[q], m0 + 64 * j, (k0 + it) * 64, &s_full[s]);
-            for (int j = 0; j < pr.boxes_b; ++j)
-                tma_load_2d(sa + 16384u + (uint32_t)j * 8192u, &a.b[q], n0 + 64 * j, (k0 + it) * 64, &s_full[s]);
+            mbar_expect_tx(&s_full[s], kDwStage);
+            tma_load_2d(sa, &a.a[q], m0, it * 64, &s_full[s]);
+            tma_load_2d(sa + 8192u, &a.a[q], m0 + 64, it * 64, &s_full[s]);
+            tma_load_2d(sa + 16384u, &a.b[q], n0, it * 64, &s_full[s]);
         }
-        s_issued = it;
+        if (lane == 0) s_issued = it;
     }
-    if (warp == 1 && lane == 0) {
-        const uint32_t idesc = idesc_bf16_f32(128, 64 * pr.boxes_b, true, true);
+    if (warp == 1) {
+        const uint32_t idesc = idesc_bf16_f32(128, 64, true, true);
         int it = 0;
-        for (; it < nk; ++it) {
+        for (; it < a.nk; ++it) {
             const int s = it % kDwStages;
-            if (!mbar_wait(&s_full[s], (uint32_t)(it / kDwStages) & 1u, a.wait_ns) || *fail) {
+            if (__any_sync(0xFFFFFFFFu,
+                           !mbar_wait(&s_full[s], (uint32_t)(it / kDwStages) & 1u, a.wait_ns) || *fail)) {
                 *fail = 1;
                 break;
             }
@@ -620,7 +640,7 @@ __global__ void __launch_bounds__(kDwThreads, 2) gemm_dw_kernel(const __grid_con
                        smem_desc_mn128(sa + 16384u + (uint32_t)kk * 2048u, 8192u), idesc, (it > 0 || kk > 0) ? 1u : 0u);
             tc_commit(&s_empty[s]);
         }
-        s_consumed = it;
+        if (lane == 0) s_consumed = it;
         tc_commit(&s_acc);  // arrives when every MMA issued above has completed
     }
     __syncthreads();
@@ -630,7 +650,7 @@ __global__ void __launch_bounds__(kDwThreads, 2) gemm_dw_kernel(const __grid_con
         const int quarter = warp & 3, half = warp >> 2;
         const uint32_t acc = tmem + ((uint32_t)(quarter * 32) << 16);
         const int row = m0 + quarter * 32 + lane;
-        float* out = a.part + (size_t)split * a.stride + pr.offset;
+        float* out = a.grad + pr.offset;
         if (pr.transposed) {
             float v[16];
             tc_ld16(acc, v);
@@ -638,9 +658,9 @@ __global__ void __launch_bounds__(kDwThreads, 2) gemm_dw_kernel(const __grid_con
                 for (int o = 0; o < 4; ++o) out[(size_t)o * 512 + row] = v[o];
         } else {
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
+            for (int c = 0; c < 2; ++c) {
                 float v[16];
-                const int col = half * 64 + c * 16;
+                const int col = half * 32 + c * 16;
                 tc_ld16(acc + (uint32_t)col, v);
                 float* o = out + (size_t)row * pr.cols + n0 + col;
                 st_global_v8(o, reinterpret_cast<const uint32_t*>(v));
@@ -656,7 +676,7 @@ __global__ void __launch_bounds__(kDwThreads, 2) gemm_dw_kernel(const __grid_con
     __syncthreads();
     if (warp == 0) {
         tc_fence_after();
-        tc_dealloc(tmem, 128u);
+        tc_dealloc(tmem, 64u);
     }
 }
 

@@ -10,10 +10,6 @@ struct dvc_value_net;  // value network state (dvc_value.cu)
 struct dvc_ctx;
 struct dvc_state;
 void dvc_value_free(dvc_ctx* c);
-// Win probabilities (n x 4, absolute seats) of n leaves by the context's
-// value network, enqueued on st; no argument checks (library-internal).
-int dvc_value_forward_probs(dvc_ctx* c, const dvc_state* d_leaves, int n, float* d_probs, cudaStream_t st);
-
 // Value-network activations owned by one caller (a forest's value-mode
 // pipeline), so that a captured graph never points into the context's own
 // workspace, which other calls may reallocate.  rows: a multiple of 128.

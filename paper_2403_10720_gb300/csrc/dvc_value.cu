@@ -18,8 +18,10 @@
 #include <vector>
 
 #include "dvc_device.cuh"
+#include "dvc_features.cuh"
 #include "dvc_gemm.cuh"
 #include "dvc_internal.h"
+#include "dvc_mlp.cuh"
 
 using namespace dvc;
 using namespace dvc_host;
@@ -33,10 +35,6 @@ constexpr int kLogitFloats = kHeadParts * 4 > VO ? kHeadParts * 4 : VO;
 constexpr size_t OFF_W1 = 0, OFF_B1 = OFF_W1 + (size_t)VH * VF, OFF_W2 = OFF_B1 + VH, OFF_B2 = OFF_W2 + (size_t)VH * VH,
                  OFF_W3 = OFF_B2 + VH, OFF_B3 = OFF_W3 + (size_t)VH * VH, OFF_W4 = OFF_B3 + VH,
                  OFF_B4 = OFF_W4 + 4 * VH, NPARAM = OFF_B4 + 4;
-// row splits of the weight gradients (280 CTAs at two per SM: one wave), and
-// floats from one split to the next (32-byte aligned)
-constexpr int kDwSplits = 5;
-constexpr size_t kDwStride = (NPARAM + 7) / 8 * 8;
 
 }  // namespace
 
@@ -44,12 +42,12 @@ struct dvc_value_net {
     float *master, *m, *v, *grad;
     __nv_bfloat16 *W1, *W2, *W3, *W4;  // W4: 64 x 512, rows 4.. zero
     float* b4p;                        // 16
+    int clusters;                      // clusters of the small-batch kernel that run at once
     int cap;                           // workspace rows (multiple of 128)
     __nv_bfloat16 *X, *H1, *H2, *H3, *dZ[3], *dZ4;  // dZ of layers 1..3; of the output layer, 64 columns
     float *Z1, *Z2, *Z3, *L;
     float* colsum;                     // bias gradients of layers 1..3 by 32 rows: 3 x (rows / 32) x 512
     float* rowpart;                    // per CTA of the loss kernel: loss, four output-bias gradients, padding (8)
-    float* dwpart;                     // weight gradients by row split: kDwSplits x kDwStride
     long long step;
 };
 
@@ -57,136 +55,52 @@ namespace {
 
 // ------------------------------------------------------------------ kernels
 
-__device__ __forceinline__ uint32_t unknown_mask(const G& g) { return g.tmask & ~g.hand(g.cur) & ~g.rev; }
+// Feature bits of 32 states per CTA, four warps: warp 0 sets the tiles' bits,
+// warp k the slots of opponent k, lane r works on row r.  The bits meet in
+// shared memory, from where all threads write the rows: a byte of feature bits
+// becomes 8 BF16 values through a 256-entry table (4 FP32 values per nibble for
+// Xf).  Rows n .. npad-1 are written as zeros.  What bounds it is the chain of one
+// row's slots; with a thread per row 8,192 rows took 11.9 us, now 6.4.
+constexpr int kFeatThreads = 128, kFeatRows = 32;
 
-// One thread per state: the row's 640 feature bits are built in registers at
-// fixed positions (every loop below is unrolled), parked in the thread's own
-// shared-memory row, and then each warp writes its 32 consecutive rows -- one
-// contiguous stretch of X -- with coalesced 16-byte stores: a byte of feature
-// bits becomes 8 BF16 values through a 256-entry table (4 FP32 values per
-// nibble for Xf).  Rows n .. npad-1 are written as zeros.  Blocks of 256.
-constexpr int kFeatWords = VF / 32;         // 20
-constexpr int kFeatPitch = kFeatWords + 1;  // 21: the 32 rows of a warp start in 32 different banks
-
-// OR a field of `width` bits into the bit vector f at position pos (both
-// known at compile time once the caller's loops are unrolled).
-__device__ __forceinline__ void or_bits(uint32_t* f, int pos, uint32_t field, int width) {
-    const int w = pos >> 5, sh = pos & 31;
-    f[w] |= field << sh;
-    if (sh + width > 32) f[w + 1] |= field >> (32 - sh);
-}
-
-__global__ void __launch_bounds__(256) features_kernel(const dvc_state* states, int n, int npad, __nv_bfloat16* X,
-                                                       float* Xf, int blocked) {
-    __shared__ uint32_t s_rows[256 * kFeatPitch];
+__global__ void __launch_bounds__(kFeatThreads)
+    features_kernel(const dvc_state* states, int n, int npad, __nv_bfloat16* X, float* Xf, int blocked) {
+    __shared__ uint32_t s_rows[kFeatRows * kFeatPitch];
     __shared__ uint4 s_lut[256];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (int b = tid; b < 256; b += blockDim.x) {
-        uint32_t w[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-            w[j] = (((b >> (2 * j)) & 1) ? 0x3F80u : 0u) | (((b >> (2 * j + 1)) & 1) ? 0x3F800000u : 0u);
-        s_lut[b] = make_uint4(w[0], w[1], w[2], w[3]);
-    }
-    uint32_t f[kFeatWords];
-#pragma unroll
-    for (int k = 0; k < kFeatWords; ++k) f[k] = 0u;
-    const int row = blockIdx.x * blockDim.x + tid;
-    if (row < n) {
-        const G g = load_state(states[row]);
-        uint32_t q1 = g.cur + 1u, q2 = g.cur + 2u, q3 = g.cur + 3u;
-        q1 = q1 >= g.np ? q1 - g.np : q1;
-        q2 = q2 >= g.np ? q2 - g.np : q2;
-        q3 = q3 >= g.np ? q3 - g.np : q3;
-        const uint32_t M1 = g.hand(q1), M2 = g.np > 2u ? g.hand(q2) : 0u, M3 = g.np > 3u ? g.hand(q3) : 0u;
-        const uint32_t held = g.h0 | g.h1 | g.h2 | g.h3;
-        // tiles: bit 7t + (owner seat relative to the mover), 7t + 4 + face-up,
-        // 7t + 6 if drawn this turn; tiles in the pool have none
-#pragma unroll
-        for (int t = 0; t < 26; ++t) {
-            const uint32_t r = ((M1 >> t) & 1u) | (((M2 >> t) & 1u) << 1) | (((M3 >> t) & 1u) * 3u);
-            const uint32_t grp = (1u << r) | (16u << ((g.rev >> t) & 1u)) | ((uint32_t)t == g.drawn ? 64u : 0u);
-            or_bits(f, 7 * t, ((held >> t) & 1u) ? grp : 0u, 7);
-        }
-        const uint32_t U = unknown_mask(g);
-        const uint32_t jok = (U & kJokerMask) ? 1u << 12 : 0u;
-        // opponent k (seat cur + k), slot s: 13 bits at 182 + ((k - 1) * 11 + s) * 13;
-        // a face-up tile sets its value (a joker 12); a face-down slot sets every
-        // value the mover cannot see strictly between its face-up numbered
-        // neighbours, plus bit 12 if a joker is unseen.  Slots are walked left
-        // to right: numbered tiles ascend by id, each joker stands where its
-        // gap puts it, and a joker's right-hand threshold is the next numbered
-        // tile of the row (or 24).
-#pragma unroll
-        for (int k = 1; k < 4; ++k) {
-            const uint32_t hq = k == 1 ? M1 : (k == 2 ? M2 : M3);
-            const uint32_t len = (uint32_t)k < g.np ? (uint32_t)__popc(hq) : 0u;
-            const uint32_t num = hq & kNumMask, R = num & g.rev;
-            const uint32_t jp0 = (hq >> 24) & 1u ? joker_pos(g, hq, 0u) : 0xFFu;
-            const uint32_t jp1 = (hq >> 25) & 1u ? joker_pos(g, hq, 1u) : 0xFFu;
-            uint32_t rem = num;
-#pragma unroll
-            for (int sl = 0; sl < 11; ++sl) {
-                if ((uint32_t)sl < len) {
-                    const bool j0 = (uint32_t)sl == jp0, j1 = (uint32_t)sl == jp1;
-                    const uint32_t low = rem ? (uint32_t)__ffs(rem) - 1u : 24u;
-                    const uint32_t t = j0 ? 24u : (j1 ? 25u : low);
-                    const uint32_t thr = low;  // a numbered slot's own tile, or the tile right of a joker
-                    if (!j0 && !j1) rem &= rem - 1u;
-                    uint32_t field;
-                    if ((g.rev >> t) & 1u) {
-                        field = 1u << (t < 24u ? t >> 1 : 12u);
-                    } else {
-                        const uint32_t below_thr = thr >= 32u ? 0xFFFFFFFFu : (1u << thr) - 1u;
-                        const uint32_t left = R & below_thr, right = R & ~below_thr;
-                        const int lo = left ? 31 - __clz(left) : -1;
-                        const int hi = right ? __ffs(right) - 1 : 24;
-                        const uint32_t above = lo < 0 ? 0x00FFFFFFu : (0x00FFFFFFu & ~((2u << lo) - 1u));
-                        const uint32_t below = (1u << hi) - 1u;
-                        const uint32_t m = U & above & below;
-                        uint32_t x = (m | (m >> 1)) & 0x00555555u;
-                        x = (x | (x >> 1)) & 0x00333333u;
-                        x = (x | (x >> 2)) & 0x000F0F0Fu;
-                        x = ((x | (x >> 4)) & 0x000000FFu) | ((x >> 8) & 0x00000F00u);
-                        field = x | jok;
-                    }
-                    or_bits(f, 182 + ((k - 1) * 11 + sl) * 13, field, 13);
-                }
-            }
-        }
-    }
+    const int row0 = blockIdx.x * kFeatRows, row = row0 + lane;
+    dvc_state st = {};
+    if (row < n) st = states[row];
+    for (int b = tid; b < 256; b += kFeatThreads) s_lut[b] = feature_bf16((uint32_t)b);
+    for (int e = tid; e < kFeatRows * kFeatPitch; e += kFeatThreads) s_rows[e] = 0u;
+    __syncthreads();
+    uint32_t* mine = s_rows + lane * kFeatPitch;
+    if (row < n) feature_bits(load_state(st), warp, mine);
+    __syncthreads();
     if (blocked) {
-        // K-blocked X (npad a multiple of 128): each thread writes its own row,
-        // 16 bytes per 8 features; the warp's 32 rows are contiguous in a block
-        __syncthreads();  // the table
+        // K-blocked X (npad a multiple of 128): 16 bytes per 8 features; a warp's
+        // 32 rows are contiguous in a block
         if (X && row < npad) {
             __nv_bfloat16* xr = X + kblocked_index(row, 0, VF);
-#pragma unroll
-            for (int b = 0; b < VF / 8; ++b)
+            for (int b = warp; b < VF / 8; b += kFeatThreads / 32)
                 *reinterpret_cast<uint4*>(xr + (size_t)(b >> 1) * 2048 + (size_t)(b & 1) * 1024) =
-                    s_lut[(f[b >> 2] >> (8 * (b & 3))) & 0xFFu];
+                    s_lut[(mine[b >> 2] >> (8 * (b & 3))) & 0xFFu];
         }
         return;
     }
-    uint32_t* mine = s_rows + tid * kFeatPitch;
-#pragma unroll
-    for (int k = 0; k < kFeatWords; ++k) mine[k] = f[k];
-    __syncthreads();
-    const int row0 = blockIdx.x * blockDim.x + warp * 32;
-    const int nrows = min(32, npad - row0);
-    const uint32_t* wrows = s_rows + warp * 32 * kFeatPitch;
+    const int nrows = min(kFeatRows, npad - row0);
     if (X && nrows > 0) {
         uint4* dst = reinterpret_cast<uint4*>(X + (size_t)row0 * VF);
-        for (int c = lane; c < nrows * (VF / 8); c += 32) {
+        for (int c = tid; c < nrows * (VF / 8); c += kFeatThreads) {
             const int r = c / (VF / 8), k = c - r * (VF / 8);
-            dst[c] = s_lut[(wrows[r * kFeatPitch + (k >> 2)] >> (8 * (k & 3))) & 0xFFu];
+            dst[c] = s_lut[(s_rows[r * kFeatPitch + (k >> 2)] >> (8 * (k & 3))) & 0xFFu];
         }
     }
     if (Xf && nrows > 0) {
         float4* dst = reinterpret_cast<float4*>(Xf + (size_t)row0 * VF);
-        for (int c = lane; c < nrows * (VF / 4); c += 32) {
+        for (int c = tid; c < nrows * (VF / 4); c += kFeatThreads) {
             const int r = c / (VF / 4), k = c - r * (VF / 4);
-            const uint32_t nib = (wrows[r * kFeatPitch + (k >> 3)] >> (4 * (k & 7))) & 0xFu;
+            const uint32_t nib = (s_rows[r * kFeatPitch + (k >> 3)] >> (4 * (k & 7))) & 0xFu;
             dst[c] = make_float4((float)(nib & 1u), (float)((nib >> 1) & 1u), (float)((nib >> 2) & 1u),
                                  (float)((nib >> 3) & 1u));
         }
@@ -199,9 +113,6 @@ __global__ void __launch_bounds__(256) features_kernel(const dvc_state* states, 
 __global__ void softmax_head_kernel(const float* parts, const float* b4, const dvc_state* states, int n, float* out) {
     const int row = blockIdx.x * blockDim.x + threadIdx.x;
     if (row >= n) return;
-    const dvc_state& s = states[row];
-    const int P = (s.nplayers >= 2 && s.nplayers <= 4) ? s.nplayers : 2;
-    const int cur = s.cur < P ? s.cur : 0;
     const float4* pp = reinterpret_cast<const float4*>(parts) + (size_t)row * kHeadParts;
     float4 z = make_float4(b4[0], b4[1], b4[2], b4[3]);
 #pragma unroll
@@ -212,17 +123,7 @@ __global__ void softmax_head_kernel(const float* parts, const float* b4, const d
         z.z += q.z;
         z.w += q.w;
     }
-    const float zz[4] = {z.x, z.y, z.z, z.w};
-    float mx = zz[0];
-    for (int r = 1; r < P; ++r) mx = fmaxf(mx, zz[r]);
-    float e[4], sum = 0.0f;
-    for (int r = 0; r < P; ++r) {
-        e[r] = expf(zz[r] - mx);
-        sum += e[r];
-    }
-    float* o = out + (size_t)row * 4;
-    o[0] = o[1] = o[2] = o[3] = 0.0f;
-    for (int r = 0; r < P; ++r) o[(cur + r) % P] = e[r] / sum;
+    softmax_seats(states[row], z, out + (size_t)row * 4);
 }
 
 // Cross-entropy against soft labels (absolute seats) and dL/dlogits / n.
@@ -309,36 +210,28 @@ __device__ __forceinline__ void store_bf16_weights(const dvc_value_net& v, size_
         make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
 }
 
-// End of a training step in one launch: sum the partial gradients (weights over
-// the row splits, biases over the 32-row column sums, output biases and loss
-// over the loss kernel's CTAs, all in a fixed order), AdamW, BF16 copies.
-// CTAs 0 .. kAdamMain-1 take four weights per thread; then 16 CTAs per hidden
-// layer take 32 biases each, and the last one the output biases and the loss.
-// What bounds it is memory: gradient partials, master, moments and their updates.
+// End of a training step in one launch: sum the partial gradients (biases over the
+// 32-row column sums, output biases and loss over the loss kernel's CTAs, in a
+// fixed order), AdamW, BF16 copies.  CTAs 0 .. kAdamMain-1 take four weights per
+// thread; then 16 CTAs per hidden layer take 32 biases each, and the last one the
+// output biases and the loss.  What bounds it is memory: gradients, master,
+// moments and their updates.
 constexpr int kAdamThreads = 256;
 constexpr int kAdamMain = (int)((NPARAM / 4 + kAdamThreads - 1) / kAdamThreads);
 constexpr int kAdamGrid = kAdamMain + 3 * (VH / 32) + 1;
 __global__ void __launch_bounds__(kAdamThreads)
-    adamw_kernel(dvc_value_net v, int splits, int row_blocks, int loss_ctas, int n, AdamCoef a, float* loss_out) {
+    adamw_kernel(dvc_value_net v, int row_blocks, int loss_ctas, int n, AdamCoef a, float* loss_out) {
     const int tid = threadIdx.x;
     if ((int)blockIdx.x < kAdamMain) {
         const size_t i = ((size_t)blockIdx.x * kAdamThreads + tid) * 4;
         if (i >= NPARAM || is_bias_index(i)) return;  // tensors begin at multiples of four
-        float4 g = *reinterpret_cast<const float4*>(v.dwpart + i);
-        for (int s = 1; s < splits; ++s) {
-            const float4 x = *reinterpret_cast<const float4*>(v.dwpart + (size_t)s * kDwStride + i);
-            g.x += x.x;
-            g.y += x.y;
-            g.z += x.z;
-            g.w += x.w;
-        }
+        const float4 g = *reinterpret_cast<const float4*>(v.grad + i);
         float4 w = *reinterpret_cast<const float4*>(v.master + i), m = *reinterpret_cast<const float4*>(v.m + i);
         float4 u = *reinterpret_cast<const float4*>(v.v + i);
         w.x = adamw_one(w.x, m.x, u.x, g.x, false, a);
         w.y = adamw_one(w.y, m.y, u.y, g.y, false, a);
         w.z = adamw_one(w.z, m.z, u.z, g.z, false, a);
         w.w = adamw_one(w.w, m.w, u.w, g.w, false, a);
-        *reinterpret_cast<float4*>(v.grad + i) = g;
         *reinterpret_cast<float4*>(v.master + i) = w;
         *reinterpret_cast<float4*>(v.m + i) = m;
         *reinterpret_cast<float4*>(v.v + i) = u;
@@ -518,31 +411,47 @@ cudaError_t gemm_back(const __nv_bfloat16* dZn, int K, const __nv_bfloat16* Wn, 
     return launch_gemm<256, true, true>(a, st);
 }
 
-// Weight gradients of all four layers into v->dwpart, in `splits` row splits.
-cudaError_t gemm_dw(dvc_value_net* v, int npad, int32_t* flags, int& splits, cudaStream_t st) {
+// Weight gradients of all four layers into v->grad.
+cudaError_t gemm_dw(dvc_value_net* v, int npad, int32_t* flags, cudaStream_t st) {
     DwArgs a{};
     const __nv_bfloat16* A[4] = {v->dZ[0], v->dZ[1], v->dZ[2], v->H3};
     const __nv_bfloat16* B[4] = {v->X, v->H1, v->H2, v->dZ4};
-    const int wa[4] = {VH, VH, VH, VH}, wb[4] = {VF, VH, VH, 64};
+    const int wb[4] = {VF, VH, VH, 64};
     const size_t off[4] = {OFF_W1, OFF_W2, OFF_W3, OFF_W4};
     int first = 0;
     for (int q = 0; q < 4; ++q) {
-        if (!encode_kmajor(&a.a[q], A[q], npad, wa[q], 64) || !encode_kmajor(&a.b[q], B[q], npad, wb[q], 64))
+        if (!encode_kmajor(&a.a[q], A[q], npad, VH, 64) || !encode_kmajor(&a.b[q], B[q], npad, wb[q], 64))
             return cudaErrorInvalidValue;
-        const int tn = std::max(1, wb[q] / 128);
-        a.p[q] = DwProblem{first, tn, wb[q], wb[q] >= 128 ? 2 : 1, q == 3 ? 1 : 0, off[q]};
-        first += wa[q] / 128 * tn;
+        a.p[q] = DwProblem{first, wb[q] / 64, wb[q], q == 3 ? 1 : 0, off[q]};
+        first += VH / 128 * (wb[q] / 64);
     }
-    a.ctas = first;
     a.nk = npad / 64;
-    splits = std::min(kDwSplits, a.nk);
-    a.splits = splits;
-    a.part = v->dwpart;
-    a.stride = kDwStride;
+    a.grad = v->grad;
     a.flags = flags;
     a.wait_ns = kGemmWaitNs;
-    gemm_dw_kernel<<<a.ctas * splits, kDwThreads, kDwSmem, st>>>(a);
+    gemm_dw_kernel<<<first, kDwThreads, kDwSmem, st>>>(a);
     return cudaGetLastError();
+}
+
+cudaError_t mlp_attributes() {
+    return cudaFuncSetAttribute(mlp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMlpSmem);
+}
+
+// Clusters of mlp_kernel that the device holds at once.
+cudaError_t mlp_clusters(int* out) {
+    cudaError_t e = mlp_attributes();
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kMlpCluster);
+    cfg.blockDim = dim3(kMlpThreads);
+    cfg.dynamicSmemBytes = kMlpSmem;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = kMlpCluster;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaOccupancyMaxActiveClusters(out, mlp_kernel, &cfg);
 }
 
 int net_alloc(dvc_ctx* c) {
@@ -561,17 +470,20 @@ int net_alloc(dvc_ctx* c) {
         c->vnet = v;
         return fail(c, DVC_E_OOM, "value network: parameter allocation");
     }
+    const cudaError_t e = mlp_clusters(&v->clusters);
+    if (e != cudaSuccess) v->clusters = 0;  // the layer-by-layer path serves every size
+    cudaGetLastError();
     c->vnet = v;
     return DVC_OK;
 }
 
 void free_work(dvc_value_net* v) {
     void* ptrs[] = {v->X, v->H1, v->H2, v->H3, v->dZ[0], v->dZ[1], v->dZ[2], v->dZ4,
-                    v->Z1, v->Z2, v->Z3, v->L, v->colsum, v->rowpart, v->dwpart};
+                    v->Z1, v->Z2, v->Z3, v->L, v->colsum, v->rowpart};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     v->X = v->H1 = v->H2 = v->H3 = v->dZ[0] = v->dZ[1] = v->dZ[2] = v->dZ4 = nullptr;
-    v->Z1 = v->Z2 = v->Z3 = v->L = v->colsum = v->rowpart = v->dwpart = nullptr;
+    v->Z1 = v->Z2 = v->Z3 = v->L = v->colsum = v->rowpart = nullptr;
     v->cap = 0;
 }
 
@@ -586,8 +498,7 @@ int ensure_work(dvc_ctx* c, int npad) {
                     al((void**)&v->dZ[1], r * VH * 2) && al((void**)&v->dZ[2], r * VH * 2) &&
                     al((void**)&v->dZ4, r * 64 * 2) && al((void**)&v->Z1, r * VH * 4) && al((void**)&v->Z2, r * VH * 4) &&
                     al((void**)&v->Z3, r * VH * 4) && al((void**)&v->L, r * kLogitFloats * 4) &&
-                    al((void**)&v->colsum, 3 * (r / 32) * VH * 4) && al((void**)&v->rowpart, r / kLossThreads * 8 * 4) &&
-                    al((void**)&v->dwpart, (size_t)kDwSplits * kDwStride * 4);
+                    al((void**)&v->colsum, 3 * (r / 32) * VH * 4) && al((void**)&v->rowpart, r / kLossThreads * 8 * 4);
     if (!ok) {
         cudaGetLastError();
         free_work(v);
@@ -628,7 +539,7 @@ int forward_into(dvc_ctx* c, const dvc_state* states, int n, int npad, __nv_bflo
     int32_t* fl = c->d_flags;
     // inference (head folded in): X, H1 and H2 in the K-blocked layout; training keeps them row-major
     const bool kb = head;
-    features_kernel<<<(npad + 255) / 256, 256, 0, st>>>(states, n, npad, X, nullptr, kb ? 1 : 0);
+    features_kernel<<<(npad + kFeatRows - 1) / kFeatRows, kFeatThreads, 0, st>>>(states, n, npad, X, nullptr, kb ? 1 : 0);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = gemm(X, v->W1, v->master + OFF_B1, H1, Z1, npad, VH, VF, kActGelu, fl, st, kb, kb);
     if (e == cudaSuccess) e = gemm(H1, v->W2, v->master + OFF_B2, H2, Z2, npad, VH, VH, kActGelu, fl, st, kb, kb);
@@ -642,10 +553,31 @@ int forward_into(dvc_ctx* c, const dvc_state* states, int n, int npad, __nv_bflo
     return DVC_OK;
 }
 
-int forward(dvc_ctx* c, const dvc_state* states, int n, int npad, bool train, cudaStream_t st) {
+// Win probabilities of n leaves, activations in the given buffers (npad rows).
+// One launch of clusters (dvc_mlp.cuh) while its 128-row tiles run at once: 28.9
+// us for 128 rows, 30.8 for 3,000, against 45 us layer by layer up to 7,000 rows;
+// a second wave would take 57 us (4,864 rows), and the layers use a full chip
+// better (65,536 rows: 148 us against 418).
+int infer(dvc_ctx* c, const dvc_state* states, int n, int npad, __nv_bfloat16* X, __nv_bfloat16* H1, __nv_bfloat16* H2,
+          float* L, float* probs, cudaStream_t st) {
     dvc_value_net* v = c->vnet;
-    return forward_into(c, states, n, npad, v->X, v->H1, v->H2, v->H3, v->L, train ? v->Z1 : nullptr,
-                        train ? v->Z2 : nullptr, train ? v->Z3 : nullptr, !train, st);
+    if (npad / 128 <= v->clusters) {
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        cudaError_t e = cudaStreamIsCapturing(st, &cs);
+        if (e == cudaSuccess && cs == cudaStreamCaptureStatusNone) e = mlp_attributes();
+        CUtensorMap w1, w2, w3;
+        if (e == cudaSuccess && (!encode_kmajor(&w1, v->W1, VH, VF, kMlpCols) || !encode_kmajor(&w2, v->W2, VH, VH, kMlpCols) ||
+                                 !encode_kmajor(&w3, v->W3, VH, VH, kMlpCols)))
+            e = cudaErrorInvalidValue;
+        if (e != cudaSuccess) return cuda_fail(c, e, "value network");
+        const MlpArgs a{{v->master + OFF_B1, v->master + OFF_B2, v->master + OFF_B3}, v->W4, v->b4p, states, n,
+                        probs, c->d_flags, kGemmWaitNs};
+        mlp_kernel<<<npad / 128 * kMlpCluster, kMlpThreads, kMlpSmem, st>>>(w1, w2, w3, a);
+        return check_launch(c, "mlp_kernel");
+    }
+    if (int rc = forward_into(c, states, n, npad, X, H1, H2, nullptr, L, nullptr, nullptr, nullptr, true, st)) return rc;
+    softmax_head_kernel<<<(n + 127) / 128, 128, 0, st>>>(L, v->b4p, states, n, probs);
+    return check_launch(c, "softmax_head_kernel");
 }
 
 int check_states_args(dvc_ctx* c, const void* d_states, int n) {
@@ -697,7 +629,7 @@ int dvc_value_features(dvc_ctx* c, const dvc_state* d_states, int n, float* d_ou
     if (n == 0) return DVC_OK;
     if (!is_device_ptr(d_out, c->device)) return fail(c, DVC_E_INVALID, "dvc_value_features: d_out must be device memory");
     if (int rc = set_device(c)) return rc;
-    features_kernel<<<(n + 255) / 256, 256, 0, (cudaStream_t)stream>>>(d_states, n, n, nullptr, d_out, 0);
+    features_kernel<<<(n + kFeatRows - 1) / kFeatRows, kFeatThreads, 0, (cudaStream_t)stream>>>(d_states, n, n, nullptr, d_out, 0);
     return check_launch(c, "features_kernel");
 }
 
@@ -711,9 +643,8 @@ int dvc_value_eval(dvc_ctx* c, const dvc_state* d_leaves, int n, float* d_winpro
     const int npad = (n + 127) / 128 * 128;
     if (int rc = ensure_work(c, npad)) return rc;
     cudaStream_t st = (cudaStream_t)stream;
-    if (int rc = forward(c, d_leaves, n, npad, false, st)) return rc;
-    softmax_head_kernel<<<(n + 127) / 128, 128, 0, st>>>(c->vnet->L, c->vnet->b4p, d_leaves, n, d_winprob);
-    return check_launch(c, "softmax_head_kernel");
+    dvc_value_net* v = c->vnet;
+    return infer(c, d_leaves, n, npad, v->X, v->H1, v->H2, v->L, d_winprob, st);
 }
 
 int dvc_value_train_step(dvc_ctx* c, const dvc_state* d_states, const float* d_labels, int n, float lr, float* d_loss,
@@ -730,7 +661,8 @@ int dvc_value_train_step(dvc_ctx* c, const dvc_state* d_states, const float* d_l
     cudaStream_t st = (cudaStream_t)stream;
     dvc_value_net* v = c->vnet;
     int32_t* fl = c->d_flags;
-    if (int rc = forward(c, d_states, n, npad, true, st)) return rc;
+    if (int rc = forward_into(c, d_states, n, npad, v->X, v->H1, v->H2, v->H3, v->L, v->Z1, v->Z2, v->Z3, false, st))
+        return rc;
     loss_grad_kernel<<<npad / kLossThreads, kLossThreads, 0, st>>>(v->L, d_states, d_labels, n, npad, v->dZ4,
                                                                   v->rowpart);
     if (int rc = check_launch(c, "loss_grad_kernel")) return rc;
@@ -740,14 +672,13 @@ int dvc_value_train_step(dvc_ctx* c, const dvc_state* d_states, const float* d_l
     if (e == cudaSuccess)
         e = gemm_back(v->dZ[2], VH, v->W3, v->Z2, v->dZ[1], v->colsum + blocks, npad, fl, st);
     if (e == cudaSuccess) e = gemm_back(v->dZ[1], VH, v->W2, v->Z1, v->dZ[0], v->colsum, npad, fl, st);
-    int splits = 1;
-    if (e == cudaSuccess) e = gemm_dw(v, npad, fl, splits, st);
+    if (e == cudaSuccess) e = gemm_dw(v, npad, fl, st);
     if (e != cudaSuccess) return cuda_fail(c, e, "value backward");
     v->step += 1;
     AdamCoef a{lr, 0.9f, 0.999f, 1e-8f, 1e-4f, 0.0f, 0.0f};
     a.c1 = 1.0f - powf(a.b1, (float)v->step);
     a.c2 = 1.0f - powf(a.b2, (float)v->step);
-    adamw_kernel<<<kAdamGrid, kAdamThreads, 0, st>>>(*v, splits, npad / 32, npad / kLossThreads, n, a, d_loss);
+    adamw_kernel<<<kAdamGrid, kAdamThreads, 0, st>>>(*v, npad / 32, npad / kLossThreads, n, a, d_loss);
     return check_launch(c, "adamw_kernel");
 }
 
@@ -849,15 +780,6 @@ int dvc_gemm_bf16(dvc_ctx* c, const void* d_A, const void* d_B, const float* d_b
 
 }  // extern "C"
 
-int dvc_value_forward_probs(dvc_ctx* c, const dvc_state* d_leaves, int n, float* d_probs, cudaStream_t st) {
-    if (int rc = need_net(c)) return rc;
-    const int npad = (n + 127) / 128 * 128;
-    if (int rc = ensure_work(c, npad)) return rc;
-    if (int rc = forward(c, d_leaves, n, npad, false, st)) return rc;
-    softmax_head_kernel<<<(n + 127) / 128, 128, 0, st>>>(c->vnet->L, c->vnet->b4p, d_leaves, n, d_probs);
-    return check_launch(c, "softmax_head_kernel");
-}
-
 int dvc_value_rows_alloc(dvc_ctx* c, dvc_value_rows* r, int rows) {
     dvc_value_rows_free(r);
     const size_t n = (size_t)rows;
@@ -887,6 +809,7 @@ int dvc_value_prepare(dvc_ctx* c) {
     if (e == cudaSuccess) e = gemm_attributes<64>();
     if (e == cudaSuccess) e = gemm_attributes<32>();
     if (e == cudaSuccess) e = gemm_attributes<16>();
+    if (e == cudaSuccess) e = mlp_attributes();
     return e == cudaSuccess ? DVC_OK : cuda_fail(c, e, "value network attributes");
 }
 
@@ -896,13 +819,8 @@ int dvc_value_forward_rows(dvc_ctx* c, const dvc_state* d_leaves, int n, dvc_val
     const int npad = (n + 127) / 128 * 128;
     if (row0 < 0 || row0 + npad > r->rows) return fail(c, DVC_E_INVALID, "value network: activation rows");
     const size_t o = (size_t)row0;
-    float* L = r->L + o * kLogitFloats;
-    if (int rc = forward_into(c, d_leaves, n, npad, (__nv_bfloat16*)r->X + o * VF, (__nv_bfloat16*)r->H1 + o * VH,
-                              (__nv_bfloat16*)r->H2 + o * VH, (__nv_bfloat16*)r->H3 + o * VH, L, nullptr, nullptr,
-                              nullptr, true, st))
-        return rc;
-    softmax_head_kernel<<<(n + 127) / 128, 128, 0, st>>>(L, c->vnet->b4p, d_leaves, n, d_probs);
-    return check_launch(c, "softmax_head_kernel");
+    return infer(c, d_leaves, n, npad, (__nv_bfloat16*)r->X + o * VF, (__nv_bfloat16*)r->H1 + o * VH,
+                 (__nv_bfloat16*)r->H2 + o * VH, r->L + o * kLogitFloats, d_probs, st);
 }
 
 void dvc_value_free(dvc_ctx* c) {
