@@ -358,10 +358,10 @@ __global__ void mcts_select_kernel(ForestDev F, SearchParams sp, int n, Descent*
     Descent dd;
     TreeWords tw;
     tw.open(sp.seed, tm.tree_id, (uint32_t)tm.done);
-    tw.b0 = tw.block(0u);
+    tw.b = tw.block(0u);
     const Node* nodes = F.nodes + tm.node_off;
     const Node r = nodes[0];
-    descend(det, root.cur, WalkNode{0, r.child, r.meta >> 12, F.csl[tm.node_off]}, nodes, F.link + tm.node_off,
+    descend<true>(det, root.cur, WalkNode{0, r.child, r.meta >> 12, F.csl[tm.node_off]}, nodes, F.link + tm.node_off,
             F.ucb + tm.node_off, F.csl + tm.node_off, sp, tw, paths + (size_t)t * kPathMax,
             movers + (size_t)t * kPathMax, s_E[wl], dd, set_table(F, tm));
     if (lane == 0) d = dd;
@@ -389,7 +389,7 @@ __global__ void mcts_expand_kernel(ForestDev F, int n, Descent* work, int32_t* p
     int32_t used = tm.used;
     bool ok = true;
     if (d.found)
-        ok = expand_child(d, F.nodes + tm.node_off, F.link + tm.node_off, F.created + tm.node_off, tm, next_free, used,
+        ok = expand_child<true>(d, F.nodes + tm.node_off, F.link + tm.node_off, F.created + tm.node_off, tm, next_free, used,
                           (uint32_t)tm.done, paths + (size_t)t * kPathMax, movers + (size_t)t * kPathMax,
                           set_table(F, tm));
     if (lane == 0) {
@@ -977,9 +977,13 @@ int dvc_forest_create(dvc_ctx* c, int n, const dvc_state* d_roots, const int32_t
     // slot (CTAs hold trees_per_cta trees): balances uneven forests.
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
-    // enough trees to fill the GPU: the pipeline; small forests: the fused
-    // lockstep kernel
-    f->engine = n > 4 * std::max(sms, 1) ? 2 : 1;
+    // small forests: the fused lockstep kernel; enough playouts per iteration to
+    // fill the GPU: the pipeline.  The line lies where both take the same time per
+    // iteration (us, fused / pipeline): 32 playouts, 2,400 trees 15.4 / 19.6 (two
+    // players) and 23.0 / 29.4 (four), 4,096 trees 28.4 / 26.0 and 43.2 / 38.9; one
+    // playout, 2,400 trees 10.3 / 15.9, 8,192 34 / 30; 128 playouts, 600 trees 13.7 /
+    // 18.3, 1,200 22.6 / 21.6; 256 playouts, 600 trees 22.5 / 21.9.
+    f->engine = (long long)n * std::max(c->cfg.playouts, 32) > 640LL * std::max(sms, 1) ? 2 : 1;
     default_shape(n, sms, f->engine, c->cfg.playouts, f->trees_per_cta, f->warps_per_cta, f->chains);
     std::vector<int32_t> order(n);
     {
@@ -1139,31 +1143,35 @@ int launch_fused(dvc_forest* f, int n_iterations, cudaStream_t st) {
     const int threads = 32 * W;
     const bool fast2 = c->cfg.nplayers == 2 && c->cfg.ntiles == 24;
     cudaError_t e;
-#define DVC_LAUNCH_POOL(MT, F2, ORD)                                                                              \
+#define DVC_LAUNCH_POOL(MT, F2, ORD, VAN)                                                                         \
     do {                                                                                                          \
-        e = cudaFuncSetAttribute(mcts_pool_kernel<MT, F2, ORD>, cudaFuncAttributeMaxDynamicSharedMemorySize,      \
+        e = cudaFuncSetAttribute(mcts_pool_kernel<MT, F2, ORD, VAN>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
                                  (int)L.bytes);                                                                   \
         if (e == cudaSuccess)                                                                                     \
-            mcts_pool_kernel<MT, F2, ORD><<<grid, threads, L.bytes, st>>>(dev_of(f), params_of(f), n_iterations,  \
-                                                                          f->order, f->n, T, f->pipe.det,         \
-                                                                          f->pipe.tree0);                         \
+            mcts_pool_kernel<MT, F2, ORD, VAN><<<grid, threads, L.bytes, st>>>(                                   \
+                dev_of(f), params_of(f), n_iterations, f->order, f->n, T, f->pipe.det, f->pipe.tree0);            \
     } while (0)
-    if (c->cfg.policy && threads <= 512) {  // ordering-aware playouts
-        if (fast2) DVC_LAUNCH_POOL(512, true, true);
-        else DVC_LAUNCH_POOL(512, false, true);
-    } else if (c->cfg.policy) {
-        if (fast2) DVC_LAUNCH_POOL(1024, true, true);
-        else DVC_LAUNCH_POOL(1024, false, true);
+#define DVC_LAUNCH_POOL2(MT, ORD, VAN)                 \
+    do {                                               \
+        if (fast2) DVC_LAUNCH_POOL(MT, true, ORD, VAN); \
+        else DVC_LAUNCH_POOL(MT, false, ORD, VAN);     \
+    } while (0)
+    if (c->cfg.policy) {  // ordering-aware playouts
+        if (threads <= 512) DVC_LAUNCH_POOL2(512, true, true);
+        else DVC_LAUNCH_POOL2(1024, true, true);
+    } else if (c->cfg.vanilla) {
+        if (threads <= 512) DVC_LAUNCH_POOL2(512, false, true);
+        else DVC_LAUNCH_POOL2(1024, false, true);
+    } else if (threads <= 128) {
+        DVC_LAUNCH_POOL2(128, false, false);
     } else if (threads <= 512) {
-        if (fast2) DVC_LAUNCH_POOL(512, true, false);
-        else DVC_LAUNCH_POOL(512, false, false);
+        DVC_LAUNCH_POOL2(512, false, false);
     } else if (threads <= 768) {
-        if (fast2) DVC_LAUNCH_POOL(768, true, false);
-        else DVC_LAUNCH_POOL(768, false, false);
+        DVC_LAUNCH_POOL2(768, false, false);
     } else {
-        if (fast2) DVC_LAUNCH_POOL(1024, true, false);
-        else DVC_LAUNCH_POOL(1024, false, false);
+        DVC_LAUNCH_POOL2(1024, false, false);
     }
+#undef DVC_LAUNCH_POOL2
 #undef DVC_LAUNCH_POOL
     if (e != cudaSuccess) return cuda_fail(c, e, "mcts_pool_kernel attributes");
     return check_launch(c, "mcts_pool_kernel");

@@ -136,15 +136,15 @@ __global__ void __launch_bounds__(128)
     Descent d;
     TreeWords tw;
     tw.open(sp.seed, tm.tree_id, it);
-    tw.b0 = tree0;
+    tw.b = tree0;
     const SetTable st = VANILLA ? set_table(F, tm) : SetTable{nullptr, nullptr, 0u};
     // the determinization leaves the seat to move, who is the observer
-    descend(det, det.cur, WalkNode{0, root.child, root.meta >> 12, csl[0]}, nodes, link, ucb, csl, sp, tw, path, mover,
+    descend<VANILLA>(det, det.cur, WalkNode{0, root.child, root.meta >> 12, csl[0]}, nodes, link, ucb, csl, sp, tw, path, mover,
             s_E[wl], d, st);
     bool ok = true;
     int32_t next_free = tm.next_free, used = tm.used;
     if (d.found)
-        ok = expand_child(d, nodes, link, F.created + tm.node_off, tm, next_free, used, it, path, mover, st);
+        ok = expand_child<VANILLA>(d, nodes, link, F.created + tm.node_off, tm, next_free, used, it, path, mover, st);
     if (lane == 0) {
         tmr.done = done;
         tmr.next_free = next_free;

@@ -77,8 +77,9 @@ struct PoolLayout {
 // det_ahead / tree0_ahead: kDetAhead determinized roots and first in-tree
 // stream blocks per tree (the forest's pipeline buffers; rewritten at the
 // start of every launch).
-template <int MAXT, bool FAST2, bool ORD = false>
-__global__ void __launch_bounds__(MAXT, 1)
+// VANILLA: the trees have a plausible-set layer.
+template <int MAXT, bool FAST2, bool ORD, bool VANILLA>
+__global__ void __launch_bounds__(MAXT, MAXT == 128 ? 4 : 1)
     mcts_pool_kernel(ForestDev F, SearchParams sp, int n_iter, const int32_t* order, int n_trees, int T,
                      dvc_state* det_ahead, uint4* tree0_ahead) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -162,19 +163,19 @@ __global__ void __launch_bounds__(MAXT, 1)
             const G det = load_state(det_ahead[a]);
             TreeWords tw;
             tw.open(sp.seed, tm.tree_id, it);
-            tw.b0 = tree0_ahead[a];
+            tw.b = tree0_ahead[a];
             const Node root = nodes[0];
             Descent d;
             int32_t* path = s_path + s * kPathMax;
             uint8_t* mover = s_mover + s * kPathMax;
-            const SetTable st = set_table(F, tm);
+            const SetTable st = VANILLA ? set_table(F, tm) : SetTable{nullptr, nullptr, 0u};
             // the determinization leaves the seat to move, who is the observer
-            descend(det, det.cur, WalkNode{0, root.child, root.meta >> 12, F.csl[tm.node_off]}, nodes, link,
+            descend<VANILLA>(det, det.cur, WalkNode{0, root.child, root.meta >> 12, F.csl[tm.node_off]}, nodes, link,
                     F.ucb + tm.node_off, F.csl + tm.node_off, sp, tw, path, mover, s_E + warp * 104u, d, st);
             bool ok = true;
             if (d.found) {
                 int32_t next_free = tm.next_free, used = tm.used;
-                ok = expand_child(d, nodes, link, created, tm, next_free, used, it, path, mover, st);
+                ok = expand_child<VANILLA>(d, nodes, link, created, tm, next_free, used, it, path, mover, st);
                 if (lane == 0) {
                     tm.next_free = next_free;
                     tm.used = used;

@@ -173,19 +173,18 @@ __device__ __forceinline__ int32_t block_dir(const int32_t* link, int32_t blk0, 
     return dir;
 }
 
-// The words of an iteration's tree stream (tag 3), the same on every lane:
-// block 0 is given (b0, sampled ahead or block(0)); the blocks after it are
-// computed at the first need, one per lane.
+// The words of an iteration's tree stream (tag 3), the same on every lane.
+// b holds the block the next word is in; block 0 is given, as sampled ahead or by
+// block(0).
 struct TreeWords {
     uint32_t k0, k1, i, tw;
-    uint4 b0, more;  // block 0; this lane's block 1 + lane
+    uint4 b;
     uint32_t used;
-    bool ahead;
 
     __device__ __forceinline__ uint4 block(uint32_t blk) const {
-        uint32_t a = blk, b = 0u, c = i, d = tw;
-        philox10(a, b, c, d, k0, k1);
-        return make_uint4(a, b, c, d);
+        uint32_t x0 = blk, x1 = 0u, x2 = i, x3 = tw;
+        philox10(x0, x1, x2, x3, k0, k1);
+        return make_uint4(x0, x1, x2, x3);
     }
     __device__ __forceinline__ void open(uint64_t seed, uint32_t tree, uint32_t it) {
         k0 = (uint32_t)seed;
@@ -193,21 +192,11 @@ struct TreeWords {
         i = it;
         tw = kTagTree + 16u * (uint32_t)(seed >> 32);
         used = 0u;
-        ahead = false;
-    }
-    // Make the next two words (the most a ply takes) available.
-    __device__ __forceinline__ void ensure() {
-        if (used > 2u && !ahead) {
-            more = block(1u + (threadIdx.x & 31u));
-            ahead = true;
-        }
     }
     __device__ __forceinline__ uint32_t next() {
         const uint32_t n = used++, k = n & 3u;
-        const uint4 q = n < 4u ? b0 : more;
-        const uint32_t v = k == 0u ? q.x : k == 1u ? q.y : k == 2u ? q.z : q.w;
-        // at most two words per ply and at most kPathMax plies: 32 blocks suffice
-        return n < 4u ? v : __shfl_sync(0xFFFFFFFFu, v, (n - 4u) >> 2);
+        if (k == 0u && n) b = block(n >> 2);
+        return k == 0u ? b.x : k == 1u ? b.y : k == 2u ? b.z : b.w;
     }
 };
 
@@ -250,7 +239,6 @@ __device__ __forceinline__ void warp_apply(G& g, const Rows& v, uint32_t code, T
         g.drawn = kNone;
         return;
     }
-    tw.ensure();
     const uint32_t n = __umulhi(tw.next(), __popc(pool));
     const bool here = ((pool >> lane) & 1u) && (uint32_t)__popc(pool & ((1u << lane) - 1u)) == n;
     const uint32_t t = (uint32_t)__ffs(__ballot_sync(0xFFFFFFFFu, here)) - 1u;
@@ -290,9 +278,10 @@ struct WalkNode {
 // node's UCB1 terms, refreshed whenever its counts change (backprop), so a
 // selection scan costs one multiply-add per child.  They are the same IEEE
 // values a scan would compute from the counts.
-// st: the plausible-set table of a vanilla tree.  The determinization's set
+// VANILLA: st is the tree's plausible-set table.  The determinization's set
 // node is the first step below the root; a set not seen before is this
 // iteration's expansion (act = kSet) and its leaf is the determinized root.
+template <bool VANILLA>
 __device__ __forceinline__ void descend(const G& det, uint32_t obs, WalkNode at, const Node* nodes,
                                         const int32_t* link, const float2* ucb, const float* csl_of,
                                         const SearchParams& sp, TreeWords& tw, int32_t* path, uint8_t* mover,
@@ -307,7 +296,7 @@ __device__ __forceinline__ void descend(const G& det, uint32_t obs, WalkNode at,
         mover[0] = (uint8_t)obs;
     }
     uint32_t depth = 0;
-    if (st.cells) {
+    if (VANILLA && st.cells) {
         const uint4 key = set_key(d.s, obs);
         uint32_t cell;
         const int32_t slot = set_find(st, key, cell);
@@ -372,7 +361,7 @@ __device__ __forceinline__ void descend(const G& det, uint32_t obs, WalkNode at,
             // two chunks of 32 children in flight
             uint32_t seen = 0u;
             for (uint32_t c0 = 0; c0 < at.nchild; c0 += 64u) {
-                Node ch[2];
+                int2 ch[2];  // first child block, meta
                 float2 u[2];
                 float cs[2];
                 int32_t sl[2];
@@ -384,7 +373,7 @@ __device__ __forceinline__ void descend(const G& det, uint32_t obs, WalkNode at,
                         const int32_t s = place(c);
                         if (c < at.nchild) {
                             sl[h] = s;
-                            ch[h] = nodes[s];
+                            ch[h] = reinterpret_cast<const int2*>(nodes + s)[1];
                             u[h] = ucb[s];  // set by the child's first backprop
                             cs[h] = csl_of[s];
                         }
@@ -393,7 +382,7 @@ __device__ __forceinline__ void descend(const G& det, uint32_t obs, WalkNode at,
 #pragma unroll
                 for (uint32_t h = 0; h < 2u; ++h) {
                     if (sl[h] < 0) continue;
-                    const uint32_t code = ch[h].meta & 0xFFFu;
+                    const uint32_t code = (uint32_t)ch[h].y & 0xFFFu;
                     const uint32_t q = code >> 10, x = code & 31u;
                     const uint32_t off = q > cur ? q - cur - 1u : q + np - cur - 1u;
                     const uint32_t m = off == 0u ? m1 : off == 1u ? m2 : m3;
@@ -410,8 +399,8 @@ __device__ __forceinline__ void descend(const G& det, uint32_t obs, WalkNode at,
                         best_sc = sc;
                         best_rank = rank;
                         best_slot = sl[h];
-                        best_meta = ch[h].meta;
-                        best_blk = ch[h].child;
+                        best_meta = (uint32_t)ch[h].y;
+                        best_blk = ch[h].x;
                         best_csl = cs[h];
                     }
                 }
@@ -486,6 +475,7 @@ __device__ __forceinline__ void descend(const G& det, uint32_t obs, WalkNode at,
 // tree's set table).  Lane-uniform; lane 0 writes memory.  next_free is the
 // tree's allocator (uniform register copy).  Returns false if the arena is
 // exhausted.
+template <bool VANILLA>
 __device__ __forceinline__ bool expand_child(Descent& d, Node* nodes, int32_t* link, int32_t* created,
                                              const TreeMeta& tm, int32_t& next_free, int32_t& used, uint32_t it,
                                              int32_t* path, uint8_t* mover,
@@ -521,7 +511,7 @@ __device__ __forceinline__ bool expand_child(Descent& d, Node* nodes, int32_t* l
         nodes[d.node].meta += 1u << 12;
         path[d.np] = slot;
         mover[d.np] = (uint8_t)d.who;
-        if (d.act == kSet) {
+        if (VANILLA && d.act == kSet) {
             st.key[d.set_cell] = d.set_key;
             st.slot[d.set_cell] = slot;
         }
