@@ -266,8 +266,8 @@ int dvc_mcts_step(dvc_forest* f, int n_iterations, int mode, void* stream);
  * lane compaction a group's playouts are pooled in one CTA of warps_per_cta
  * warps.  The determinizations of the graph's 64 iterations are sampled
  * up front, one thread per tree and iteration.  engine 0 keeps the current
- * engine (the default is 1 while trees x max(playouts, 32) is at most 640 per SM,
- * else 2).
+ * engine (the default is 1 while trees x max(playouts, 16) is at most 512 per SM,
+ * with the ordering-aware policy trees x max(playouts, 128); else 2).
  * trees_per_cta, warps_per_cta, chains 0 = the engine's defaults (fused:
  * ceil(n_trees / SMs) trees, at most 32, and a warp per tree or one playout
  * per thread, whichever is more, up to 16 warps;

@@ -40,7 +40,9 @@ void default_shape(int n, int sms, int engine, int P, int& T, int& W, int& chain
         // a warp per tree, and enough warps for one playout per thread (16 at most)
         T = std::max(1, std::min(32, (n + S - 1) / S));
         W = std::min(16, std::max(T, (T * std::max(P, 1) + 31) / 32));
-        chains = 1;
+        // for value mode alone: one chain up to 16 trees per SM (2,432 trees 37.3 us
+        // per iteration against 38.5 with eight; 4,864 trees 48.6 against 44.8)
+        chains = n <= 16 * S ? 1 : std::max(1, std::min(24, (int)std::lround(n / (1.12 * S))));
     }
 }
 }  // namespace
@@ -977,13 +979,16 @@ int dvc_forest_create(dvc_ctx* c, int n, const dvc_state* d_roots, const int32_t
     // slot (CTAs hold trees_per_cta trees): balances uneven forests.
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
-    // small forests: the fused lockstep kernel; enough playouts per iteration to
-    // fill the GPU: the pipeline.  The line lies where both take the same time per
-    // iteration (us, fused / pipeline): 32 playouts, 2,400 trees 15.4 / 19.6 (two
-    // players) and 23.0 / 29.4 (four), 4,096 trees 28.4 / 26.0 and 43.2 / 38.9; one
-    // playout, 2,400 trees 10.3 / 15.9, 8,192 34 / 30; 128 playouts, 600 trees 13.7 /
-    // 18.3, 1,200 22.6 / 21.6; 256 playouts, 600 trees 22.5 / 21.9.
-    f->engine = (long long)n * std::max(c->cfg.playouts, 32) > 640LL * std::max(sms, 1) ? 2 : 1;
+    // The fused lockstep kernel while an SM has at most one playout per thread (512)
+    // and two trees per warp (32), else the pipeline: past that its CTAs take a
+    // second pass over playouts, or run in a second wave.  Time per iteration (us,
+    // fused / pipeline, two players then four): 32 playouts, 2,432 trees 15.0 / 19.1
+    // and 22.7 / 29.1, 2,800 trees 22.4 / 20.1 and 35.0 / 30.9; 100 playouts, 760
+    // trees 12.8 / 17.8 and 20.3 / 25.0; one playout, 4,864 trees 15.6 / 21.1 and
+    // 23.3 / 28.1.  Ordering-aware games differ most in length, and the step waits
+    // for a CTA's longest one: from four trees per SM on they go to the pipeline
+    // (four players, one playout, 1,200 trees 134 / 134, 2,432 trees 174 / 146).
+    f->engine = (long long)n * std::max(c->cfg.playouts, c->cfg.policy ? 128 : 16) > 512LL * std::max(sms, 1) ? 2 : 1;
     default_shape(n, sms, f->engine, c->cfg.playouts, f->trees_per_cta, f->warps_per_cta, f->chains);
     std::vector<int32_t> order(n);
     {
