@@ -57,6 +57,8 @@ struct dvc_forest {
     DetPlan* plans;
     unsigned long long* tables;
     Node* nodes;
+    float2* terms;  // UCB1 terms by visits (SearchParams::terms)
+    int n_terms;
     int32_t* link;
     int32_t* created;
     long long total_slots;
@@ -363,7 +365,7 @@ __global__ void mcts_select_kernel(ForestDev F, SearchParams sp, int n, Descent*
     tw.b = tw.block(0u);
     const Node* nodes = F.nodes + tm.node_off;
     const Node r = nodes[0];
-    descend<true>(det, root.cur, WalkNode{0, r.child, r.meta >> 12, F.csl[tm.node_off]}, nodes, F.link + tm.node_off,
+    descend<true>(det, root.cur, WalkNode{0, r.child, r.meta, F.csl[tm.node_off]}, nodes, F.link + tm.node_off,
             F.ucb + tm.node_off, F.csl + tm.node_off, sp, tw, paths + (size_t)t * kPathMax,
             movers + (size_t)t * kPathMax, s_E[wl], dd, set_table(F, tm));
     if (lane == 0) d = dd;
@@ -390,6 +392,8 @@ __global__ void mcts_expand_kernel(ForestDev F, int n, Descent* work, int32_t* p
     int32_t next_free = tm.next_free;
     int32_t used = tm.used;
     bool ok = true;
+    if (d.found)  // the walk was another launch's: its block directory again
+        d.dir = d.node != 0 && d.meta >> 12 ? block_dir(F.link + tm.node_off, d.blk, d.meta >> 12) : d.blk;
     if (d.found)
         ok = expand_child<true>(d, F.nodes + tm.node_off, F.link + tm.node_off, F.created + tm.node_off, tm, next_free, used,
                           (uint32_t)tm.done, paths + (size_t)t * kPathMax, movers + (size_t)t * kPathMax,
@@ -420,9 +424,15 @@ __global__ void mcts_backprop_kernel(ForestDev F, SearchParams sp, int n, const 
     if (d.np < 0) return;
     TreeMeta& tm = F.meta[t];
     backprop(F.nodes + tm.node_off, F.ucb + tm.node_off, F.csl + tm.node_off, paths + (size_t)t * kPathMax,
-             movers + (size_t)t * kPathMax, d.np, wins + 4 * t, sp.playouts, sp.c_uct);
+             movers + (size_t)t * kPathMax, d.np, wins + 4 * t, sp);
     __syncwarp();
     if ((threadIdx.x & 31u) == 0) tm.done += 1;
+}
+
+// terms[k] = visit_terms of k * playouts visits, k = 1 .. n
+__global__ void visit_terms_kernel(float2* terms, int n, int playouts, float c_uct) {
+    const int k = (int)(blockIdx.x * blockDim.x + threadIdx.x) + 1;
+    if (k <= n) terms[k] = visit_terms(__int2float_rn(k * playouts), c_uct);
 }
 
 __global__ void root_stats_kernel(ForestDev F, int n, int32_t* out) {
@@ -734,6 +744,9 @@ SearchParams params_of(const dvc_forest* f) {
     sp.cont_thr = f->ctx->cfg.cont_thr;
     sp.policy = f->ctx->cfg.policy;
     sp.tree_continue = f->ctx->cfg.tree_continue;
+    sp.terms = f->terms;
+    sp.n_terms = f->n_terms;
+    sp.inv_playouts = 1.0f / (float)sp.playouts;
     return sp;
 }
 
@@ -933,7 +946,8 @@ void dvc_forest_destroy(dvc_forest* f) {
                     f->created,   f->work,      f->paths,     f->movers,         f->leaves,        f->leaf_tree,
                     f->leaf_iter, f->d_words,   f->export_scratch, f->order,     f->ucb,           f->csl,
                     f->pipe.leaf, f->pipe.path, f->pipe.mover, f->pipe.np,       f->pipe.wins,     f->pipe.step_end,
-                    f->pipe.det,  f->pipe.tree0, f->pipe.det_base, f->probs};
+                    f->pipe.det,  f->pipe.tree0, f->pipe.det_base, f->probs,
+                    f->terms};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     delete f;
@@ -1024,6 +1038,10 @@ int dvc_forest_create(dvc_ctx* c, int n, const dvc_state* d_roots, const int32_t
         if (even)
             for (int i = 0; i < n; ++i) order[i] = i;
     }
+    // no node is visited more often than the longest budget; the table stays below a
+    // megabyte, and visits past it are computed
+    f->n_terms = std::min({n ? *std::max_element(f->h_budgets.begin(), f->h_budgets.end()) : 0, 1 << 17,
+                           INT32_MAX / c->cfg.playouts});
     auto alloc = [&](void** p, size_t bytes) {
         if (cudaMalloc(p, bytes ? bytes : 16) != cudaSuccess) {
             cudaGetLastError();
@@ -1048,6 +1066,7 @@ int dvc_forest_create(dvc_ctx* c, int n, const dvc_state* d_roots, const int32_t
         alloc((void**)&f->pipe.det, sizeof(dvc_state) * kDetAhead * (size_t)n) &&
         alloc((void**)&f->pipe.tree0, sizeof(uint4) * kDetAhead * (size_t)n) &&
         alloc((void**)&f->pipe.det_base, sizeof(int32_t) * n) &&
+        alloc((void**)&f->terms, sizeof(float2) * (size_t)(f->n_terms + 1)) &&
         (!vanilla || (alloc((void**)&f->set_key, sizeof(uint4) * (size_t)cells) &&
                       alloc((void**)&f->set_slot, sizeof(int32_t) * (size_t)cells)));
     if (!ok) {
@@ -1064,6 +1083,14 @@ int dvc_forest_create(dvc_ctx* c, int n, const dvc_state* d_roots, const int32_t
     if (e != cudaSuccess) {
         dvc_forest_destroy(f);
         return cuda_fail(c, e, "dvc_forest_create copy");
+    }
+    if (f->n_terms > 0) {
+        visit_terms_kernel<<<(f->n_terms + 127) / 128, 128, 0, st>>>(f->terms, f->n_terms, c->cfg.playouts,
+                                                                     params_of(f).c_uct);
+        if (int rc = check_launch(c, "visit_terms_kernel")) {
+            dvc_forest_destroy(f);
+            return rc;
+        }
     }
     forest_init_kernel<<<(n * 32 + 127) / 128, 128, 0, st>>>(dev_of(f), n, nullptr, f->plans, f->tables, f->table_cap,
                                                             c->cfg.nplayers, c->cfg.ntiles, f->pipe.np);

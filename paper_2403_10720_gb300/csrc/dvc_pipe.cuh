@@ -45,7 +45,7 @@ __device__ __forceinline__ void pipe_apply_pending(ForestDev& F, const SearchPar
     TreeMeta& tm = F.meta[t];
     const long long off = tm.node_off;
     backprop(F.nodes + off, F.ucb + off, F.csl + off, P.path + (size_t)t * kPathMax, P.mover + (size_t)t * kPathMax,
-             np, P.wins + 4 * t, sp.playouts, sp.c_uct);
+             np, P.wins + 4 * t, sp);
     __syncwarp();
     if ((threadIdx.x & 31u) == 0) {
         tm.done += 1;
@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(128)
         tree0 = P.tree0[(size_t)t * kDetAhead + ahead];
     }
     if (pending >= 0) {
-        backprop(nodes, ucb, csl, path, mover, pending, P.wins + 4 * t, sp.playouts, sp.c_uct);
+        backprop(nodes, ucb, csl, path, mover, pending, P.wins + 4 * t, sp);
         __syncwarp();
     }
     if (!run || ahead >= (uint32_t)kDetAhead) {
@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(128)
     tw.b = tree0;
     const SetTable st = VANILLA ? set_table(F, tm) : SetTable{nullptr, nullptr, 0u};
     // the determinization leaves the seat to move, who is the observer
-    descend<VANILLA>(det, det.cur, WalkNode{0, root.child, root.meta >> 12, csl[0]}, nodes, link, ucb, csl, sp, tw, path, mover,
+    descend<VANILLA>(det, det.cur, WalkNode{0, root.child, root.meta, csl[0]}, nodes, link, ucb, csl, sp, tw, path, mover,
             s_E[wl], d, st);
     bool ok = true;
     int32_t next_free = tm.next_free, used = tm.used;

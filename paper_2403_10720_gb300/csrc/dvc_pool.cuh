@@ -63,10 +63,10 @@ struct PoolLayout {
         path = take(4u * kPathMax * T);
         mover = take((uint32_t)kPathMax * T);
         wins = take(16u * T);
-        misc = take(16u * T);  // per slot: np, end, tree index, 0
+        misc = take(16u * T);  // per slot: np, end, tree index; 4th words: the list of leaves to play
         base = take(4u * T);   // per slot: first iteration sampled ahead
         E = take(4u * 104u * W);
-        cnt = take(4u * 8u);   // [parity][nleaf, next, ntrees, 0]
+        cnt = take(4u * 2u);   // by parity: next game to hand out (ordering-aware policy)
         ring = take(kRingBytes * W);  // words of the playouts
         bytes = o;
     }
@@ -119,14 +119,13 @@ __global__ void __launch_bounds__(MAXT, MAXT == 128 ? 4 : 1)
             s_misc[4 * s + 2] = t;
         }
     }
-    if (tid < 8) s_cnt[tid] = 0;
+    if (tid < 2) s_cnt[tid] = 0;
     if constexpr (!ORD) fill_select<Game::kChunk>(s_sel, tid, blockDim.x);
     else if constexpr (FAST2) fill_select12(s_lut12, tid, blockDim.x);
     __syncthreads();
 
     uint32_t words = 0u, nsteps = 0u;  // per lane; summed in 64 bits per warp at the end
     for (int iter = 0;; ++iter) {
-        int32_t* cnt = s_cnt + 4 * (iter & 1);
         if (iter % kDetAhead == 0) {
             // ---- 0. the next kDetAhead determinizations of every running slot
             __syncthreads();
@@ -170,8 +169,8 @@ __global__ void __launch_bounds__(MAXT, MAXT == 128 ? 4 : 1)
             uint8_t* mover = s_mover + s * kPathMax;
             const SetTable st = VANILLA ? set_table(F, tm) : SetTable{nullptr, nullptr, 0u};
             // the determinization leaves the seat to move, who is the observer
-            descend<VANILLA>(det, det.cur, WalkNode{0, root.child, root.meta >> 12, F.csl[tm.node_off]}, nodes, link,
-                    F.ucb + tm.node_off, F.csl + tm.node_off, sp, tw, path, mover, s_E + warp * 104u, d, st);
+            descend<VANILLA>(det, det.cur, WalkNode{0, root.child, root.meta, F.csl[tm.node_off]}, nodes, link,
+                             F.ucb + tm.node_off, F.csl + tm.node_off, sp, tw, path, mover, s_E + warp * 104u, d, st);
             bool ok = true;
             if (d.found) {
                 int32_t next_free = tm.next_free, used = tm.used;
@@ -192,26 +191,29 @@ __global__ void __launch_bounds__(MAXT, MAXT == 128 ? 4 : 1)
                     int32_t* w = s_wins + 4 * s;
                     w[0] = w[1] = w[2] = w[3] = 0;
                     if (d.s.winner < 4u) w[d.s.winner] = sp.playouts;  // finished in the tree
-                    atomicAdd(&cnt[2], 1);
                 }
             }
         }
         __syncthreads();
-        if (cnt[2] == 0) break;
-        if (tid == 0) {
-            int32_t* other = s_cnt + 4 * ((iter + 1) & 1);
-            other[0] = other[1] = other[2] = 0;
-            // list of leaves that need playouts: slots with a fresh, unfinished leaf
-            int32_t n = 0;
-            for (int s = 0; s < nslot; ++s)
-                if (s_tm[s].done < s_misc[4 * s + 1] && s_leaf[s].winner == kNone) s_misc[4 * (n++) + 3] = s;
-            cnt[0] = n;
+        // the leaves that need playouts, slots with a fresh, unfinished one: every
+        // warp writes the same list
+        int nleaf = 0;
+        bool ran = false;
+        for (int s0 = 0; s0 < nslot; s0 += 32) {
+            const int s = s0 + (int)lane;
+            const bool fresh = s < nslot && s_tm[s].done < s_misc[4 * s + 1];
+            const unsigned open = __ballot_sync(0xFFFFFFFFu, fresh && s_leaf[s].winner == kNone);
+            ran |= __any_sync(0xFFFFFFFFu, fresh) != 0;
+            if ((open >> lane) & 1u) s_misc[4 * (nleaf + __popc(open & ((1u << lane) - 1u))) + 3] = s;
+            nleaf += __popc(open);
         }
-        __syncthreads();
+        if (!ran) break;
+        if (ORD && tid == 0) s_cnt[(iter + 1) & 1] = 0;
+        __syncwarp();
         // ---- 2. playout phase: P playouts of each listed leaf
         if constexpr (!ORD) {
             // 32 games at a time per warp, one per lane
-            const uint32_t P = (uint32_t)sp.playouts, total = (uint32_t)cnt[0] * P;
+            const uint32_t P = (uint32_t)sp.playouts, total = (uint32_t)nleaf * P;
             const uint32_t tab = shared_addr(s_sel);
             for (uint32_t first = warp * 32u; first < total; first += blockDim.x) {
                 Game g;
@@ -240,7 +242,7 @@ __global__ void __launch_bounds__(MAXT, MAXT == 128 ? 4 : 1)
         } else {
             // handed to lanes as they free up
             const int P = sp.playouts;
-            const int total = cnt[0] * P;
+            const int total = nleaf * P;
             int slot = 0, steps = 0;
             WordQueue r;
             // state of the lane's current game
@@ -266,7 +268,7 @@ __global__ void __launch_bounds__(MAXT, MAXT == 128 ? 4 : 1)
                 // own (the fast path counts it as an iteration of its loop)
                 steps = (!FAST2 && (ls.flags & 2u)) ? 1 : 0;
             };
-            int p = atomicAdd(&cnt[1], 1);
+            int p = atomicAdd(&s_cnt[iter & 1], 1);
             bool busy = p < total;
             if (busy) start(p);
             while (__any_sync(0xFFFFFFFFu, busy)) {
@@ -291,7 +293,7 @@ __global__ void __launch_bounds__(MAXT, MAXT == 128 ? 4 : 1)
                         if (w < 4u) atomicAdd(&s_wins[4 * slot + (int)w], 1);
                         words += r.used();
                         nsteps += steps;
-                        p = atomicAdd(&cnt[1], 1);
+                        p = atomicAdd(&s_cnt[iter & 1], 1);
                         busy = p < total;
                         if (busy) start(p);
                     }
@@ -304,7 +306,7 @@ __global__ void __launch_bounds__(MAXT, MAXT == 128 ? 4 : 1)
             TreeMeta& tm = s_tm[s];
             if (tm.done >= s_misc[4 * s + 1]) continue;
             backprop(F.nodes + tm.node_off, F.ucb + tm.node_off, F.csl + tm.node_off, s_path + s * kPathMax,
-                     s_mover + s * kPathMax, s_misc[4 * s + 0], s_wins + 4 * s, sp.playouts, sp.c_uct);
+                     s_mover + s * kPathMax, s_misc[4 * s + 0], s_wins + 4 * s, sp);
             __syncwarp();
             if (lane == 0) tm.done += 1;
             __syncwarp();
