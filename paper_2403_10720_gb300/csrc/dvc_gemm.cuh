@@ -13,6 +13,7 @@
 // bounded: on time-out the kernel records an error, waits (bounded) for its
 // own copies and MMAs, frees its tensor memory and exits.
 #pragma once
+#include "dvc_chain.cuh"
 #include <cuda.h>  // CUtensorMap (the type only; maps are encoded through the runtime's driver entry point)
 #include <stdint.h>
 
@@ -305,7 +306,8 @@ constexpr int kGemmThreads = 32 * (4 + kGemmEpiWarps);  // warp 0 TMA, warp 1 MM
 // BMN: B is K x N row-major instead (a layer's own weights where the backward
 // pass needs their transpose), tB (N, K), box (64, 64), read MN-major.
 // BACK: the backward epilogue (M a multiple of 32, N of 16).
-template <int BN, bool BMN = false, bool BACK = false>
+// CHAIN: for launch_chained (dvc_chain.cuh).
+template <int BN, bool BMN = false, bool BACK = false, bool CHAIN = false>
 __global__ void __launch_bounds__(kGemmThreads, 1)
     gemm_bf16_tc_kernel(const __grid_constant__ CUtensorMap tA, const __grid_constant__ CUtensorMap tB, GemmArgs a) {
     using Cfg = GemmCfg<BN>;
@@ -345,6 +347,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = s_tmem;
+    if constexpr (CHAIN) {
+        chain_next();
+        chain_wait();  // the head's weights apart, everything read is the launch before's
+    }
     if (warp == 0) {
         // producer: K slices of every tile of this CTA, up to S in flight
         int it = 0;
@@ -605,6 +611,8 @@ __global__ void __launch_bounds__(kDwThreads, 1) gemm_dw_kernel(const __grid_con
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = s_tmem;
+    chain_next();
+    chain_wait();
     if (warp == 0) {
         int it = 0;
         for (; it < a.nk; ++it) {

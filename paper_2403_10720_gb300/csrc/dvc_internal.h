@@ -24,9 +24,10 @@ void dvc_value_rows_free(dvc_value_rows* r);
 int dvc_value_prepare(dvc_ctx* c);
 // Win probabilities of n leaves into d_probs, with the activations in rows
 // [row0, row0 + n rounded up to 128) of r.  Enqueues kernels only: no
-// allocation, no synchronisation, so it may be captured into a graph.
+// allocation, no synchronisation, so it may be captured into a graph.  chained: the
+// launch before it in the stream is a kernel that calls chain_next (dvc_chain.cuh).
 int dvc_value_forward_rows(dvc_ctx* c, const dvc_state* d_leaves, int n, dvc_value_rows* r, int row0, float* d_probs,
-                           cudaStream_t st);
+                           cudaStream_t st, bool chained);
 
 struct dvc_ctx {
     dvc_config cfg;

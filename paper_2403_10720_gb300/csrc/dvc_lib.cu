@@ -40,10 +40,20 @@ void default_shape(int n, int sms, int engine, int P, int& T, int& W, int& chain
         // a warp per tree, and enough warps for one playout per thread (16 at most)
         T = std::max(1, std::min(32, (n + S - 1) / S));
         W = std::min(16, std::max(T, (T * std::max(P, 1) + 31) / 32));
-        // for value mode alone: one chain up to 16 trees per SM (2,432 trees 37.3 us
-        // per iteration against 38.5 with eight; 4,864 trees 48.6 against 44.8)
-        chains = n <= 16 * S ? 1 : std::max(1, std::min(24, (int)std::lround(n / (1.12 * S))));
+        chains = 1;
     }
+}
+
+// Chains of value mode.  One chain's launches overlap one another (dvc_chain.cuh), so
+// up to 16 trees per SM a second gains nothing (2,432 trees: 33.9 us per iteration
+// against 34.7 with two and 35.1 with eight).  Beyond, the walks of one chain fill
+// the SMs that the network of another leaves (a tile of 128 leaves takes four SMs):
+// 4,864 trees 54.1 against 42.2 with eight.  Past one wave of clusters the network
+// runs layer by layer on the whole chip, and fewer, larger batches are better: 8,192
+// trees 56.7 against 67.6.
+int default_value_chains(int n, int sms) {
+    const int S = std::max(sms, 1);
+    return n <= 16 * S || n > 32 * S ? 1 : 8;
 }
 }  // namespace
 
@@ -76,6 +86,7 @@ struct dvc_forest {
     int32_t* order;          // tree order: CTAs get equal total budget
     int trees_per_cta;       // trees per CTA (fused kernel and pipeline rollouts)
     int warps_per_cta;       // 0: default
+    int value_chains;        // chains of value mode
     int engine;              // 1: fused lockstep kernel, 2: three-kernel pipeline
     float2* ucb;
     float* csl;
@@ -1004,6 +1015,7 @@ int dvc_forest_create(dvc_ctx* c, int n, const dvc_state* d_roots, const int32_t
     // (four players, one playout, 1,200 trees 134 / 134, 2,432 trees 174 / 146).
     f->engine = (long long)n * std::max(c->cfg.playouts, c->cfg.policy ? 128 : 16) > 512LL * std::max(sms, 1) ? 2 : 1;
     default_shape(n, sms, f->engine, c->cfg.playouts, f->trees_per_cta, f->warps_per_cta, f->chains);
+    f->value_chains = default_value_chains(n, sms);
     std::vector<int32_t> order(n);
     {
         const int T = f->trees_per_cta;
@@ -1403,26 +1415,32 @@ void value_chain(const dvc_forest* f, int k, int chains, int& t0, int& t1, int& 
     }
 }
 
-int value_chains(const dvc_forest* f) { return std::max(1, std::min({kValueChains, f->chains, f->n / 128})); }
+int value_chains(const dvc_forest* f) { return std::max(1, std::min({kValueChains, f->value_chains, f->n / 128})); }
 
-// One value-mode iteration of chain k: (pending backprop +) select, the
-// network over the chain's leaves, credit.
+// One value-mode iteration of chain k: the pending credit and backprop with the
+// select, then the network over the chain's leaves.  Two launches, each started while
+// the other runs when the chain is alone: 152 trees 34.6 -> 31.2 us per iteration (a
+// launch for the credits took 2.5 of them), 4,096 trees 41.7 -> 38.9.
 int enqueue_value_iteration(dvc_forest* f, int k, int chains, cudaStream_t st) {
     dvc_ctx* c = f->ctx;
     int t0, t1, row0;
     value_chain(f, k, chains, t0, t1, row0);
     if (t1 <= t0) return DVC_OK;
-    if (c->cfg.vanilla)
-        pipe_select_kernel<true><<<((t1 - t0) * 32 + 127) / 128, 128, 0, st>>>(dev_of(f), params_of(f), t0, t1,
-                                                                                nullptr, f->pipe);
-    else
-        pipe_select_kernel<false><<<((t1 - t0) * 32 + 127) / 128, 128, 0, st>>>(dev_of(f), params_of(f), t0, t1,
-                                                                                 nullptr, f->pipe);
-    if (int rc = check_launch(c, "pipe_select_kernel")) return rc;
-    if (int rc = dvc_value_forward_rows(c, f->pipe.leaf + t0, t1 - t0, &f->vrows, row0, f->probs + 4 * (size_t)t0, st))
-        return rc;
-    pipe_value_wins_kernel<<<(t1 - t0 + 127) / 128, 128, 0, st>>>(t0, t1, f->pipe, f->probs, f->ctx->cfg.playouts);
-    return check_launch(c, "pipe_value_wins_kernel");
+    PipeBufs pb = f->pipe;
+    pb.probs = f->probs;
+    // With several chains, blocks that wait early only hold room the other chains need.
+    const bool alone = chains == 1;
+    const auto select = c->cfg.vanilla ? pipe_select_kernel<true> : pipe_select_kernel<false>;
+    const unsigned grid = (unsigned)((t1 - t0) * 32 + 127) / 128;
+    cudaError_t e = cudaSuccess;
+    if (alone) {
+        e = launch_chained(select, grid, 128, 0, st, dev_of(f), params_of(f), t0, t1, nullptr, pb);
+    } else {
+        select<<<grid, 128, 0, st>>>(dev_of(f), params_of(f), t0, t1, nullptr, pb);
+        e = cudaGetLastError();
+    }
+    if (e != cudaSuccess) return cuda_fail(c, e, "pipe_select_kernel");
+    return dvc_value_forward_rows(c, f->pipe.leaf + t0, t1 - t0, &f->vrows, row0, f->probs + 4 * (size_t)t0, st, alone);
 }
 
 int enqueue_value_det(dvc_forest* f, int k, int chains, int count, cudaStream_t st) {
@@ -1479,7 +1497,9 @@ int launch_value_pipeline(dvc_forest* f, int n_iterations, cudaStream_t st) {
     for (; left > 0; --left)
         for (int k = 0; k < chains; ++k)
             if (int rc = enqueue_value_iteration(f, k, chains, st)) return rc;
-    pipe_backprop_kernel<<<(f->n * 32 + 127) / 128, 128, 0, st>>>(dev_of(f), params_of(f), f->n, f->pipe);
+    PipeBufs pb = f->pipe;
+    pb.probs = f->probs;
+    pipe_backprop_kernel<<<(f->n * 32 + 127) / 128, 128, 0, st>>>(dev_of(f), params_of(f), f->n, pb);
     return check_launch(c, "pipe_backprop_kernel");
 }
 
@@ -1521,8 +1541,8 @@ int dvc_forest_tune(dvc_forest* f, int engine, int trees_per_cta, int warps_per_
         f->trees_per_cta = T;
     }
     f->engine = eng;
-    const int ch = chains ? chains : dC;
-    if (W != oldW || T != oldT || ch != oldC) {
+    const int ch = chains ? chains : dC, vch = chains ? chains : default_value_chains(f->n, sms);
+    if (W != oldW || T != oldT || ch != oldC || vch != f->value_chains) {
         // the captured pipeline graphs hold the old launch shape
         if (f->chunk_exec) cudaGraphExecDestroy(f->chunk_exec);
         if (f->value_exec) cudaGraphExecDestroy(f->value_exec);
@@ -1530,6 +1550,7 @@ int dvc_forest_tune(dvc_forest* f, int engine, int trees_per_cta, int warps_per_
     }
     f->warps_per_cta = W;
     f->chains = ch;
+    f->value_chains = vch;
     return DVC_OK;
 }
 

@@ -17,7 +17,7 @@
 // 7,400, the three layers' MMAs 14,000 (about 540 a slice of 64 columns, with the
 // weights' copies ahead of them), their epilogues 6,800 and the exchanges of
 // activations (96 KB out of every SM, fences, waits for the slowest neighbour)
-// 14,000.  333 rows: 30 us a call against 50 by layers.
+// 14,000.  333 rows: 29 us a call against 50 by layers.
 //
 // Roles: warps 0-15 features and epilogue, warp 16 copies, warp 17 MMA.  Shared
 // memory: H (128 x 512 BF16 in the K-blocked layout: 128 KB) and five 16 KB ring
@@ -175,14 +175,21 @@ __global__ void __cluster_dims__(kMlpCluster, 1, 1) __launch_bounds__(kMlpThread
     cluster_sync();  // barriers stand before a neighbour arrives on them
     tc_fence_after();
     const uint32_t tmem = s_tmem;
+    chain_next();
+    if (warp != 16) chain_wait();  // the first weights are copied while the leaves are made
     if (warp == 16) {
         int it = 0;
+        bool waited = false;
         bool stop = false;
         for (int L = 0; L < 3 && !stop; ++L) {
             const CUtensorMap* w = L == 0 ? &w1 : L == 1 ? &w2 : &w3;
             for (int kc = 0; kc < (L == 0 ? 10 : 8); ++kc, ++it) {
                 const int s = mlp_slot(it);
                 const int use = mlp_use(it);  // earlier contents of the slot, features included
+                if (use > 0 && !waited) {
+                    chain_wait();
+                    waited = true;
+                }
                 if (__any_sync(0xFFFFFFFFu, (use > 0 && !mbar_wait(&s_empty[s], (uint32_t)(use - 1) & 1u, a.wait_ns)) ||
                                                 *fail)) {
                     *fail = 1;

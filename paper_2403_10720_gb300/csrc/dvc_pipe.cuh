@@ -10,6 +10,7 @@
 // runs its iterations strictly in order, so results equal the fused kernel's
 // and the oracle's bit for bit.
 #pragma once
+#include "dvc_chain.cuh"
 #include <type_traits>
 
 #include "dvc_pool.cuh"
@@ -27,6 +28,7 @@ struct PipeBufs {
     uint4* tree0;       // per tree, kDetAhead first blocks of the iterations' tree streams (tag 3)
     int32_t* det_base;  // per tree; far below zero (bytes 0xC0) when nothing is sampled ahead
     int32_t* flags;     // the context's latched error
+    const float* probs;   // value mode: 4 win probabilities per tree, else null
 };
 
 __global__ void pipe_begin_kernel(ForestDev F, int n, int n_iter, int32_t* step_end) {
@@ -38,10 +40,21 @@ __global__ void pipe_begin_kernel(ForestDev F, int n, int n_iter, int32_t* step_
     step_end[t] = usable ? min(tm.budget, tm.done + n_iter) : tm.done;
 }
 
+// Value mode: the network's win probabilities stand in for the playouts of a
+// fresh, unfinished leaf -- each seat is credited round(p * P) of the P visits (a
+// leaf that ended inside the tree keeps its exact credit).  A warp, before the
+// pending backprop.
+__device__ __forceinline__ void pipe_value_wins(const PipeBufs& P, int t, int32_t playouts) {
+    const uint32_t s = threadIdx.x & 31u;
+    if (s < 4u && P.leaf[t].winner == kNone) P.wins[4 * t + s] = (int32_t)(P.probs[4 * t + s] * (float)playouts + 0.5f);
+    __syncwarp();
+}
+
 // Backpropagate the path the previous iteration left (np >= 0), if any.
 __device__ __forceinline__ void pipe_apply_pending(ForestDev& F, const SearchParams& sp, int t, PipeBufs& P) {
     const int32_t np = P.np[t];
     if (np < 0) return;
+    if (P.probs) pipe_value_wins(P, t, sp.playouts);
     TreeMeta& tm = F.meta[t];
     const long long off = tm.node_off;
     backprop(F.nodes + off, F.ucb + off, F.csl + off, P.path + (size_t)t * kPathMax, P.mover + (size_t)t * kPathMax,
@@ -92,6 +105,10 @@ template <bool VANILLA>
 __global__ void __launch_bounds__(128)
     pipe_select_kernel(ForestDev F, SearchParams sp, int i0, int i1, const int32_t* order, PipeBufs P) {
     __shared__ uint32_t s_E[4][104];
+    if (P.probs) {  // value mode may launch it chained
+        chain_next();
+        chain_wait();
+    }
     const int i = i0 + (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     if (i >= i1) return;
     const int t = order ? order[i] : i;
@@ -118,6 +135,7 @@ __global__ void __launch_bounds__(128)
         tree0 = P.tree0[(size_t)t * kDetAhead + ahead];
     }
     if (pending >= 0) {
+        if (P.probs) pipe_value_wins(P, t, sp.playouts);
         backprop(nodes, ucb, csl, path, mover, pending, P.wins + 4 * t, sp);
         __syncwarp();
     }
@@ -640,18 +658,6 @@ __global__ void __launch_bounds__(128) pipe_backprop_kernel(ForestDev F, SearchP
     const int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (t >= n) return;
     pipe_apply_pending(F, sp, t, P);
-}
-
-// Value mode: the network's win probabilities stand in for the playouts of
-// every fresh, unfinished leaf of trees t0 .. t1-1 -- each seat is credited
-// round(p * P) of the P visits (a leaf that ended inside the tree keeps its
-// exact credit).
-__global__ void pipe_value_wins_kernel(int t0, int t1, PipeBufs P, const float* probs, int playouts) {
-    const int t = t0 + (int)(blockIdx.x * blockDim.x + threadIdx.x);
-    if (t >= t1) return;
-    if (P.np[t] < 0 || P.leaf[t].winner != kNone) return;
-    int32_t* w = P.wins + 4 * t;
-    for (int s = 0; s < 4; ++s) w[s] = (int32_t)(probs[4 * t + s] * (float)playouts + 0.5f);
 }
 
 }  // namespace dvc

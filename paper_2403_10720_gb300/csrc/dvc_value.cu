@@ -65,6 +65,7 @@ constexpr int kFeatThreads = 128, kFeatRows = 32;
 
 __global__ void __launch_bounds__(kFeatThreads)
     features_kernel(const dvc_state* states, int n, int npad, __nv_bfloat16* X, float* Xf, int blocked) {
+    chain_next();
     __shared__ uint32_t s_rows[kFeatRows * kFeatPitch];
     __shared__ uint4 s_lut[256];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -111,6 +112,7 @@ __global__ void __launch_bounds__(kFeatThreads)
 // given as 8 partial sums per row (the output layer folded into layer 3):
 // z[r] = b4[r] + parts[0][r] + ... + parts[7][r].
 __global__ void softmax_head_kernel(const float* parts, const float* b4, const dvc_state* states, int n, float* out) {
+    chain_wait();
     const int row = blockIdx.x * blockDim.x + threadIdx.x;
     if (row >= n) return;
     const float4* pp = reinterpret_cast<const float4*>(parts) + (size_t)row * kHeadParts;
@@ -133,6 +135,8 @@ constexpr int kLossThreads = 128;
 __global__ void __launch_bounds__(kLossThreads)
     loss_grad_kernel(const float* L, const dvc_state* states, const float* labels, int n, int npad,
                      __nv_bfloat16* dZ4, float* rowpart) {
+    chain_next();
+    chain_wait();
     __shared__ float s_sum[kLossThreads / 32][5];
     const int row = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float d[4] = {0.0f, 0.0f, 0.0f, 0.0f};
@@ -221,6 +225,7 @@ constexpr int kAdamMain = (int)((NPARAM / 4 + kAdamThreads - 1) / kAdamThreads);
 constexpr int kAdamGrid = kAdamMain + 3 * (VH / 32) + 1;
 __global__ void __launch_bounds__(kAdamThreads)
     adamw_kernel(dvc_value_net v, int row_blocks, int loss_ctas, int n, AdamCoef a, float* loss_out) {
+    chain_wait();
     const int tid = threadIdx.x;
     if ((int)blockIdx.x < kAdamMain) {
         const size_t i = ((size_t)blockIdx.x * kAdamThreads + tid) * 4;
@@ -308,10 +313,19 @@ __global__ void init_params_kernel(float* w, uint64_t seed) {
 
 // ------------------------------------------------------------------ host helpers
 
+// The network's own tile widths have a chained build.
+template <int BN>
+constexpr bool kChainedGemm = BN == 256 || BN == 16;
+
 template <int BN, bool BMN = false, bool BACK = false>
 cudaError_t gemm_attributes() {
-    return cudaFuncSetAttribute(gemm_bf16_tc_kernel<BN, BMN, BACK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)GemmCfg<BN>::kSmem);
+    cudaError_t e = cudaFuncSetAttribute(gemm_bf16_tc_kernel<BN, BMN, BACK, false>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GemmCfg<BN>::kSmem);
+    if constexpr (kChainedGemm<BN>)
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(gemm_bf16_tc_kernel<BN, BMN, BACK, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)GemmCfg<BN>::kSmem);
+    return e;
 }
 
 // cuTensorMapEncodeTiled through the runtime's driver entry point, so the
@@ -347,7 +361,7 @@ bool encode_kmajor(CUtensorMap* m, const __nv_bfloat16* p, int rows, int K, int 
 }
 
 template <int BN, bool BMN = false, bool BACK = false>
-cudaError_t launch_gemm(const GemmArgs& a, cudaStream_t st) {
+cudaError_t launch_gemm(const GemmArgs& a, cudaStream_t st, bool chained) {
     // inside a stream capture the attributes were set beforehand (dvc_value_prepare)
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     cudaError_t e = cudaStreamIsCapturing(st, &cs);
@@ -362,7 +376,15 @@ cudaError_t launch_gemm(const GemmArgs& a, cudaStream_t st) {
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const unsigned grid = (unsigned)std::min<long long>(tiles, std::max(sms, 1));
-    gemm_bf16_tc_kernel<BN, BMN, BACK><<<grid, kGemmThreads, GemmCfg<BN>::kSmem, st>>>(tA, tB, a);
+    // chained while every tile has an SM of its own, where the launch and the prologue
+    // are a good part of the time (a training step of 8,192 rows 179 -> 158 us); a
+    // persistent grid gains nothing and its build without is faster (65,536 rows: the
+    // whole evaluation 148 us against 151 chained)
+    if constexpr (kChainedGemm<BN>)
+        if (chained && tiles <= sms)
+            return launch_chained(gemm_bf16_tc_kernel<BN, BMN, BACK, true>, grid, kGemmThreads, GemmCfg<BN>::kSmem, st,
+                                  tA, tB, a);
+    gemm_bf16_tc_kernel<BN, BMN, BACK, false><<<grid, kGemmThreads, GemmCfg<BN>::kSmem, st>>>(tA, tB, a);
     return cudaGetLastError();
 }
 
@@ -376,11 +398,11 @@ cudaError_t gemm(const __nv_bfloat16* A, const __nv_bfloat16* B, const float* bi
     const int wide = ((uintptr_t)C % 32 == 0 && (uintptr_t)Cf % 32 == 0) ? 1 : 0;  // null counts as aligned
     GemmArgs a{A, B, bias, C, Cf, M, N, K, act, flags, kGemmWaitNs, 0, nullptr, nullptr, wide,
                bias && (uintptr_t)bias % 16 == 0, a_blocked ? 1 : 0, c_blocked ? 1 : 0};
-    if (N % 256 == 0) return launch_gemm<256>(a, st);
-    if (N % 128 == 0) return launch_gemm<128>(a, st);
-    if (N % 64 == 0) return launch_gemm<64>(a, st);
-    if (N % 32 == 0) return launch_gemm<32>(a, st);
-    return launch_gemm<16>(a, st);
+    if (N % 256 == 0) return launch_gemm<256>(a, st, true);
+    if (N % 128 == 0) return launch_gemm<128>(a, st, true);
+    if (N % 64 == 0) return launch_gemm<64>(a, st, true);
+    if (N % 32 == 0) return launch_gemm<32>(a, st, true);
+    return launch_gemm<16>(a, st, true);
 }
 
 // Layer 3 with the 512 -> 4 output layer folded into its epilogue: no H3
@@ -389,7 +411,7 @@ cudaError_t gemm_head(const __nv_bfloat16* A, const __nv_bfloat16* B, const floa
                       const __nv_bfloat16* W4, float* parts, int32_t* flags, cudaStream_t st, bool a_blocked) {
     GemmArgs a{A,     B,  bias, nullptr, Cf, M, VH, VH, kActGelu, flags, kGemmWaitNs, 0, W4, parts,
                (uintptr_t)Cf % 32 == 0, bias && (uintptr_t)bias % 16 == 0, a_blocked ? 1 : 0, 0};
-    return launch_gemm<256>(a, st);  // N = 512: two 256-column tiles x four column groups = kHeadParts
+    return launch_gemm<256>(a, st, true);  // N = 512: two 256-column tiles x four column groups = kHeadParts
 }
 
 // dZ = (dZn Wn) * gelu'(Z): the gradient at the layer below, Wn (512 outputs of
@@ -408,7 +430,7 @@ cudaError_t gemm_back(const __nv_bfloat16* dZn, int K, const __nv_bfloat16* Wn, 
     a.wait_ns = kGemmWaitNs;
     a.Z = Z;
     a.colsum = colsum;
-    return launch_gemm<256, true, true>(a, st);
+    return launch_gemm<256, true, true>(a, st, true);
 }
 
 // Weight gradients of all four layers into v->grad.
@@ -429,8 +451,7 @@ cudaError_t gemm_dw(dvc_value_net* v, int npad, int32_t* flags, cudaStream_t st)
     a.grad = v->grad;
     a.flags = flags;
     a.wait_ns = kGemmWaitNs;
-    gemm_dw_kernel<<<first, kDwThreads, kDwSmem, st>>>(a);
-    return cudaGetLastError();
+    return launch_chained(gemm_dw_kernel, (unsigned)first, kDwThreads, kDwSmem, st, a);
 }
 
 cudaError_t mlp_attributes() {
@@ -559,7 +580,7 @@ int forward_into(dvc_ctx* c, const dvc_state* states, int n, int npad, __nv_bflo
 // a second wave would take 57 us (4,864 rows), and the layers use a full chip
 // better (65,536 rows: 148 us against 418).
 int infer(dvc_ctx* c, const dvc_state* states, int n, int npad, __nv_bfloat16* X, __nv_bfloat16* H1, __nv_bfloat16* H2,
-          float* L, float* probs, cudaStream_t st) {
+          float* L, float* probs, cudaStream_t st, bool chained) {
     dvc_value_net* v = c->vnet;
     if (npad / 128 <= v->clusters) {
         cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -572,12 +593,16 @@ int infer(dvc_ctx* c, const dvc_state* states, int n, int npad, __nv_bfloat16* X
         if (e != cudaSuccess) return cuda_fail(c, e, "value network");
         const MlpArgs a{{v->master + OFF_B1, v->master + OFF_B2, v->master + OFF_B3}, v->W4, v->b4p, states, n,
                         probs, c->d_flags, kGemmWaitNs};
-        mlp_kernel<<<npad / 128 * kMlpCluster, kMlpThreads, kMlpSmem, st>>>(w1, w2, w3, a);
-        return check_launch(c, "mlp_kernel");
+        if (chained) e = launch_chained(mlp_kernel, (unsigned)(npad / 128 * kMlpCluster), kMlpThreads, kMlpSmem, st, w1, w2, w3, a);
+        else {
+            mlp_kernel<<<npad / 128 * kMlpCluster, kMlpThreads, kMlpSmem, st>>>(w1, w2, w3, a);
+            e = cudaGetLastError();
+        }
+        return e == cudaSuccess ? DVC_OK : cuda_fail(c, e, "mlp_kernel");
     }
     if (int rc = forward_into(c, states, n, npad, X, H1, H2, nullptr, L, nullptr, nullptr, nullptr, true, st)) return rc;
-    softmax_head_kernel<<<(n + 127) / 128, 128, 0, st>>>(L, v->b4p, states, n, probs);
-    return check_launch(c, "softmax_head_kernel");
+    const cudaError_t e = launch_chained(softmax_head_kernel, (unsigned)(n + 127) / 128, 128, 0, st, L, v->b4p, states, n, probs);
+    return e == cudaSuccess ? DVC_OK : cuda_fail(c, e, "softmax_head_kernel");
 }
 
 int check_states_args(dvc_ctx* c, const void* d_states, int n) {
@@ -644,7 +669,7 @@ int dvc_value_eval(dvc_ctx* c, const dvc_state* d_leaves, int n, float* d_winpro
     if (int rc = ensure_work(c, npad)) return rc;
     cudaStream_t st = (cudaStream_t)stream;
     dvc_value_net* v = c->vnet;
-    return infer(c, d_leaves, n, npad, v->X, v->H1, v->H2, v->L, d_winprob, st);
+    return infer(c, d_leaves, n, npad, v->X, v->H1, v->H2, v->L, d_winprob, st, false);
 }
 
 int dvc_value_train_step(dvc_ctx* c, const dvc_state* d_states, const float* d_labels, int n, float lr, float* d_loss,
@@ -663,12 +688,11 @@ int dvc_value_train_step(dvc_ctx* c, const dvc_state* d_states, const float* d_l
     int32_t* fl = c->d_flags;
     if (int rc = forward_into(c, d_states, n, npad, v->X, v->H1, v->H2, v->H3, v->L, v->Z1, v->Z2, v->Z3, false, st))
         return rc;
-    loss_grad_kernel<<<npad / kLossThreads, kLossThreads, 0, st>>>(v->L, d_states, d_labels, n, npad, v->dZ4,
-                                                                  v->rowpart);
-    if (int rc = check_launch(c, "loss_grad_kernel")) return rc;
+    cudaError_t e = launch_chained(loss_grad_kernel, (unsigned)(npad / kLossThreads), kLossThreads, 0, st, v->L, d_states,
+                                   d_labels, n, npad, v->dZ4, v->rowpart);
     // the gradient at each hidden layer, from the top
     const size_t blocks = (size_t)npad / 32 * VH;
-    cudaError_t e = gemm_back(v->dZ4, 64, v->W4, v->Z3, v->dZ[2], v->colsum + 2 * blocks, npad, fl, st);
+    if (e == cudaSuccess) e = gemm_back(v->dZ4, 64, v->W4, v->Z3, v->dZ[2], v->colsum + 2 * blocks, npad, fl, st);
     if (e == cudaSuccess)
         e = gemm_back(v->dZ[2], VH, v->W3, v->Z2, v->dZ[1], v->colsum + blocks, npad, fl, st);
     if (e == cudaSuccess) e = gemm_back(v->dZ[1], VH, v->W2, v->Z1, v->dZ[0], v->colsum, npad, fl, st);
@@ -678,8 +702,8 @@ int dvc_value_train_step(dvc_ctx* c, const dvc_state* d_states, const float* d_l
     AdamCoef a{lr, 0.9f, 0.999f, 1e-8f, 1e-4f, 0.0f, 0.0f};
     a.c1 = 1.0f - powf(a.b1, (float)v->step);
     a.c2 = 1.0f - powf(a.b2, (float)v->step);
-    adamw_kernel<<<kAdamGrid, kAdamThreads, 0, st>>>(*v, npad / 32, npad / kLossThreads, n, a, d_loss);
-    return check_launch(c, "adamw_kernel");
+    e = launch_chained(adamw_kernel, kAdamGrid, kAdamThreads, 0, st, *v, npad / 32, npad / kLossThreads, n, a, d_loss);
+    return e == cudaSuccess ? DVC_OK : cuda_fail(c, e, "adamw_kernel");
 }
 
 int dvc_value_grads(dvc_ctx* c, float* d_out, void* stream) {
@@ -754,11 +778,11 @@ int dvc_gemm_timeout_probe(dvc_ctx* c, const void* d_A, const void* d_B, float* 
     GemmArgs a{(const __nv_bfloat16*)d_A, (const __nv_bfloat16*)d_B, nullptr, nullptr, d_Cf, M, N, K, kActNone,
                c->d_flags, (uint64_t)wait_ms * 1000000ull, 1, nullptr, nullptr, 0};
     cudaError_t e;
-    if (N % 256 == 0) e = launch_gemm<256>(a, (cudaStream_t)stream);
-    else if (N % 128 == 0) e = launch_gemm<128>(a, (cudaStream_t)stream);
-    else if (N % 64 == 0) e = launch_gemm<64>(a, (cudaStream_t)stream);
-    else if (N % 32 == 0) e = launch_gemm<32>(a, (cudaStream_t)stream);
-    else e = launch_gemm<16>(a, (cudaStream_t)stream);
+    if (N % 256 == 0) e = launch_gemm<256>(a, (cudaStream_t)stream, false);
+    else if (N % 128 == 0) e = launch_gemm<128>(a, (cudaStream_t)stream, false);
+    else if (N % 64 == 0) e = launch_gemm<64>(a, (cudaStream_t)stream, false);
+    else if (N % 32 == 0) e = launch_gemm<32>(a, (cudaStream_t)stream, false);
+    else e = launch_gemm<16>(a, (cudaStream_t)stream, false);
     return e == cudaSuccess ? DVC_OK : cuda_fail(c, e, "dvc_gemm_timeout_probe");
 }
 
@@ -814,13 +838,13 @@ int dvc_value_prepare(dvc_ctx* c) {
 }
 
 int dvc_value_forward_rows(dvc_ctx* c, const dvc_state* d_leaves, int n, dvc_value_rows* r, int row0, float* d_probs,
-                           cudaStream_t st) {
+                           cudaStream_t st, bool chained) {
     if (n <= 0) return DVC_OK;
     const int npad = (n + 127) / 128 * 128;
     if (row0 < 0 || row0 + npad > r->rows) return fail(c, DVC_E_INVALID, "value network: activation rows");
     const size_t o = (size_t)row0;
     return infer(c, d_leaves, n, npad, (__nv_bfloat16*)r->X + o * VF, (__nv_bfloat16*)r->H1 + o * VH,
-                 (__nv_bfloat16*)r->H2 + o * VH, r->L + o * kLogitFloats, d_probs, st);
+                 (__nv_bfloat16*)r->H2 + o * VH, r->L + o * kLogitFloats, d_probs, st, chained);
 }
 
 void dvc_value_free(dvc_ctx* c) {
