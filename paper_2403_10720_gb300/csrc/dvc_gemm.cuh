@@ -576,6 +576,10 @@ struct DwArgs {
     CUtensorMap a[4], b[4];
     DwProblem p[4];
     int nk;  // 64-row slices of the batch
+    int tiles;  // CTAs with a tile; one more adds the losses
+    int n;
+    const float* losses;  // n, 16-byte aligned
+    float* loss_sum;
     float* grad;
     int32_t* flags;
     uint64_t wait_ns;
@@ -585,6 +589,37 @@ constexpr uint32_t kDwStage = 24576u;
 constexpr uint32_t kDwSmem = kDwStages * kDwStage + 1024u;
 constexpr int kDwThreads = 256;
 
+// The sum of the rows' losses in row order, one FP32 addition after another as the
+// training step has always formed it: a serial chain (some 25 us for 8,192 rows), so
+// it runs on an SM that has no tile, beside the 45 us of the weight gradients.
+__device__ __forceinline__ void add_losses(const float* x, int n, float* out, float* buf) {
+    constexpr int kChunk = 16384;
+    float acc = 0.0f;
+    for (int at = 0; at < n; at += kChunk) {
+        const int m = min(kChunk, n - at);
+        for (int i = (int)threadIdx.x; i < m; i += kDwThreads) buf[i] = x[at + i];
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            int i = 0;
+            for (; i + 32 <= m; i += 32) {
+                float4 v[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) v[j] = reinterpret_cast<const float4*>(buf + i)[j];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    acc = __fadd_rn(acc, v[j].x);
+                    acc = __fadd_rn(acc, v[j].y);
+                    acc = __fadd_rn(acc, v[j].z);
+                    acc = __fadd_rn(acc, v[j].w);
+                }
+            }
+            for (; i < m; ++i) acc = __fadd_rn(acc, buf[i]);
+        }
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) *out = acc;
+}
+
 __global__ void __launch_bounds__(kDwThreads, 1) gemm_dw_kernel(const __grid_constant__ DwArgs a) {
     extern __shared__ __align__(1024) unsigned char gsm[];
     __shared__ uint64_t s_full[kDwStages], s_empty[kDwStages], s_acc;
@@ -592,6 +627,12 @@ __global__ void __launch_bounds__(kDwThreads, 1) gemm_dw_kernel(const __grid_con
     __shared__ int s_fail, s_issued, s_consumed;
     volatile int* fail = &s_fail;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if ((int)blockIdx.x >= a.tiles) {
+        chain_next();
+        chain_wait();
+        add_losses(a.losses, a.n, a.loss_sum, reinterpret_cast<float*>(gsm));
+        return;
+    }
     int q = 0;
     while (q < 3 && (int)blockIdx.x >= a.p[q + 1].first) ++q;
     const DwProblem pr = a.p[q];

@@ -47,7 +47,7 @@ struct dvc_value_net {
     __nv_bfloat16 *X, *H1, *H2, *H3, *dZ[3], *dZ4;  // dZ of layers 1..3; of the output layer, 64 columns
     float *Z1, *Z2, *Z3, *L;
     float* colsum;                     // bias gradients of layers 1..3 by 32 rows: 3 x (rows / 32) x 512
-    float* rowpart;                    // per CTA of the loss kernel: loss, four output-bias gradients, padding (8)
+    float* rowpart;                    // per CTA of the loss kernel: four output-bias gradients, padding (8); kLossSum
     long long step;
 };
 
@@ -129,15 +129,17 @@ __global__ void softmax_head_kernel(const float* parts, const float* b4, const d
 }
 
 // Cross-entropy against soft labels (absolute seats) and dL/dlogits / n.
-// Rows >= n get zero gradient.  dZ4 (npad x 64, BF16, K-padded); per CTA the
-// sums of the losses and of the FP32 logit gradients in rowpart[cta][0..4].
+// Rows >= n get zero gradient.  dZ4 (npad x 64, BF16, K-padded); the rows' losses
+// in rowloss, and per CTA the sums of the FP32 logit gradients in rowpart[cta][0..3].
 constexpr int kLossThreads = 128;
+constexpr int kLossSum = 7;  // in the first CTA's padding of rowpart: the sum of the losses
+static_assert(kLogitFloats > VO, "the rows' losses stand behind the logits");
 __global__ void __launch_bounds__(kLossThreads)
     loss_grad_kernel(const float* L, const dvc_state* states, const float* labels, int n, int npad,
-                     __nv_bfloat16* dZ4, float* rowpart) {
+                     __nv_bfloat16* dZ4, float* rowloss, float* rowpart) {
     chain_next();
     chain_wait();
-    __shared__ float s_sum[kLossThreads / 32][5];
+    __shared__ float s_sum[kLossThreads / 32][4];
     const int row = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float d[4] = {0.0f, 0.0f, 0.0f, 0.0f};
     float loss = 0.0f;
@@ -166,21 +168,22 @@ __global__ void __launch_bounds__(kLossThreads)
             }
     }
     if (row < npad) {
+        rowloss[row] = loss;
         uint4* out = reinterpret_cast<uint4*>(dZ4 + (size_t)row * 64);
         const __nv_bfloat162 lo = __floats2bfloat162_rn(d[0], d[1]), hi = __floats2bfloat162_rn(d[2], d[3]);
         out[0] = make_uint4(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi), 0u, 0u);
 #pragma unroll
         for (int j = 1; j < 8; ++j) out[j] = make_uint4(0u, 0u, 0u, 0u);
     }
-    float v[5] = {loss, d[0], d[1], d[2], d[3]};
+    float v[4] = {d[0], d[1], d[2], d[3]};
 #pragma unroll
-    for (int k = 0; k < 5; ++k) {
+    for (int k = 0; k < 4; ++k) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xFFFFFFFFu, v[k], o);
         if (lane == 0) s_sum[warp][k] = v[k];
     }
     __syncthreads();
-    if (threadIdx.x < 5) {
+    if (threadIdx.x < 4) {
         float acc = 0.0f;
         for (int w = 0; w < kLossThreads / 32; ++w) acc += s_sum[w][threadIdx.x];
         rowpart[(size_t)blockIdx.x * 8 + threadIdx.x] = acc;
@@ -215,8 +218,8 @@ __device__ __forceinline__ void store_bf16_weights(const dvc_value_net& v, size_
 }
 
 // End of a training step in one launch: sum the partial gradients (biases over the
-// 32-row column sums, output biases and loss over the loss kernel's CTAs, in a
-// fixed order), AdamW, BF16 copies.  CTAs 0 .. kAdamMain-1 take four weights per
+// 32-row column sums, output biases over the loss kernel's CTAs, in a fixed
+// order), AdamW, BF16 copies.  CTAs 0 .. kAdamMain-1 take four weights per
 // thread; then 16 CTAs per hidden layer take 32 biases each, and the last one the
 // output biases and the loss.  What bounds it is memory: gradients, master,
 // moments and their updates.
@@ -259,16 +262,16 @@ __global__ void __launch_bounds__(kAdamThreads)
         i = (layer == 0 ? OFF_B1 : layer == 1 ? OFF_B2 : OFF_B3) + (size_t)col;
         mine = tid < 32;
     } else {
-        const int k = tid & 7;  // 0: loss, 1..4: output biases
-        if (k < 5)
+        const int k = tid & 7;  // 0..3: output biases
+        if (k < 4)
             for (int r = tid >> 3; r < loss_ctas; r += kAdamThreads / 8) acc += v.rowpart[(size_t)r * 8 + k];
         s_part[tid] = acc;
         __syncthreads();
         acc = 0.0f;
         for (int w = 0; w < kAdamThreads / 8; ++w) acc += s_part[w * 8 + k];
-        if (tid == 0 && loss_out) *loss_out = acc / (float)n;
-        i = OFF_B4 + (size_t)(k - 1);
-        mine = tid >= 1 && tid < 5;
+        if (tid == 0 && loss_out) *loss_out = v.rowpart[kLossSum] / (float)n;
+        i = OFF_B4 + (size_t)k;
+        mine = tid < 4;
     }
     if (!mine) return;
     float m = v.m[i], u = v.v[i];
@@ -434,7 +437,7 @@ cudaError_t gemm_back(const __nv_bfloat16* dZn, int K, const __nv_bfloat16* Wn, 
 }
 
 // Weight gradients of all four layers into v->grad.
-cudaError_t gemm_dw(dvc_value_net* v, int npad, int32_t* flags, cudaStream_t st) {
+cudaError_t gemm_dw(dvc_value_net* v, int n, int npad, int32_t* flags, cudaStream_t st) {
     DwArgs a{};
     const __nv_bfloat16* A[4] = {v->dZ[0], v->dZ[1], v->dZ[2], v->H3};
     const __nv_bfloat16* B[4] = {v->X, v->H1, v->H2, v->dZ4};
@@ -447,11 +450,15 @@ cudaError_t gemm_dw(dvc_value_net* v, int npad, int32_t* flags, cudaStream_t st)
         a.p[q] = DwProblem{first, wb[q] / 64, wb[q], q == 3 ? 1 : 0, off[q]};
         first += VH / 128 * (wb[q] / 64);
     }
+    a.tiles = first;
+    a.losses = v->L + (size_t)npad * VO;
+    a.n = n;
+    a.loss_sum = v->rowpart + kLossSum;
     a.nk = npad / 64;
     a.grad = v->grad;
     a.flags = flags;
     a.wait_ns = kGemmWaitNs;
-    return launch_chained(gemm_dw_kernel, (unsigned)first, kDwThreads, kDwSmem, st, a);
+    return launch_chained(gemm_dw_kernel, (unsigned)first + 1u, kDwThreads, kDwSmem, st, a);
 }
 
 cudaError_t mlp_attributes() {
@@ -689,14 +696,14 @@ int dvc_value_train_step(dvc_ctx* c, const dvc_state* d_states, const float* d_l
     if (int rc = forward_into(c, d_states, n, npad, v->X, v->H1, v->H2, v->H3, v->L, v->Z1, v->Z2, v->Z3, false, st))
         return rc;
     cudaError_t e = launch_chained(loss_grad_kernel, (unsigned)(npad / kLossThreads), kLossThreads, 0, st, v->L, d_states,
-                                   d_labels, n, npad, v->dZ4, v->rowpart);
+                                   d_labels, n, npad, v->dZ4, v->L + (size_t)npad * VO, v->rowpart);
     // the gradient at each hidden layer, from the top
     const size_t blocks = (size_t)npad / 32 * VH;
     if (e == cudaSuccess) e = gemm_back(v->dZ4, 64, v->W4, v->Z3, v->dZ[2], v->colsum + 2 * blocks, npad, fl, st);
     if (e == cudaSuccess)
         e = gemm_back(v->dZ[2], VH, v->W3, v->Z2, v->dZ[1], v->colsum + blocks, npad, fl, st);
     if (e == cudaSuccess) e = gemm_back(v->dZ[1], VH, v->W2, v->Z1, v->dZ[0], v->colsum, npad, fl, st);
-    if (e == cudaSuccess) e = gemm_dw(v, npad, fl, st);
+    if (e == cudaSuccess) e = gemm_dw(v, n, npad, fl, st);
     if (e != cudaSuccess) return cuda_fail(c, e, "value backward");
     v->step += 1;
     AdamCoef a{lr, 0.9f, 0.999f, 1e-8f, 1e-4f, 0.0f, 0.0f};
