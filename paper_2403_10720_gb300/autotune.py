@@ -86,11 +86,11 @@ def tune(dvc, ctx, roots, budgets, seed, scale=0.05, candidates=None, use_cache=
 # The tail of an uneven forest, measured on four-player forests in chunks of
 # 2,000 iterations (budgets 1k-100k): with at most 16 running trees per SM the
 # fused engine with 4 trees x 4 warps per CTA, its CTAs filled with running
-# trees of similar remaining budgets, beats the pipeline (76 against 90 us per
-# iteration with 2,438 trees left, 64 against 85 with 1,785); with at most 5
-# per SM one tree per CTA is fastest (52 against 55 us with 770 left).  Without
-# the repacking, CTAs of several trees keep their finished trees' warps and
-# lose to one tree per CTA.
+# trees of similar remaining budgets, beats the pipeline (23.1 against 29.4 us
+# per iteration of 32 playouts with 2,400 trees left, 17.1 against 23.1 with
+# 1,200); with at most 5 per SM one tree per CTA is as fast (15.3 against 15.1
+# us with 600 left) and soon faster (14.6 against 15.1 with 152).  Without the
+# repacking, CTAs of several trees keep their finished trees' warps.
 PACK_TREES_PER_SM = 16
 PACK_SHAPE = (1, 4, 4, 0)
 TAIL_TREES_PER_SM = 5

@@ -26,9 +26,9 @@ constexpr int kValueChains = 16;  // at most, in value mode (each chain pads its
 
 // Default launch shape of an engine for n trees on `sms` SMs with P playouts
 // per leaf.  Pipeline: small rollout CTAs of at least two trees, warps enough
-// for one playout per thread (4 to 16), and as many chains (up to 16) as give
-// each chain about 0.85 CTAs per SM, so that the tree walks of some chains
-// run beside the playouts of the others.  Fused: every SM holds a CTA, one
+// for one playout per thread (4 to 16; the ordering-aware and compacting kernels
+// only), and as many chains (up to 24) as give each chain about 1.1 trees per SM,
+// so that the tree walks of some chains run beside the playouts of the others.  Fused: every SM holds a CTA, one
 // warp per tree up to 16.
 void default_shape(int n, int sms, int engine, int P, int& T, int& W, int& chains) {
     const int S = std::max(sms, 1);
