@@ -69,7 +69,7 @@ DRAM_PER_LAUNCH = {"select": 346_507, "rollout": 74_384, "det": 200_512}
 # x 4,096 iterations), summed over every kernel of the step by ncu
 # (graph-level capture, instruction counts only), and lanes active per warp
 # instruction; the capture is summarised under profiles/ with its command.
-ISSUE_PROFILE = {"warp_instructions_per_step": 5.2416e11, "lanes_active_per_instruction": 23.73,
+ISSUE_PROFILE = {"warp_instructions_per_step": 3.1076e11, "lanes_active_per_instruction": 31.40,
                  "source": "ncu smsp__inst_executed.sum / smsp__thread_inst_executed.sum over every kernel and "
                            "graph of one counting-free step at this shape (ncu summary under profiles/)"}
 
