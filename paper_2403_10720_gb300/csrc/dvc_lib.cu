@@ -67,7 +67,7 @@ struct dvc_forest {
     DetPlan* plans;
     unsigned long long* tables;
     Node* nodes;
-    float2* terms;  // UCB1 terms by visits (SearchParams::terms)
+    float2* terms;  // UCB1 terms by visits (SearchParams::terms); stands behind csl
     int n_terms;
     int32_t* link;
     int32_t* created;
@@ -957,8 +957,7 @@ void dvc_forest_destroy(dvc_forest* f) {
                     f->created,   f->work,      f->paths,     f->movers,         f->leaves,        f->leaf_tree,
                     f->leaf_iter, f->d_words,   f->export_scratch, f->order,     f->ucb,           f->csl,
                     f->pipe.leaf, f->pipe.path, f->pipe.mover, f->pipe.np,       f->pipe.wins,     f->pipe.step_end,
-                    f->pipe.det,  f->pipe.tree0, f->pipe.det_base, f->probs,
-                    f->terms};
+                    f->pipe.det,  f->pipe.tree0, f->pipe.det_base, f->probs};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     delete f;
@@ -1071,20 +1070,22 @@ int dvc_forest_create(dvc_ctx* c, int n, const dvc_state* d_roots, const int32_t
         alloc((void**)&f->tables, sizeof(unsigned long long) * (size_t)f->table_cap * n) &&
         alloc((void**)&f->nodes, sizeof(Node) * (size_t)slots) && alloc((void**)&f->link, sizeof(int32_t) * (size_t)slots) &&
         alloc((void**)&f->created, sizeof(int32_t) * (size_t)slots) && alloc((void**)&f->order, sizeof(int32_t) * n) &&
-        alloc((void**)&f->ucb, sizeof(float2) * (size_t)slots) && alloc((void**)&f->csl, sizeof(float) * (size_t)slots) &&
+        alloc((void**)&f->ucb, sizeof(float2) * (size_t)slots) &&
+        alloc((void**)&f->csl,
+              sizeof(float) * (size_t)(slots + (slots & 1)) + sizeof(float2) * (size_t)(f->n_terms + 1)) &&
         alloc((void**)&f->pipe.leaf, sizeof(dvc_state) * n) && alloc((void**)&f->pipe.path, sizeof(int32_t) * kPathMax * n) &&
         alloc((void**)&f->pipe.mover, (size_t)kPathMax * n) && alloc((void**)&f->pipe.np, sizeof(int32_t) * n) &&
         alloc((void**)&f->pipe.wins, sizeof(int32_t) * 4 * n) && alloc((void**)&f->pipe.step_end, sizeof(int32_t) * n) &&
         alloc((void**)&f->pipe.det, sizeof(dvc_state) * kDetAhead * (size_t)n) &&
         alloc((void**)&f->pipe.tree0, sizeof(uint4) * kDetAhead * (size_t)n) &&
         alloc((void**)&f->pipe.det_base, sizeof(int32_t) * n) &&
-        alloc((void**)&f->terms, sizeof(float2) * (size_t)(f->n_terms + 1)) &&
         (!vanilla || (alloc((void**)&f->set_key, sizeof(uint4) * (size_t)cells) &&
                       alloc((void**)&f->set_slot, sizeof(int32_t) * (size_t)cells)));
     if (!ok) {
         dvc_forest_destroy(f);
         return fail(c, DVC_E_OOM, "dvc_forest_create: device allocation of " + std::to_string(slots) + " node slots");
     }
+    f->terms = reinterpret_cast<float2*>(f->csl + (slots + (slots & 1)));
     // pageable source: the copy is staged before cudaMemcpyAsync returns
     cudaError_t e = cudaMemcpyAsync(f->meta, hm.data(), sizeof(TreeMeta) * n, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(f->roots, d_roots, sizeof(dvc_state) * n, cudaMemcpyDeviceToDevice, st);
