@@ -83,7 +83,9 @@ __device__ __forceinline__ uint32_t shared_addr(const void* p) { return (uint32_
 // some index); tab: shared address of the tables.  q carries the shift of the
 // chunk that holds the bit in its low five bits and, above them, minus the row
 // length times the ranks before that chunk plus the place of that chunk's table.
-template <uint32_t CH>
+// ORDERED: the read stays behind the barrier that follows the fill whatever m and n
+// come from, for callers that may have them from before it.
+template <uint32_t CH, bool ORDERED = false>
 __device__ __forceinline__ uint32_t select_bit(uint32_t tab, uint32_t m, uint32_t n) {
     using T = SelectTable<CH>;
     static_assert(T::kOff1 % 32u == CH && T::kOff2 % 32u == 2u * CH, "the low five bits are the chunk's shift");
@@ -95,9 +97,10 @@ __device__ __forceinline__ uint32_t select_bit(uint32_t tab, uint32_t m, uint32_
     const uint32_t chunk = __funnelshift_r(m, 0u, q) & (T::kRow - 1u);  // shifts by q mod 32
     const uint32_t a = tab + (n * T::kRow + q) + chunk;
     uint32_t v;
-    // not volatile: the tables do not change after they are filled, and m or n
-    // comes from a load behind the barrier that follows the fill
-    asm("ld.shared.u8 %0, [%1];" : "=r"(v) : "r"(a));
+    // otherwise not volatile: the tables do not change after they are filled, and a
+    // step's n comes from its random words, which lds32 reads behind the barrier
+    if constexpr (ORDERED) asm volatile("ld.shared.u8 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+    else asm("ld.shared.u8 %0, [%1];" : "=r"(v) : "r"(a));
     return v;
 }
 
@@ -271,7 +274,8 @@ struct PlayN {
         if (!(held & jb)) return;
         const uint32_t h = (a0 & jb) ? a0 : (a1 & jb) ? a1 : (a2 & jb) ? a2 : a3;
         const uint32_t hn = h & ~(j0 | j1), k = min(gap, (uint32_t)__popc(hn));
-        uint32_t p = k ? select_bit<9>(tab, hn, k - 1u) + 1u : 0u;
+        // ordered: the record may have been loaded before the tables were filled
+        uint32_t p = k ? select_bit<9, true>(tab, hn, k - 1u) + 1u : 0u;
         if (other == 1u << p) ++p;
         const uint32_t in0 = a0 & jb, in1 = a1 & jb, in2 = a2 & jb, up = rev & jb;
         a0 &= ~jb;
