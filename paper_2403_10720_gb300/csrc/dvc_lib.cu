@@ -1518,7 +1518,16 @@ int dvc_mcts_step(dvc_forest* f, int n_iterations, int mode, void* stream) {
     if (int rc = set_device(c)) return rc;
     cudaStream_t st = (cudaStream_t)stream;
     if (mode == DVC_MODE_VALUE) return launch_value_pipeline(f, n_iterations, st);
-    return f->engine == 2 ? launch_pipeline(f, n_iterations, st) : launch_fused(f, n_iterations, st);
+    // The pipeline launches its chunks as graphs, which a stream that is being captured
+    // refuses: there the fused engine, a plain launch with the same results, takes their
+    // place, so that a step may be captured whatever engine the forest's size takes.
+    bool fused = f->engine != 2;
+    if (!fused && n_iterations >= kChunkIters) {
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) cudaGetLastError();
+        fused = cs == cudaStreamCaptureStatusActive;
+    }
+    return fused ? launch_fused(f, n_iterations, st) : launch_pipeline(f, n_iterations, st);
 }
 
 int dvc_forest_tune(dvc_forest* f, int engine, int trees_per_cta, int warps_per_cta, int chains) {
