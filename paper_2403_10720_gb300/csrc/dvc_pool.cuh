@@ -46,17 +46,6 @@ __device__ __forceinline__ SetTable set_table(const ForestDev& F, const TreeMeta
 
 __device__ __forceinline__ void latch_error(int32_t* flags, int32_t code) { atomicCAS(&flags[0], 0, code); }
 
-// A lane's count of random words and game steps over a launch, in 64 bits: the warp of
-// a lone tree of 32 playouts counts about 400 steps per iteration, and a launch may run
-// 2^24 iterations.  `w` and `s` are those of one pass over the playouts.
-struct WorkSum {
-    unsigned long long words, steps;
-    __host__ __device__ void add(uint32_t w, uint32_t s) {
-        words += w;
-        steps += s;
-    }
-};
-
 // Shared-memory layout of one CTA with T slots and W warps.
 struct PoolLayout {
     uint32_t pl, meta, root, leaf, path, mover, wins, misc, base, E, cnt, ring, bytes;
@@ -135,8 +124,7 @@ __global__ void __launch_bounds__(MAXT, MAXT == 128 ? 4 : 1)
     else if constexpr (FAST2) fill_select12(s_lut12, tid, blockDim.x);
     __syncthreads();
 
-    // words per lane; steps per lane under the ordering-aware policy, else the warp's
-    WorkSum work{0ull, 0ull};
+    uint32_t words = 0u, nsteps = 0u;  // per lane; summed in 64 bits per warp at the end
     for (int iter = 0;; ++iter) {
         if (iter % kDetAhead == 0) {
             // ---- 0. the next kDetAhead determinizations of every running slot
@@ -245,10 +233,8 @@ __global__ void __launch_bounds__(MAXT, MAXT == 128 ? 4 : 1)
                     pend = st.mstop != 0u;
                     r.open(sp.seed, s_tm[slot].tree_id, p - k * P, (uint32_t)s_tm[slot].done);
                 }
-                uint32_t words = 0u, steps = 0u;
                 const uint32_t w =
-                    play_games<Game, true, true, FAST2>(g, r, busy, pend, sp.seed, sp.cont_thr, tab, words, steps);
-                work.add(words, steps);
+                    play_games<Game, true, true, FAST2>(g, r, busy, pend, sp.seed, sp.cont_thr, tab, words, nsteps);
                 credit_wins(s_wins, (uint32_t)slot, w);
                 // no winner after 128 steps is a broken invariant
                 if (busy && w >= 4u) latch_error(F.flags, DVC_E_INTERNAL);
@@ -305,7 +291,8 @@ __global__ void __launch_bounds__(MAXT, MAXT == 128 ? 4 : 1)
                         if (res != kGameOver) latch_error(F.flags, DVC_E_INTERNAL);
                         const uint32_t w = res == kGameOver ? winner : kNone;
                         if (w < 4u) atomicAdd(&s_wins[4 * slot + (int)w], 1);
-                        work.add(r.used(), (uint32_t)steps);
+                        words += r.used();
+                        nsteps += steps;
                         p = atomicAdd(&s_cnt[iter & 1], 1);
                         busy = p < total;
                         if (busy) start(p);
@@ -336,9 +323,9 @@ __global__ void __launch_bounds__(MAXT, MAXT == 128 ? 4 : 1)
         }
     }
     if (F.words) {  // F.words[0]: random words, F.words[1]: game steps (guesses)
-        const unsigned long long sum = warp_sum_u64(work.words);
+        const unsigned long long sum = warp_sum_u64((unsigned long long)words);
         // counted per lane, or (one game per lane) the same on every lane
-        const unsigned long long st = ORD ? warp_sum_u64(work.steps) : work.steps;
+        const unsigned long long st = ORD ? warp_sum_u64((unsigned long long)nsteps) : (unsigned long long)nsteps;
         if (lane == 0 && sum) atomicAdd(F.words, sum);
         if (lane == 0 && st) atomicAdd(F.words + 1, st);
     }
