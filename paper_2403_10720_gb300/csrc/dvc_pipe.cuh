@@ -238,9 +238,12 @@ __global__ void __launch_bounds__(32 * kPlayWarps, FAST2 ? 12 : 8)
     // no winner after 128 steps is a broken invariant
     if (mine && w >= 4u) latch_error(P.flags, DVC_E_INTERNAL);
     if (CNT && words_out) {  // words_out[0]: random words, words_out[1]: game steps (guesses)
-        const unsigned long long sum = warp_sum_u64((unsigned long long)words);
-        if (lane == 0 && sum) atomicAdd(words_out, sum);
-        if (lane == 0 && steps) atomicAdd(words_out + 1, (unsigned long long)steps);
+        // both sums of a warp's 32 games in one: each is far below 2^32
+        const unsigned long long sum = warp_sum_u64((unsigned long long)steps << 32 | words);
+        if (lane == 0 && sum) {
+            atomicAdd(words_out, sum & 0xFFFFFFFFull);
+            atomicAdd(words_out + 1, sum >> 32);
+        }
     }
 }
 

@@ -411,8 +411,7 @@ struct PlayN {
 // state and stream begun); pend: it starts with the continue coin.  Returns
 // the lane's winner, kNone if it has no game or, after 128 steps, no result (a
 // game has at most |T| guesses, each turning one tile face up).  CNT: adds the
-// words of this lane's game to `words` and the warp's steps to `steps` (the
-// same on every lane).
+// words and steps of this lane's game to `words` and `steps`.
 // ALONE: for a warp that has its scheduler to itself (two-player games in the
 // fused engine), where a step costs the length of its dependent chain and not
 // its operations: two steps and the next block of words, which neither needs,
@@ -435,7 +434,7 @@ __device__ __forceinline__ uint32_t play_games(Game& g, PlayWords& r, bool busy,
         if constexpr (ALONE) next = r.block(seed);
 #pragma unroll
         for (int k = 0; k < kSteps; ++k) {
-            if constexpr (CNT) steps += __popc(__ballot_sync(0xFFFFFFFFu, busy));
+            if constexpr (CNT) steps += busy ? 1u : 0u;
             uint32_t winner;
             const uint32_t before = r.used();
             const bool over =
