@@ -266,8 +266,9 @@ int dvc_mcts_step(dvc_forest* f, int n_iterations, int mode, void* stream);
  * lane compaction a group's playouts are pooled in one CTA of warps_per_cta
  * warps.  The determinizations of the graph's 64 iterations are sampled
  * up front, one thread per tree and iteration.  engine 0 keeps the current
- * engine (the default is 1 while trees x max(playouts, 16) is at most 512 per SM,
- * with the ordering-aware policy trees x max(playouts, 128); else 2).
+ * engine.  The default, with T = ceil(n_trees / SMs): 1 while T x max(playouts, 16) is
+ * at most 512, else 2; with the ordering-aware policy 1 while T is at most 2, or 3
+ * unless T x playouts is from 513 to 1,024, or T x max(playouts, 128) at most 512.
  * trees_per_cta, warps_per_cta, chains 0 = the engine's defaults (fused:
  * ceil(n_trees / SMs) trees, at most 32, and a warp per tree or one playout
  * per thread, whichever is more, up to 16 warps;

@@ -15,6 +15,7 @@
 
 #include "dvc_internal.h"
 #include "dvc_pipe.cuh"
+#include "dvc_shape.cuh"
 
 using namespace dvc;
 using namespace dvc_host;
@@ -23,38 +24,6 @@ namespace {
 constexpr int kMaxChains = 32;  // independent chains of the pipeline graph
 constexpr long long kMaxGrid = 1ll << 30;  // CTAs per playout launch
 constexpr int kValueChains = 16;  // at most, in value mode (each chain pads its leaves to 128 rows)
-
-// Default launch shape of an engine for n trees on `sms` SMs with P playouts
-// per leaf.  Pipeline: small rollout CTAs of at least two trees, warps enough
-// for one playout per thread (4 to 16; the ordering-aware and compacting kernels
-// only), and as many chains (up to 24) as give each chain about 1.1 trees per SM,
-// so that the tree walks of some chains run beside the playouts of the others.  Fused: every SM holds a CTA, one
-// warp per tree up to 16.
-void default_shape(int n, int sms, int engine, int P, int& T, int& W, int& chains) {
-    const int S = std::max(sms, 1);
-    if (engine == 2) {
-        chains = std::max(1, std::min(24, (int)std::lround(n / (1.12 * S))));
-        T = std::max(2, std::min(64, (int)std::ceil(n / (chains * 0.85 * S))));
-        W = std::max(4, std::min(16, (T * std::max(P, 1) + 31) / 32));
-    } else {
-        // a warp per tree, and enough warps for one playout per thread (16 at most)
-        T = std::max(1, std::min(32, (n + S - 1) / S));
-        W = std::min(16, std::max(T, (T * std::max(P, 1) + 31) / 32));
-        chains = 1;
-    }
-}
-
-// Chains of value mode.  One chain's launches overlap one another (dvc_chain.cuh), so
-// up to 16 trees per SM a second gains nothing (2,432 trees: 33.9 us per iteration
-// against 34.7 with two and 35.1 with eight).  Beyond, the walks of one chain fill
-// the SMs that the network of another leaves (a tile of 128 leaves takes four SMs):
-// 4,864 trees 54.1 against 42.2 with eight.  Past one wave of clusters the network
-// runs layer by layer on the whole chip, and fewer, larger batches are better: 8,192
-// trees 56.7 against 67.6.
-int default_value_chains(int n, int sms) {
-    const int S = std::max(sms, 1);
-    return n <= 16 * S || n > 32 * S ? 1 : 8;
-}
 }  // namespace
 
 struct dvc_forest {
@@ -1003,16 +972,7 @@ int dvc_forest_create(dvc_ctx* c, int n, const dvc_state* d_roots, const int32_t
     // slot (CTAs hold trees_per_cta trees): balances uneven forests.
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
-    // The fused lockstep kernel while an SM has at most one playout per thread (512)
-    // and two trees per warp (32), else the pipeline: past that its CTAs take a
-    // second pass over playouts, or run in a second wave.  Time per iteration (us,
-    // fused / pipeline, two players then four): 32 playouts, 2,432 trees 15.0 / 19.1
-    // and 22.7 / 29.1, 2,800 trees 22.4 / 20.1 and 35.0 / 30.9; 100 playouts, 760
-    // trees 12.8 / 17.8 and 20.3 / 25.0; one playout, 4,864 trees 15.6 / 21.1 and
-    // 23.3 / 28.1.  Ordering-aware games differ most in length, and the step waits
-    // for a CTA's longest one: from four trees per SM on they go to the pipeline
-    // (four players, one playout, 1,200 trees 134 / 134, 2,432 trees 174 / 146).
-    f->engine = (long long)n * std::max(c->cfg.playouts, c->cfg.policy ? 128 : 16) > 512LL * std::max(sms, 1) ? 2 : 1;
+    f->engine = default_engine(n, sms, c->cfg.playouts, c->cfg.policy != 0);
     default_shape(n, sms, f->engine, c->cfg.playouts, f->trees_per_cta, f->warps_per_cta, f->chains);
     f->value_chains = default_value_chains(n, sms);
     std::vector<int32_t> order(n);

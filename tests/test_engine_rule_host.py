@@ -1,0 +1,62 @@
+"""The default engine of a forest (host logic, no GPU): the library's own rule,
+compiled for the host, follows the fullest CTA of the fused engine, not the
+chip's average, and under the ordering-aware policy a forest of few trees never
+leaves the fused engine, whose CTAs of one and two trees its pipeline loses to."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+SRC = r'''
+#include <cstdio>
+#include "dvc_shape.cuh"
+int main() {
+    int n, sms, P, o;
+    while (std::scanf("%d %d %d %d", &n, &sms, &P, &o) == 4)
+        std::printf("%d\n", dvc::default_engine(n, sms, P, o != 0));
+    return 0;
+}
+'''
+
+
+@pytest.fixture(scope="module")
+def engine(tmp_path_factory):
+    if shutil.which("nvcc") is None:
+        pytest.skip("nvcc not found")
+    d = tmp_path_factory.mktemp("rule")
+    src, exe = d / "r.cu", d / "r"
+    src.write_text(SRC)
+    subprocess.run(["nvcc", "-std=c++17", "-I" + os.path.join(ROOT, "paper_2403_10720_gb300", "csrc"), str(src), "-o",
+                    str(exe)], check=True, capture_output=True)
+
+    def ask(rows):
+        text = "\n".join(" ".join(map(str, r)) for r in rows)
+        out = subprocess.run([str(exe)], input=text, check=True, capture_output=True, text=True).stdout
+        return [int(x) for x in out.split()]
+    return ask
+
+
+TREES = [1, 2, 3, 40, 75, 151, 152, 153, 304, 305, 457, 608, 609, 1217, 2281, 2432, 2433, 4864, 4865, 1 << 20]
+PLAYOUTS = [1, 15, 16, 17, 32, 33, 57, 128, 129, 170, 171, 256, 257, 512, 513, 1024, 65536, 1 << 20]
+
+
+@pytest.mark.parametrize("sms", [152, 76, 1])
+def test_uniform_playouts_follow_the_fullest_cta(engine, sms):
+    rows = [(n, sms, P, 0) for n in TREES for P in PLAYOUTS]
+    for (n, _, P, _), e in zip(rows, engine(rows)):
+        trees = -(-n // sms)
+        assert e == (1 if trees <= 32 and trees * P <= 512 else 2), (n, P)
+
+
+def test_ordering_aware(engine):
+    rows = [(n, 152, P, 1) for n in TREES for P in PLAYOUTS]
+    for (n, _, P, _), e in zip(rows, engine(rows)):
+        if n <= 304:
+            assert e == 1, (n, P)
+        elif n > 608:
+            assert e == 2, (n, P)
+        elif -(-n // 152) * P <= 512:
+            assert e == 1, (n, P)
+    assert engine([(400, 152, 200, 1), (400, 152, 256, 1), (400, 152, 400, 1), (608, 152, 129, 1)]) == [2, 2, 1, 2]
