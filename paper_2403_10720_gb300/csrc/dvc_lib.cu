@@ -1144,7 +1144,7 @@ int launch_fused(dvc_forest* f, int n_iterations, cudaStream_t st) {
     const int W = std::max(1, std::min(32, f->warps_per_cta ? f->warps_per_cta : std::min(T, 16)));
     const int n_run = f->active_prefix > 0 ? std::min(f->n, f->active_prefix) : f->n;
     const int grid = (n_run + T - 1) / T;
-    const PoolLayout L(T, W);
+    const PoolLayout L(T, W, c->cfg.policy != 0);
     const int threads = 32 * W;
     const bool fast2 = c->cfg.nplayers == 2 && c->cfg.ntiles == 24;
     cudaError_t e;
@@ -1504,7 +1504,7 @@ int dvc_forest_tune(dvc_forest* f, int engine, int trees_per_cta, int warps_per_
     const int T = trees_per_cta ? trees_per_cta : dT;
     const int W = warps_per_cta ? warps_per_cta : (trees_per_cta && eng == 1 ? std::min(T, 16) : dW);
     const int oldT = f->trees_per_cta, oldW = f->warps_per_cta, oldC = f->chains;
-    const PoolLayout L(T, W);
+    const PoolLayout L(T, W, f->ctx->cfg.policy != 0);
     if (L.bytes > 200 * 1024) return fail(f->ctx, DVC_E_UNSUPPORTED, "dvc_forest_tune: CTA state exceeds shared memory");
     if (T != f->trees_per_cta) {
         if (int rc = set_default_order(f, T)) return rc;

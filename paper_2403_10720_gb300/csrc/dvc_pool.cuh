@@ -46,10 +46,11 @@ __device__ __forceinline__ SetTable set_table(const ForestDev& F, const TreeMeta
 
 __device__ __forceinline__ void latch_error(int32_t* flags, int32_t code) { atomicCAS(&flags[0], 0, code); }
 
-// Shared-memory layout of one CTA with T slots and W warps.
+// Shared-memory layout of one CTA with T slots and W warps; the ordering-aware kernels
+// keep their words in registers and have no ring.
 struct PoolLayout {
     uint32_t pl, meta, root, leaf, path, mover, wins, misc, base, E, cnt, ring, bytes;
-    __host__ __device__ PoolLayout(int T, int W) {
+    __host__ __device__ PoolLayout(int T, int W, bool ordered) {
         uint32_t o = 0;
         auto take = [&](uint32_t n) {
             const uint32_t at = o;
@@ -67,7 +68,7 @@ struct PoolLayout {
         base = take(4u * T);   // per slot: first iteration sampled ahead
         E = take(4u * 104u * W);
         cnt = take(4u * 2u);   // by parity: next game to hand out (ordering-aware policy)
-        ring = take(kRingBytes * W);  // words of the playouts
+        ring = take(ordered ? 0u : kRingBytes * W);  // words of the playouts
         bytes = o;
     }
 };
@@ -87,7 +88,7 @@ __global__ void __launch_bounds__(MAXT, MAXT == 128 ? 4 : 1)
     using Game = typename std::conditional<FAST2, Play2, PlayN>::type;
     __shared__ __align__(16) unsigned char s_sel[ORD ? 16 : SelectTable<Game::kChunk>::kBytes];
     const int W = (int)(blockDim.x >> 5);
-    const PoolLayout L(T, W);
+    const PoolLayout L(T, W, ORD);
     DetPlan* s_pl = (DetPlan*)(smem + L.pl);
     TreeMeta* s_tm = (TreeMeta*)(smem + L.meta);
     dvc_state* s_root = (dvc_state*)(smem + L.root);
