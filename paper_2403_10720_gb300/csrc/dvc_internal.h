@@ -34,8 +34,8 @@ struct dvc_ctx {
     int device;
     std::string err;
     int32_t* d_flags;  // [0]: latched error code (0 = none)
-    unsigned long long* d_ws;  // determinization workspace
-    size_t ws_cells;
+    unsigned long long* d_ws[2];  // determinization workspace: the second half for calls of more roots
+    bool ws_joint;             // ... both in one allocation
     dvc_value_net* vnet;       // created on first use of a dvc_value_* call
 };
 

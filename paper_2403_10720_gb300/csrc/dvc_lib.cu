@@ -78,10 +78,11 @@ struct dvc_forest {
 
 namespace {
 
-// dvc_determinize: CTAs, and table slots in the workspace (128 MB); tables of
-// up to kDetSharedCells cells stand in shared memory instead (48 KB, four CTAs
-// per SM).
-constexpr int kDetSlots = 512;
+// dvc_determinize: table slots, one per CTA, in each half of the workspace (64 MB a
+// half, the second allocated by the first call of more roots; without it such a call
+// goes through its roots with half the CTAs); tables of up to kDetSharedCells cells
+// stand in shared memory instead (48 KB, four CTAs per SM).
+constexpr int kDetSlots = 256;
 constexpr uint32_t kDetSharedCells = 6144;
 constexpr int kDetThreads = 256;
 
@@ -166,9 +167,12 @@ __global__ void init_kernel(dvc_config cfg, uint64_t seed, int n, dvc_state* out
 // is how many roots are under way and how short a layer is.  1,000 four-player
 // joker roots: 59 us, against 31.1 ms with one thread per root (each filling
 // up to 32,768 cells by itself) in launches of 256 roots.
+// SPLIT: slots from kDetSlots on stand at ws1 (two allocations; to choose costs 3 %).
+template <bool SPLIT>
 __global__ void __launch_bounds__(kDetThreads, 4)
     determinize_kernel(const dvc_state* roots, int n, int observer, uint64_t seed, const uint32_t* tree_ids,
-                       const uint32_t* iter_ids, dvc_state* out, unsigned long long* ws, int32_t* flags) {
+                       const uint32_t* iter_ids, dvc_state* out, unsigned long long* ws, unsigned long long* ws1,
+                       int32_t* flags) {
     extern __shared__ __align__(16) unsigned long long s_table[];  // kDetSharedCells
     __shared__ DetPlan pl;
     for (int idx = blockIdx.x; idx < n; idx += gridDim.x) {
@@ -182,7 +186,9 @@ __global__ void __launch_bounds__(kDetThreads, 4)
                 out[idx] = roots[idx];
             }
         } else {
-            unsigned long long* F = pl.cells <= kDetSharedCells ? s_table : ws + (size_t)blockIdx.x * kDetMaxCells;
+            unsigned long long* F = s_table;
+            if (pl.cells > kDetSharedCells)
+                F = (SPLIT && blockIdx.x >= kDetSlots ? ws1 : ws) + (size_t)blockIdx.x * kDetMaxCells;
             det_fill(pl, F, threadIdx.x, kDetThreads, [] { __syncthreads(); });
             if (threadIdx.x == 0u) {
                 Rng r;
@@ -759,8 +765,8 @@ int dvc_create(dvc_ctx** out, const dvc_config* cfg, int device) {
     c->cfg = *cfg;
     c->device = device;
     c->d_flags = nullptr;
-    c->d_ws = nullptr;
-    c->ws_cells = 0;
+    c->d_ws[0] = c->d_ws[1] = nullptr;
+    c->ws_joint = false;
     if (cudaSetDevice(device) != cudaSuccess || cudaMalloc(&c->d_flags, 16) != cudaSuccess ||
         cudaMemset(c->d_flags, 0, 16) != cudaSuccess) {
         cudaGetLastError();
@@ -777,7 +783,8 @@ void dvc_destroy(dvc_ctx* c) {
     cudaSetDevice(c->device);
     dvc_value_free(c);
     if (c->d_flags) cudaFree(c->d_flags);
-    if (c->d_ws) cudaFree(c->d_ws);
+    if (c->d_ws[1] && !c->ws_joint) cudaFree(c->d_ws[1]);
+    if (c->d_ws[0]) cudaFree(c->d_ws[0]);
     delete c;
 }
 
@@ -831,28 +838,46 @@ int dvc_determinize(dvc_ctx* c, const dvc_state* d_roots, int n, int observer, u
     if (ranges_overlap(d_roots, d_out, sizeof(dvc_state) * (size_t)n))
         return fail(c, DVC_E_INVALID, "dvc_determinize: d_out may not overlap d_roots");
     if (int rc = set_device(c)) return rc;
-    if (!c->d_ws) {
-        const size_t cells = (size_t)kDetSlots * kDetMaxCells;
-        if (cudaMalloc(&c->d_ws, cells * sizeof(unsigned long long)) != cudaSuccess) {
-            cudaGetLastError();
-            c->d_ws = nullptr;
-            return fail(c, DVC_E_OOM, "dvc_determinize: workspace");
+    cudaStream_t st = (cudaStream_t)stream;
+    constexpr size_t half = (size_t)kDetSlots * kDetMaxCells;
+    auto take = [&](unsigned long long** p, size_t cells) {
+        if (cudaMalloc(p, cells * sizeof(unsigned long long)) == cudaSuccess) return true;
+        cudaGetLastError();
+        *p = nullptr;
+        return false;
+    };
+    if (!c->d_ws[0]) {
+        // both halves in one piece if the first call needs both
+        c->ws_joint = n > kDetSlots && take(&c->d_ws[0], 2 * half);
+        if (c->ws_joint) c->d_ws[1] = c->d_ws[0] + half;
+        else if (!take(&c->d_ws[0], half)) return fail(c, DVC_E_OOM, "dvc_determinize: workspace");
+        cudaError_t e = cudaSuccess;
+        for (auto k : {determinize_kernel<false>, determinize_kernel<true>}) {
+            if (e == cudaSuccess)
+                e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)(kDetSharedCells * sizeof(unsigned long long)));
+            if (e == cudaSuccess)
+                e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                         (int)cudaSharedmemCarveoutMaxShared);
         }
-        cudaError_t e = cudaFuncSetAttribute(determinize_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)(kDetSharedCells * sizeof(unsigned long long)));
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(determinize_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                     (int)cudaSharedmemCarveoutMaxShared);
         if (e != cudaSuccess) {
-            cudaFree(c->d_ws);
-            c->d_ws = nullptr;
+            cudaFree(c->d_ws[0]);
+            c->d_ws[0] = c->d_ws[1] = nullptr;
+            c->ws_joint = false;
             return cuda_fail(c, e, "dvc_determinize attributes");
         }
-        c->ws_cells = cells;
     }
-    determinize_kernel<<<std::min(n, kDetSlots), kDetThreads, kDetSharedCells * sizeof(unsigned long long),
-                         (cudaStream_t)stream>>>(d_roots, n, observer, seed, d_tree_ids, d_iter_ids, d_out, c->d_ws,
-                                                 c->d_flags);
+    if (n > kDetSlots && !c->d_ws[1]) {
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusActive;  // nothing is allocated during a capture
+        if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) cudaGetLastError();
+        else if (cs == cudaStreamCaptureStatusNone) take(&c->d_ws[1], half);
+    }
+    const int grid = std::min(n, c->d_ws[1] ? 2 * kDetSlots : kDetSlots);
+    const bool split = grid > kDetSlots && !c->ws_joint;
+    const auto kernel = split ? determinize_kernel<true> : determinize_kernel<false>;
+    kernel<<<grid, kDetThreads, kDetSharedCells * sizeof(unsigned long long), st>>>(
+        d_roots, n, observer, seed, d_tree_ids, d_iter_ids, d_out, c->d_ws[0], split ? c->d_ws[1] - half : nullptr,
+        c->d_flags);
     return check_launch(c, "determinize_kernel");
 }
 
