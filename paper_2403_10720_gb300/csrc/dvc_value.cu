@@ -532,8 +532,12 @@ int ensure_work(dvc_ctx* c, int npad) {
         free_work(v);
         return fail(c, DVC_E_OOM, "value network: workspace of " + std::to_string(npad) + " rows");
     }
-    // a training step's own kernels: their attributes are set here, so that a step may be captured after any call
-    cudaError_t e = gemm_attributes<256, true, true>();
+    // Attributes of a training step's kernels, set here so that a step of as many rows may
+    // be captured after any call: evaluations of up to a wave of clusters launch none of
+    // its forward GEMMs.
+    cudaError_t e = gemm_attributes<256>();
+    if (e == cudaSuccess) e = gemm_attributes<16>();
+    if (e == cudaSuccess) e = gemm_attributes<256, true, true>();
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(gemm_dw_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDwSmem);
     if (e != cudaSuccess) return cuda_fail(c, e, "value network attributes");
