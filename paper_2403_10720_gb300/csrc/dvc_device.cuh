@@ -76,15 +76,6 @@ struct Rng {
         left = 4;
         ++blk;
     }
-    // Take block 0 as computed elsewhere (e.g. ahead of time); right after open().
-    __device__ __forceinline__ void preload(uint4 b0) {
-        w0 = b0.x;
-        w1 = b0.y;
-        w2 = b0.z;
-        w3 = b0.w;
-        left = 4;
-        blk = 1;
-    }
     // Block 0 of a stream, as refill() computes it.
     __device__ __forceinline__ uint4 block0() const {
         uint32_t a = 0u, b = j, c = i, d = tw;
@@ -282,17 +273,6 @@ __device__ __forceinline__ uint32_t seq_tile(const G& g, uint32_t p, uint32_t s)
     return nth_set(hp & kNumMask, s - before);
 }
 
-// Sequence position of tile t held in hand p.
-__device__ __forceinline__ uint32_t seq_pos(const G& g, uint32_t p, uint32_t t) {
-    const uint32_t hp = g.hand(p);
-    if (t >= 24u) return joker_pos(g, hp, t - 24u);
-    const uint32_t k = __popc(hp & kNumMask & ((1u << t) - 1u));
-    uint32_t pos = k;
-    if ((hp >> 24) & 1u) pos += g.jg0 <= k;
-    if ((hp >> 25) & 1u) pos += g.jg1 <= k;
-    return pos;
-}
-
 // Tile in the h-th face-down slot (left to right) of the hand with tiles hp.
 template <class S>
 __device__ __forceinline__ uint32_t hidden_in(const S& g, uint32_t hp, uint32_t h) {
@@ -413,7 +393,6 @@ __device__ __forceinline__ void next_turn(G& g, R& r) {
 // floor(k / n) for k < 4096 and 1 <= n <= 31 from magic[n] = floor((2^32-1)/n) + 1:
 // k * magic / 2^32 exceeds k/n by less than 2^-20 < 1/n, so the floor is exact.
 __device__ __forceinline__ uint32_t div_small(uint32_t k, uint32_t n, const uint32_t* magic) {
-    if (magic == nullptr) return k / n;
     return n == 1u ? k : __umulhi(k, magic[n]);
 }
 
@@ -427,7 +406,7 @@ __device__ __forceinline__ void fill_magic(uint32_t* magic, uint32_t tid, uint32
 // The guess (slot s, identity index i) is correct iff i is the rank of the
 // slot's tile among the unknown identities, so only one select is needed.
 template <class R>
-__device__ __forceinline__ int random_guess(G& g, R& r, uint32_t cont_thr, const uint32_t* magic = nullptr) {
+__device__ __forceinline__ int random_guess(G& g, R& r, uint32_t cont_thr) {
     const uint32_t U = g.tmask & ~g.hand(g.cur) & ~g.rev;
     const uint32_t nid = __popc(U);
     uint32_t cnt[3], qs[3], nslots = 0;
@@ -441,7 +420,7 @@ __device__ __forceinline__ int random_guess(G& g, R& r, uint32_t cont_thr, const
         nslots += c;
     }
     const uint32_t k = pick(r.next(), nslots * nid);
-    uint32_t s = div_small(k, nid, magic);
+    uint32_t s = k / nid;
     const uint32_t i = k - s * nid;
     uint32_t q = qs[0];
     if (s >= cnt[0]) {

@@ -14,8 +14,8 @@ void dvc_value_free(dvc_ctx* c);
 // pipeline), so that a captured graph never points into the context's own
 // workspace, which other calls may reallocate.  rows: a multiple of 128.
 struct dvc_value_rows {
-    void *X, *H1, *H2, *H3;  // BF16: rows x 640, rows x 512 (three)
-    float* L;                // rows x 16 logits
+    void *X, *H1, *H2;  // BF16: rows x 640, rows x 512 (two)
+    float* L;           // rows x 8 partial logits of four seats
     int rows;
 };
 int dvc_value_rows_alloc(dvc_ctx* c, dvc_value_rows* r, int rows);

@@ -1759,7 +1759,9 @@ struct ServerLane {
 // Device bytes of one search slot of context c sized for max_budget
 // iterations: node arena (36 B per slot: node, UCB terms, link, creation
 // stamp), counting table, plan, meta and pipeline buffers (determinizations
-// sampled ahead included), plus the lane's staging per slot.
+// sampled ahead included), plus the lane's staging per slot.  What a lane holds besides
+// is not in it: the visit terms (at most 1 MB) and, in value mode, the network's
+// activations (3.4 KB per slot).
 size_t server_slot_bytes(const dvc_ctx* c, int max_budget) {
     const size_t arena = (size_t)(1 + kRootReserve + 4LL * max_budget) * 36;
     const size_t table = (size_t)(c->cfg.nplayers == 2 ? kDetMaxCells2p : kDetMaxCells) * 8;

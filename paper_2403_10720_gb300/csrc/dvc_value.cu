@@ -556,8 +556,6 @@ int need_net(dvc_ctx* c) {
     return DVC_OK;
 }
 
-// Forward pass for n rows (npad = n rounded up to 128).  With train = true,
-// keeps pre-activations and transposed activations for the backward pass.
 // Features and the four layers of npad rows (n live) into the given
 // activation buffers; Z1..Z3 (pre-activation FP32, training) may be null.
 // With head = true (inference) the output layer is folded into layer 3's
@@ -819,7 +817,7 @@ int dvc_value_rows_alloc(dvc_ctx* c, dvc_value_rows* r, int rows) {
     dvc_value_rows_free(r);
     const size_t n = (size_t)rows;
     const bool ok = cudaMalloc(&r->X, n * VF * 2) == cudaSuccess && cudaMalloc(&r->H1, n * VH * 2) == cudaSuccess &&
-                    cudaMalloc(&r->H2, n * VH * 2) == cudaSuccess && cudaMalloc(&r->H3, n * VH * 2) == cudaSuccess &&
+                    cudaMalloc(&r->H2, n * VH * 2) == cudaSuccess &&
                     cudaMalloc(&r->L, n * kLogitFloats * 4) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
@@ -831,7 +829,7 @@ int dvc_value_rows_alloc(dvc_ctx* c, dvc_value_rows* r, int rows) {
 }
 
 void dvc_value_rows_free(dvc_value_rows* r) {
-    void* ptrs[] = {r->X, r->H1, r->H2, r->H3, r->L};
+    void* ptrs[] = {r->X, r->H1, r->H2, r->L};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     *r = dvc_value_rows{};
