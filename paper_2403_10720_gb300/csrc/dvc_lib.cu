@@ -1172,19 +1172,24 @@ int launch_fused(dvc_forest* f, int n_iterations, cudaStream_t st) {
     const PoolLayout L(T, W, c->cfg.policy != 0);
     const int threads = 32 * W;
     const bool fast2 = c->cfg.nplayers == 2 && c->cfg.ntiles == 24;
+    int sms = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
+    const bool alone = play_alone(grid, sms, T, W, c->cfg.playouts);
     cudaError_t e;
-#define DVC_LAUNCH_POOL(MT, F2, ORD, VAN)                                                                         \
-    do {                                                                                                          \
-        e = cudaFuncSetAttribute(mcts_pool_kernel<MT, F2, ORD, VAN>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                                 (int)L.bytes);                                                                   \
-        if (e == cudaSuccess)                                                                                     \
-            mcts_pool_kernel<MT, F2, ORD, VAN><<<grid, threads, L.bytes, st>>>(                                   \
-                dev_of(f), params_of(f), n_iterations, f->order, f->n, T, f->pipe.det, f->pipe.tree0);            \
+#define DVC_LAUNCH_POOL(...)                                                                                        \
+    do {                                                                                                            \
+        e = cudaFuncSetAttribute(mcts_pool_kernel<__VA_ARGS__>, cudaFuncAttributeMaxDynamicSharedMemorySize,        \
+                                 (int)L.bytes);                                                                     \
+        if (e == cudaSuccess)                                                                                       \
+            mcts_pool_kernel<__VA_ARGS__><<<grid, threads, L.bytes, st>>>(dev_of(f), params_of(f), n_iterations,    \
+                                                                          f->order, f->n, T, f->pipe.det,           \
+                                                                          f->pipe.tree0);                           \
     } while (0)
-#define DVC_LAUNCH_POOL2(MT, ORD, VAN)                 \
-    do {                                               \
-        if (fast2) DVC_LAUNCH_POOL(MT, true, ORD, VAN); \
-        else DVC_LAUNCH_POOL(MT, false, ORD, VAN);     \
+#define DVC_LAUNCH_POOL2(MT, ORD, VAN)                                       \
+    do {                                                                     \
+        if (!fast2) DVC_LAUNCH_POOL(MT, false, ORD, VAN, false);             \
+        else if (alone) DVC_LAUNCH_POOL(MT, true, ORD, VAN, !ORD);           \
+        else DVC_LAUNCH_POOL(MT, true, ORD, VAN, false);                     \
     } while (0)
     if (c->cfg.policy) {  // ordering-aware playouts
         if (threads <= 512) DVC_LAUNCH_POOL2(512, true, true);

@@ -412,12 +412,12 @@ struct PlayN {
 // the lane's winner, kNone if it has no game or, after 128 steps, no result (a
 // game has at most |T| guesses, each turning one tile face up).  CNT: adds the
 // words and steps of this lane's game to `words` and `steps`.
-// ALONE: for a warp that has its scheduler to itself (two-player games in the
-// fused engine), where a step costs the length of its dependent chain and not
-// its operations: two steps and the next block of words, which neither needs,
-// form one stretch of code without a branch, and draws are selected early.  One
-// game alone 10,400 -> 9,450 cycles, 32 games 11,900 -> 10,700.  The other games'
-// step is twice as long and loses to instruction fetch that way (12 one-warp
+// ALONE: for a warp that has its scheduler nearly to itself (two-player games in
+// the fused engine, by the rule play_alone in dvc_shape.cuh), where a step costs the
+// length of its dependent chain and not its operations: two steps and the next
+// block of words, which neither needs, form one stretch of code without a branch,
+// and draws are selected early.  One game alone 10,400 -> 9,450 cycles, 32 games
+// 11,900 -> 10,700.  The other games' step is twice as long and loses to instruction fetch that way (12 one-warp
 // CTAs per SM: 40,400 -> 53,300 cycles).
 template <class Game, bool PEND, bool CNT, bool ALONE>
 __device__ __forceinline__ uint32_t play_games(Game& g, PlayWords& r, bool busy, bool pend, uint64_t seed,

@@ -79,7 +79,8 @@ struct PoolLayout {
 // stream blocks per tree (the forest's pipeline buffers; rewritten at the
 // start of every launch).
 // VANILLA: the trees have a plausible-set layer.
-template <int MAXT, bool FAST2, bool ORD, bool VANILLA>
+// ALONE: the form of the playouts for few warps per scheduler (play_alone, dvc_shape.cuh).
+template <int MAXT, bool FAST2, bool ORD, bool VANILLA, bool ALONE>
 __global__ void __launch_bounds__(MAXT, MAXT == 128 ? 4 : 1)
     mcts_pool_kernel(ForestDev F, SearchParams sp, int n_iter, const int32_t* order, int n_trees, int T,
                      dvc_state* det_ahead, uint4* tree0_ahead) {
@@ -252,7 +253,7 @@ __global__ void __launch_bounds__(MAXT, MAXT == 128 ? 4 : 1)
                     r.open(sp.seed, s_tm[slot].tree_id, p - k * P, (uint32_t)s_tm[slot].done);
                 }
                 const uint32_t w =
-                    play_games<Game, true, true, FAST2>(g, r, busy, pend, sp.seed, sp.cont_thr, tab, words, nsteps);
+                    play_games<Game, true, true, ALONE>(g, r, busy, pend, sp.seed, sp.cont_thr, tab, words, nsteps);
                 credit_wins(s_wins, (uint32_t)slot, w);
                 // no winner after 128 steps is a broken invariant
                 if (busy && w >= 4u) latch_error(F.flags, DVC_E_INTERNAL);

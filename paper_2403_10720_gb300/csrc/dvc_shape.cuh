@@ -62,6 +62,20 @@ inline void default_shape(int n, int sms, int engine, int P, int& T, int& W, int
     }
 }
 
+// Whether the fused engine's two-player playouts take the longer form that suits a warp
+// with its scheduler nearly to itself (play_games, ALONE): up to three warps that play
+// per scheduler, for `grid` CTAs of T trees and W warps (the builds of up to four warps
+// stand on an SM by four, the others alone; warps 0, 4, 8, .. of every CTA share a
+// scheduler).  Time per iteration (us, that form / the plain one): a lone tree, 32
+// playouts 6.4 / 7.2, 512 (four warps per scheduler) 10.4 / 9.9; 152 trees x 256 (two)
+// 8.9 / 9.4; 1,000 trees x 32 (two) 9.3 / 9.8, 2,000 x 32 (four) 13.2 / 12.8; CTAs of four trees and
+// four warps, two per SM 9.2 / 9.9, three 11.4 / 11.4, four 13.8 / 12.9.
+inline bool play_alone(int grid, int sms, int T, int W, int P) {
+    const int S = std::max(sms, 1), ctas = std::min((grid + S - 1) / S, W <= 4 ? 4 : 1);
+    const int warps = (int)std::min<long long>(W, ((long long)T * P + 31) / 32);
+    return ctas * ((warps + 3) / 4) <= 3;
+}
+
 // Chains of value mode.  One chain's launches overlap one another (dvc_chain.cuh), so
 // up to 16 trees per SM a second gains nothing (2,432 trees: 33.9 us per iteration
 // against 34.7 with two and 35.1 with eight).  Beyond, the walks of one chain fill

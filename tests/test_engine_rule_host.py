@@ -13,9 +13,10 @@ SRC = r'''
 #include <cstdio>
 #include "dvc_shape.cuh"
 int main() {
-    int n, sms, P, o;
-    while (std::scanf("%d %d %d %d", &n, &sms, &P, &o) == 4)
-        std::printf("%d\n", dvc::default_engine(n, sms, P, o != 0));
+    char what;
+    int a, b, c, d, e;
+    while (std::scanf(" %c %d %d %d %d %d", &what, &a, &b, &c, &d, &e) == 6)
+        std::printf("%d\n", what == 'e' ? dvc::default_engine(a, b, c, d != 0) : (int)dvc::play_alone(a, b, c, d, e));
     return 0;
 }
 '''
@@ -31,8 +32,8 @@ def engine(tmp_path_factory):
     subprocess.run(["nvcc", "-std=c++17", "-I" + os.path.join(ROOT, "paper_2403_10720_gb300", "csrc"), str(src), "-o",
                     str(exe)], check=True, capture_output=True)
 
-    def ask(rows):
-        text = "\n".join(" ".join(map(str, r)) for r in rows)
+    def ask(rows, what="e"):
+        text = "\n".join(" ".join(map(str, (what, *r, *[0] * (5 - len(r))))) for r in rows)
         out = subprocess.run([str(exe)], input=text, check=True, capture_output=True, text=True).stdout
         return [int(x) for x in out.split()]
     return ask
@@ -60,3 +61,11 @@ def test_ordering_aware(engine):
         elif -(-n // 152) * P <= 512:
             assert e == 1, (n, P)
     assert engine([(400, 152, 200, 1), (400, 152, 256, 1), (400, 152, 400, 1), (608, 152, 129, 1)]) == [2, 2, 1, 2]
+
+
+def test_form_of_two_player_playouts(engine):
+    # CTAs, SMs, trees and warps of a CTA, playouts
+    rows = {(1, 152, 1, 1, 1): 1, (1, 152, 1, 12, 384): 1, (1, 152, 1, 13, 385): 0, (1, 152, 1, 16, 1 << 20): 0,
+            (152, 152, 7, 7, 32): 1, (143, 152, 14, 14, 32): 0, (152, 152, 32, 16, 8): 1, (152, 152, 32, 16, 16): 0,
+            (456, 152, 4, 4, 32): 1, (457, 152, 4, 4, 32): 0, (457, 152, 4, 4, 1): 0, (1 << 18, 152, 4, 5, 1): 1}
+    assert engine(list(rows), "p") == list(rows.values())
