@@ -78,14 +78,17 @@ inline bool play_alone(int grid, int sms, int T, int W, int P) {
 
 // Chains of value mode.  One chain's launches overlap one another (dvc_chain.cuh), so
 // up to 16 trees per SM a second gains nothing (2,432 trees: 33.9 us per iteration
-// against 34.7 with two and 35.1 with eight).  Beyond, the walks of one chain fill
-// the SMs that the network of another leaves (a tile of 128 leaves takes four SMs):
-// 4,864 trees 54.1 against 42.2 with eight.  Past one wave of clusters the network
-// runs layer by layer on the whole chip, and fewer, larger batches are better: 8,192
-// trees 56.7 against 67.6.
+// against 34.7 with two and 35.1 with eight).  Beyond, the walks of one chain fill the
+// SMs that the network of another leaves, as long as the tiles of 128 leaves of all
+// eight, four SMs each, about fill the chip once (two players / four with jokers, one
+// chain against eight): 4,096 trees 38.9 / 40.5 against 37.4 / 39.1, 4,864 53.1 / 55.2
+// against 41.5 / 43.7, 5,000 46.9 / 49.1 against 41.7 / 44.1.  Past that (from 5,121
+// trees on, six tiles a chain) the network runs layer by layer on the whole chip, and
+// fewer, larger batches are better: 5,200 47.2 / 49.1 against 47.8 / 50.0, 6,000 48.4 /
+// 50.9 against 49.6 / 52.2, 8,192 54.3 / 57.2 against 65.9 / 69.6.
 inline int default_value_chains(int n, int sms) {
-    const int S = std::max(sms, 1);
-    return n <= 16 * S || n > 32 * S ? 1 : 8;
+    const int S = std::max(sms, 1), tiles = (S + 16) / 32;  // of each of eight chains, to the nearest
+    return n <= 16 * S || n > 8 * 128 * tiles ? 1 : 8;
 }
 
 }  // namespace dvc

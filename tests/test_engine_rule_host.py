@@ -16,7 +16,9 @@ int main() {
     char what;
     int a, b, c, d, e;
     while (std::scanf(" %c %d %d %d %d %d", &what, &a, &b, &c, &d, &e) == 6)
-        std::printf("%d\n", what == 'e' ? dvc::default_engine(a, b, c, d != 0) : (int)dvc::play_alone(a, b, c, d, e));
+        std::printf("%d\n", what == 'e'   ? dvc::default_engine(a, b, c, d != 0)
+                            : what == 'p' ? (int)dvc::play_alone(a, b, c, d, e)
+                                          : dvc::default_value_chains(a, b));
     return 0;
 }
 '''
@@ -69,3 +71,10 @@ def test_form_of_two_player_playouts(engine):
             (152, 152, 7, 7, 32): 1, (143, 152, 14, 14, 32): 0, (152, 152, 32, 16, 8): 1, (152, 152, 32, 16, 16): 0,
             (456, 152, 4, 4, 32): 1, (457, 152, 4, 4, 32): 0, (457, 152, 4, 4, 1): 0, (1 << 18, 152, 4, 5, 1): 1}
     assert engine(list(rows), "p") == list(rows.values())
+
+
+def test_value_chains(engine):
+    # 152 SMs: eight chains of up to five tiles of 128 leaves
+    rows = {(1, 152): 1, (2432, 152): 1, (2433, 152): 8, (5120, 152): 8, (5121, 152): 1, (1 << 20, 152): 1,
+            (1216, 76): 1, (1217, 76): 8, (2048, 76): 8, (2049, 76): 1, (100, 4): 1}
+    assert engine(list(rows), "v") == list(rows.values())
