@@ -60,11 +60,11 @@ ISSUE_LANES_PER_CLOCK = 128
 VALUE_MACS_PER_LEAF = 640 * 512 + 2 * 512 * 512 + 512 * 4  # dense layers of the value network
 L2_FLUSH_BYTES = 256 << 20  # > 129 MB L2
 # DRAM bytes per launch of the pipeline's kernels at the default shape of the
-# 4,096-tree workload (24 chains of 170 or 171 trees; 2 trees x 16 warps per
-# rollout CTA), from ncu captures (cold cache) of the counting-free kernels,
-# summarised under profiles/ with their commands.
+# 4,096-tree workload (24 chains of 170 or 171 trees), from ncu captures (cold
+# cache) of the counting-free kernels, summarised under profiles/ with their
+# commands.
 PROFILED_SHAPE = (24, 2, 16)
-DRAM_PER_LAUNCH = {"select": 346_507, "rollout": 74_384, "det": 200_512}
+DRAM_PER_LAUNCH = {"select": 247_280, "rollout": 38_885, "det": 257_792}
 # Warp instructions per step of the same workload at that shape (4,096 trees
 # x 4,096 iterations), summed over every kernel of the step by ncu
 # (graph-level capture, instruction counts only), and lanes active per warp

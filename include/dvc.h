@@ -248,7 +248,9 @@ int dvc_forest_reset(dvc_forest* f, const dvc_state* d_roots, void* stream);
  * round(p * cfg->playouts) of the cfg->playouts visits; a leaf that ended in
  * the tree credits its winner in both modes), and add cfg->playouts visits
  * and each node's mover's wins along the path.  Rollout results are
- * bit-exact with the split steps for every engine and launch shape.
+ * bit-exact with the split steps for every engine and launch shape.  A step in
+ * mode ROLLOUT may be captured into a CUDA graph by the caller; of 64
+ * iterations and more it then runs on engine 1 (dvc_forest_tune).
  */
 int dvc_mcts_step(dvc_forest* f, int n_iterations, int mode, void* stream);
 

@@ -548,9 +548,9 @@ __device__ __forceinline__ float2 visit_terms(float dv, float c_uct) {
 // `playouts`, so their terms come from the forest's table (sp.terms, entry k
 // for k * playouts visits).  One warp issues this step, an instruction every four
 // cycles, so what bounds it is their number: with the two square roots, the division
-// and the logarithm it took 1,600 cycles of a lone tree's iteration, now 980 (of
-// 18,000; the search of 10,000 iterations 94.1 -> 90.6 ms with the list of leaves by
-// ballots and the new child's block taken from the walk).
+// and the logarithm it took 1,600 cycles of a lone tree's iteration, now 980 (the
+// search of 10,000 iterations 94.1 -> 92.4 ms with the list of leaves by ballots and
+// the new child's block taken from the walk).
 __device__ __forceinline__ void backprop(Node* nodes, float2* ucb, float* csl, const int32_t* path,
                                          const uint8_t* mover, int32_t np, const int32_t* wins,
                                          const SearchParams& sp) {
