@@ -31,6 +31,7 @@ struct dvc_forest {
     int n;
     uint64_t seed;
     std::vector<int32_t> h_budgets;
+    int max_budget;  // the longest of them: no tree runs more iterations
     dvc_state* roots;
     TreeMeta* meta;
     DetPlan* plans;
@@ -1038,8 +1039,8 @@ int dvc_forest_create(dvc_ctx* c, int n, const dvc_state* d_roots, const int32_t
     }
     // no node is visited more often than the longest budget; the table stays below a
     // megabyte, and visits past it are computed
-    f->n_terms = std::min({n ? *std::max_element(f->h_budgets.begin(), f->h_budgets.end()) : 0, 1 << 17,
-                           INT32_MAX / c->cfg.playouts});
+    f->max_budget = n ? *std::max_element(f->h_budgets.begin(), f->h_budgets.end()) : 0;
+    f->n_terms = std::min({f->max_budget, 1 << 17, INT32_MAX / c->cfg.playouts});
     auto alloc = [&](void** p, size_t bytes) {
         if (cudaMalloc(p, bytes ? bytes : 16) != cudaSuccess) {
             cudaGetLastError();
@@ -1177,15 +1178,19 @@ int launch_fused(dvc_forest* f, int n_iterations, cudaStream_t st) {
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
     const bool alone = play_alone(grid, sms, T, W, c->cfg.playouts);
+    const int all = std::max(1, std::min(n_iterations, f->max_budget));
+    const int most = fused_launch_iterations(T, W, c->cfg.playouts);
     cudaError_t e;
 #define DVC_LAUNCH_POOL(...)                                                                                        \
     do {                                                                                                            \
         e = cudaFuncSetAttribute(mcts_pool_kernel<__VA_ARGS__>, cudaFuncAttributeMaxDynamicSharedMemorySize,        \
                                  (int)L.bytes);                                                                     \
-        if (e == cudaSuccess)                                                                                       \
-            mcts_pool_kernel<__VA_ARGS__><<<grid, threads, L.bytes, st>>>(dev_of(f), params_of(f), n_iterations,    \
-                                                                          f->order, f->n, T, f->pipe.det,           \
-                                                                          f->pipe.tree0);                           \
+        for (int left = all; e == cudaSuccess && left > 0; left -= most) {                                          \
+            mcts_pool_kernel<__VA_ARGS__><<<grid, threads, L.bytes, st>>>(dev_of(f), params_of(f),                  \
+                                                                          std::min(left, most), f->order, f->n, T, \
+                                                                          f->pipe.det, f->pipe.tree0);              \
+            e = cudaGetLastError();                                                                                 \
+        }                                                                                                           \
     } while (0)
 #define DVC_LAUNCH_POOL2(MT, ORD, VAN)                                       \
     do {                                                                     \
@@ -1210,8 +1215,7 @@ int launch_fused(dvc_forest* f, int n_iterations, cudaStream_t st) {
     }
 #undef DVC_LAUNCH_POOL2
 #undef DVC_LAUNCH_POOL
-    if (e != cudaSuccess) return cuda_fail(c, e, "mcts_pool_kernel attributes");
-    return check_launch(c, "mcts_pool_kernel");
+    return e == cudaSuccess ? DVC_OK : cuda_fail(c, e, "mcts_pool_kernel");
 }
 
 int pipe_rollout_threads(const dvc_forest* f) { return 32 * (f->warps_per_cta ? f->warps_per_cta : 32); }

@@ -126,26 +126,12 @@ __global__ void __launch_bounds__(MAXT, MAXT == 128 ? 4 : 1)
     else if constexpr (FAST2) fill_select12(s_lut12, tid, blockDim.x);
     __syncthreads();
 
-    // This lane's random words and game steps since they were last added to the forest's
-    // 64-bit counters, every kDetAhead iterations: a launch may run 2^24 iterations, so
-    // that 32 bits do not hold its counts, and 64-bit ones here cost the ordering-aware
-    // kernels, at 127 of 128 registers, up to 5 % (one four-player tree 69.4 -> 73.4 us
-    // per iteration).
-    static_assert((unsigned long long)kDetAhead * (32ull << 20) / 512u * 128u * 4u < 1ull << 32,
-                  "32 trees of 2^20 playouts on 16 warps, games of at most 128 steps of 4 words");
+    // This lane's random words and game steps; a launch has no more iterations than these
+    // hold (fused_launch_iterations, dvc_shape.cuh).  In 64 bits, or added to the forest's
+    // counters on the way, they cost four-player forests of a tree or a few per SM 1 to 5 %.
     uint32_t words = 0u, nsteps = 0u;
-    const auto flush = [&] {
-        if (F.words) {  // F.words[0]: random words, F.words[1]: game steps (guesses)
-            const unsigned long long w = warp_sum_u64((unsigned long long)words);
-            const unsigned long long st = warp_sum_u64((unsigned long long)nsteps);
-            if (lane == 0 && w) atomicAdd(F.words, w);
-            if (lane == 0 && st) atomicAdd(F.words + 1, st);
-        }
-        words = nsteps = 0u;
-    };
     for (int iter = 0;; ++iter) {
         if (iter % kDetAhead == 0) {
-            flush();
             // ---- 0. the next kDetAhead determinizations of every running slot
             __syncthreads();
             for (int idx = (int)tid; idx < nslot * kDetAhead; idx += (int)blockDim.x) {
@@ -344,7 +330,12 @@ __global__ void __launch_bounds__(MAXT, MAXT == 128 ? 4 : 1)
             dst.failed = s_tm[s].failed;
         }
     }
-    flush();
+    if (F.words) {  // F.words[0]: random words, F.words[1]: game steps (guesses)
+        const unsigned long long sum = warp_sum_u64((unsigned long long)words);
+        const unsigned long long st = warp_sum_u64((unsigned long long)nsteps);
+        if (lane == 0 && sum) atomicAdd(F.words, sum);
+        if (lane == 0 && st) atomicAdd(F.words + 1, st);
+    }
 }
 
 }  // namespace dvc

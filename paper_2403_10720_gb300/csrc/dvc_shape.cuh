@@ -62,6 +62,15 @@ inline void default_shape(int n, int sms, int engine, int P, int& T, int& W, int
     }
 }
 
+// Iterations of one launch of the fused engine: as many as its lanes' 32-bit counts of
+// random words hold, each lane playing T P games an iteration shared among 32 W lanes, of
+// at most 128 steps of four words.  8.4 million for up to one game a lane (a minute and
+// more); a longer step takes several launches.
+inline int fused_launch_iterations(int T, int W, int P) {
+    const long long lanes = 32LL * W, games = ((long long)T * P + lanes - 1) / lanes;
+    return (int)std::max<long long>(1, ((1LL << 32) - 1) / (games * 128 * 4));
+}
+
 // Whether the fused engine's two-player playouts take the longer form that suits a warp
 // with its scheduler nearly to itself (play_games, ALONE): up to three warps that play
 // per scheduler, for `grid` CTAs of T trees and W warps (the builds of up to four warps

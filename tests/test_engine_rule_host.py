@@ -18,6 +18,7 @@ int main() {
     while (std::scanf(" %c %d %d %d %d %d", &what, &a, &b, &c, &d, &e) == 6)
         std::printf("%d\n", what == 'e'   ? dvc::default_engine(a, b, c, d != 0)
                             : what == 'p' ? (int)dvc::play_alone(a, b, c, d, e)
+                            : what == 'l' ? dvc::fused_launch_iterations(a, b, c)
                                           : dvc::default_value_chains(a, b));
     return 0;
 }
@@ -78,3 +79,12 @@ def test_value_chains(engine):
     rows = {(1, 152): 1, (2432, 152): 1, (2433, 152): 8, (5120, 152): 8, (5121, 152): 1, (1 << 20, 152): 1,
             (1216, 76): 1, (1217, 76): 8, (2048, 76): 8, (2049, 76): 1, (100, 4): 1}
     assert engine(list(rows), "v") == list(rows.values())
+
+
+def test_launches_end_before_their_counts_wrap(engine):
+    # trees and warps of a CTA, playouts; a game has at most 128 steps of four words
+    rows = [(T, W, P) for T in (1, 2, 14, 32, 64) for W in (1, 3, 16, 32) for P in (1, 32, 256, 4096, 1 << 20)]
+    for (T, W, P), n in zip(rows, engine(rows, "l")):
+        games = -(-T * P // (32 * W))
+        assert n >= 1 and n * games * 512 < 1 << 32
+        assert (n + 1) * games * 512 > 0.99 * (1 << 32) or n > 1000

@@ -1,6 +1,6 @@
 """The fused engine's counts of random words and game steps over launches of
-several stretches of 64 iterations, with trees that end inside them: the
-oracle's."""
+several stretches of 64 iterations, with trees that end inside them, and over
+steps that take more than one launch: the oracle's."""
 import numpy as np
 import pytest
 
