@@ -168,14 +168,17 @@ __global__ void init_kernel(dvc_config cfg, uint64_t seed, int n, dvc_state* out
 // is how many roots are under way and how short a layer is.  1,000 four-player
 // joker roots: 59 us, against 31.1 ms with one thread per root (each filling
 // up to 32,768 cells by itself) in launches of 256 roots.
-// SPLIT: slots from kDetSlots on stand at ws1 (two allocations; to choose costs 3 %).
-template <bool SPLIT>
+// Slots from kDetSlots on stand at ws1.  A CTA's slot is kept in shared memory: worked out
+// where a table is chosen it costs registers (62 against 53) and 5,000 roots take 304 us
+// against 280.
 __global__ void __launch_bounds__(kDetThreads, 4)
     determinize_kernel(const dvc_state* roots, int n, int observer, uint64_t seed, const uint32_t* tree_ids,
                        const uint32_t* iter_ids, dvc_state* out, unsigned long long* ws, unsigned long long* ws1,
                        int32_t* flags) {
     extern __shared__ __align__(16) unsigned long long s_table[];  // kDetSharedCells
     __shared__ DetPlan pl;
+    __shared__ unsigned long long* s_slot;
+    if (threadIdx.x == 0u) s_slot = (blockIdx.x < kDetSlots ? ws : ws1) + (size_t)blockIdx.x * kDetMaxCells;
     for (int idx = blockIdx.x; idx < n; idx += gridDim.x) {
         const G g = load_state(roots[idx]);
         const uint32_t obs = observer < 0 ? g.cur : (uint32_t)observer;
@@ -187,9 +190,7 @@ __global__ void __launch_bounds__(kDetThreads, 4)
                 out[idx] = roots[idx];
             }
         } else {
-            unsigned long long* F = s_table;
-            if (pl.cells > kDetSharedCells)
-                F = (SPLIT && blockIdx.x >= kDetSlots ? ws1 : ws) + (size_t)blockIdx.x * kDetMaxCells;
+            unsigned long long* F = pl.cells <= kDetSharedCells ? s_table : s_slot;
             det_fill(pl, F, threadIdx.x, kDetThreads, [] { __syncthreads(); });
             if (threadIdx.x == 0u) {
                 Rng r;
@@ -854,15 +855,11 @@ int dvc_determinize(dvc_ctx* c, const dvc_state* d_roots, int n, int observer, u
         c->ws_joint = n > kDetSlots && take(&c->d_ws[0], 2 * half);
         if (c->ws_joint) c->d_ws[1] = c->d_ws[0] + half;
         else if (!take(&c->d_ws[0], half)) return fail(c, DVC_E_OOM, "dvc_determinize: workspace");
-        cudaError_t e = cudaSuccess;
-        for (auto k : {determinize_kernel<false>, determinize_kernel<true>}) {
-            if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)(kDetSharedCells * sizeof(unsigned long long)));
-            if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                         (int)cudaSharedmemCarveoutMaxShared);
-        }
+        cudaError_t e = cudaFuncSetAttribute(determinize_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)(kDetSharedCells * sizeof(unsigned long long)));
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(determinize_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                     (int)cudaSharedmemCarveoutMaxShared);
         if (e != cudaSuccess) {
             cudaFree(c->d_ws[0]);
             c->d_ws[0] = c->d_ws[1] = nullptr;
@@ -876,11 +873,9 @@ int dvc_determinize(dvc_ctx* c, const dvc_state* d_roots, int n, int observer, u
         else if (cs == cudaStreamCaptureStatusNone) take(&c->d_ws[1], half);
     }
     const int grid = std::min(n, c->d_ws[1] ? 2 * kDetSlots : kDetSlots);
-    const bool split = grid > kDetSlots && !c->ws_joint;
-    const auto kernel = split ? determinize_kernel<true> : determinize_kernel<false>;
-    kernel<<<grid, kDetThreads, kDetSharedCells * sizeof(unsigned long long), st>>>(
-        d_roots, n, observer, seed, d_tree_ids, d_iter_ids, d_out, c->d_ws[0], split ? c->d_ws[1] - half : nullptr,
-        c->d_flags);
+    determinize_kernel<<<grid, kDetThreads, kDetSharedCells * sizeof(unsigned long long), st>>>(
+        d_roots, n, observer, seed, d_tree_ids, d_iter_ids, d_out, c->d_ws[0],
+        c->d_ws[1] ? c->d_ws[1] - half : nullptr, c->d_flags);
     return check_launch(c, "determinize_kernel");
 }
 
